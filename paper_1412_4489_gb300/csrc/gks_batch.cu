@@ -177,10 +177,10 @@ __global__ void __launch_bounds__(kThreads, BatchBlocks<R>::value) k_batch(Args<
       const R dt = step_dt<R>(c);
       if (w.w == 0) {
         if (i <= g.nx && j < g.ny)
-          flux_face<0, R, TW, NSM>(g, a.fc[2 * w.x], a.rec + o.rec, a.Wx[par ^ 1] + o.wx, a.Fx + o.fx, i, j, dt);
+          flux_face<0, R, TW, NSM, sizeof(R) == 4>(g, a.fc[2 * w.x], a.rec + o.rec, a.Wx[par ^ 1] + o.wx, a.Fx + o.fx, i, j, dt);
       } else {
         if (i < g.nx && j <= g.ny)
-          flux_face<1, R, TW, NSM>(g, a.fc[2 * w.x + 1], a.rec + o.rec, a.Wy[par ^ 1] + o.wy, a.Fy + o.fy, i, j,
+          flux_face<1, R, TW, NSM, sizeof(R) == 4>(g, a.fc[2 * w.x + 1], a.rec + o.rec, a.Wy[par ^ 1] + o.wy, a.Fy + o.fy, i, j,
                                    dt);
       }
     }

@@ -23,6 +23,8 @@ template <class R> struct Prec;
 // series_terms: the sums stop before x^series_terms / series_terms!, at which the largest
 // relative truncation error over x < series_below is below the type's rounding (FP64: 17
 // terms reach it, FP32: 18);
+// exp_zero: exp(-x) is exactly 0 from here on, and not evaluated (FP32: always evaluated, a
+// branch costs more than its two instructions);
 // tie: relative width within which two cross-derivative candidates count as equal.
 // FP64: far above its rounding noise, far below any real difference.  FP32: ~16
 // ulps, just above the rounding noise of the candidates; a wider band makes FP32
@@ -31,18 +33,18 @@ template <class R> struct Prec;
 template <> struct Prec<double> {
   static constexpr double series_below = 0.5;
   static constexpr int series_terms = 18;
+  static constexpr double exp_zero = 746.0;
   static constexpr double tie = 1e-8;
 };
 template <> struct Prec<float> {
   static constexpr float series_below = 2.0f;
   static constexpr int series_terms = 18;
+  static constexpr float exp_zero = INFINITY;
   static constexpr float tie = 1e-6f;
 };
 
 __device__ __forceinline__ double d_exp(double x) { return exp(x); }
 __device__ __forceinline__ float d_exp(float x) { return __expf(x); }
-__device__ __forceinline__ double d_expm1(double x) { return expm1(x); }
-__device__ __forceinline__ float d_expm1(float x) { return expm1f(x); }
 __device__ __forceinline__ double d_erfc(double x) { return erfc(x); }
 __device__ __forceinline__ float d_erfc(float x) { return erfcf(x); }
 __device__ __forceinline__ double d_sqrt(double x) { return sqrt(x); }
@@ -64,26 +66,26 @@ template <class R, int NU, int NV>
 struct Moments {
   R u[NU];
   R v[NV];
-  R xi2, xi4;
-  R kap;  // <xi^4> - <xi^2>^2 = 2 K var^2
+  R xi2;
 };
 
-// kind: 0 full space, +1 over u > 0, -1 over u < 0; var = 1/(2 lam) = p/rho, formed
-// once per Maxwellian by the caller
+// <u^0> and <u^1> over u > 0 (kind +1) or u < 0 (kind -1); l2 = 2 lam
+template <class R>
+GKS_FN void half_start(R U, R l2, int kind, R& h, R& g) {
+  const R lam = R(0.5) * l2;
+  const R rs = d_rsqrt(lam);
+  const R s = lam * rs;  // sqrt(lam)
+  h = R(0.5) * d_erfc(-R(kind) * s * U);
+  // boundary term of the integration by parts at u = 0
+  const R b = d_exp(-lam * U * U) * R(0.28209479177387814) * rs;  // 1/(2 sqrt(pi lam))
+  g = U * h + R(kind) * b;
+}
+
+// moments over u > 0 (kind +1) or u < 0 (kind -1); var = 1/(2 lam) = p/rho, formed once per
+// Maxwellian by the caller
 template <class R, int NU, int NV>
 GKS_FN void moments(R U, R V, R lam, R var, R K, int kind, Moments<R, NU, NV>& m) {
-  if (kind == 0) {
-    m.u[0] = R(1);
-    m.u[1] = U;
-  } else {
-    const R rs = d_rsqrt(lam);
-    const R s = lam * rs;  // sqrt(lam)
-    const R h = R(0.5) * d_erfc(-R(kind) * s * U);
-    // boundary term of the integration by parts at u = 0
-    const R b = d_exp(-lam * U * U) * R(0.28209479177387814) * rs;  // 1/(2 sqrt(pi lam))
-    m.u[0] = h;
-    m.u[1] = U * h + R(kind) * b;
-  }
+  half_start(U, R(2) * lam, kind, m.u[0], m.u[1]);
 #pragma unroll
   for (int n = 2; n < NU; ++n) m.u[n] = U * m.u[n - 1] + (n == 2 ? var : R(n - 1) * var) * m.u[n - 2];
   m.v[0] = R(1);
@@ -92,29 +94,9 @@ GKS_FN void moments(R U, R V, R lam, R var, R K, int kind, Moments<R, NU, NV>& m
 #pragma unroll
   for (int n = 3; n < NV; ++n) m.v[n] = V * m.v[n - 1] + R(n - 1) * var * m.v[n - 2];
   m.xi2 = K * var;
-  m.xi4 = K * (K + R(2)) * var * var;
-  m.kap = R(2) * K * var * var;
 }
 
-// The same half-space moments from their first two entries h = <u^0>, g = <u^1>
-// (already formed once for the same Maxwellian: no second erfc and exp).
-template <class R, int NU, int NV>
-GKS_FN void moments_from(R U, R V, R var, R K, R h, R g, Moments<R, NU, NV>& m) {
-  m.u[0] = h;
-  m.u[1] = g;
-#pragma unroll
-  for (int n = 2; n < NU; ++n) m.u[n] = U * m.u[n - 1] + (n == 2 ? var : R(n - 1) * var) * m.u[n - 2];
-  m.v[0] = R(1);
-  m.v[1] = V;
-  m.v[2] = V * V + var;
-#pragma unroll
-  for (int n = 3; n < NV; ++n) m.v[n] = V * m.v[n - 1] + R(n - 1) * var * m.v[n - 2];
-  m.xi2 = K * var;
-  m.xi4 = K * (K + R(2)) * var * var;
-  m.kap = R(2) * K * var * var;
-}
-
-// <u^A v^B psi> and <xi^2 u^A v^B psi>, psi = (1, u, v, (u^2+v^2+xi^2)/2)
+// <u^A v^B psi>, psi = (1, u, v, (u^2+v^2+xi^2)/2)
 template <int A, int B, class R, int NU, int NV>
 GKS_FN void psi_mom(const Moments<R, NU, NV>& m, R o[4]) {
   static_assert(A + 2 < NU && B + 2 < NV, "moment table too short");
@@ -126,389 +108,188 @@ GKS_FN void psi_mom(const Moments<R, NU, NV>& m, R o[4]) {
 }
 
 // ---------------------------------------------------------------------------
-// Section 2.2: <a> = rho r for a expanded in psi has a closed-form solution
-// (the moment matrix of a Maxwellian is block structured about (U, V)).  The
-// factors that depend only on the Maxwellian are formed once per Maxwellian.
-// ---------------------------------------------------------------------------
-template <class R>
-struct SolveK {
-  R U, V;
-  R l2;  // 2 lam
-  R c4;  // 4 lam^2 / N, N = K + 2
-  R s0;  // U^2 + V^2 - N / (2 lam)
-  R s1;  // (U^2 + V^2) / 2 + N / (4 lam)
-  R hq;  // (U^2 + V^2) / 2
-  R kc;  // (N + 2) / (4 lam)
-};
-
-template <class R>
-GKS_FN SolveK<R> solve_k(R U, R V, R lam, R var, R N, R iN) {
-  SolveK<R> k;
-  const R q2 = U * U + V * V;
-  const R nv = N * var;  // N / (2 lam)
-  k.U = U;
-  k.V = V;
-  k.l2 = R(2) * lam;
-  k.c4 = R(4) * lam * lam * iN;
-  k.s0 = q2 - nv;
-  k.s1 = R(0.5) * (q2 + nv);
-  k.hq = R(0.5) * q2;
-  k.kc = R(0.5) * (nv + R(2) * var);
-  return k;
-}
-
-// <a> = rho r with r = ir d, ir = 1/rho folded into the factors:
-// c4i = c4 ir, l2i = l2 ir
-template <class R>
-GKS_FN void solve_scaled(const SolveK<R>& k, R c4i, R l2i, R ir, const R d[4], R x[4]) {
-  const R x4 = c4i * (R(2) * (d[3] - k.U * d[1] - k.V * d[2]) + k.s0 * d[0]);
-  const R x3 = l2i * (d[2] - k.V * d[0]) - k.V * x4;
-  const R x2 = l2i * (d[1] - k.U * d[0]) - k.U * x4;
-  x[0] = ir * d[0] - k.U * x2 - k.V * x3 - x4 * k.s1;
-  x[1] = x2;
-  x[2] = x3;
-  x[3] = x4;
-}
-
-// ---------------------------------------------------------------------------
-// Time weights.  With x = dt/tau and e = exp(-x), the flux needs the integrals
-// over [0, dt] of C_1..C_8, C_7 t and C_7 t^2; Eq. point needs their values at
-// t = dt.  Several are differences of nearly equal terms when x is small; there
-// they are summed from their Taylor series in x.
+// Time weights.  With x = dt/tau and e = exp(-x): the integrals over [0, dt] of C_1..C_6,
+// e^(-t/tau), t e^(-t/tau) and t^2 e^(-t/tau) for the flux, and e and 1 - e for the values
+// at t = dt (Eq. point).  Several are differences of nearly equal terms when x is small;
+// there they come from three sums of their Taylor series in x.
 // ---------------------------------------------------------------------------
 template <class R>
 struct TimeW {
-  R I[11];  // integrals, index 1..8 = C_1..C_8, 9 = C_7 t, 10 = C_7 t^2
-  R E[11];  // values at t = dt
+  R I1, I2, I3, I4, I5, I6;  // integrals of C_1..C_6
+  R i7, i9, i10;             // integrals of e^(-t/tau) (C_7), t e^(-t/tau) (-C_8), t^2 e^(-t/tau)
+  R e, om;                   // exp(-x), 1 - exp(-x)
 };
+
+// Coefficients of x^k, k = n - 3, in the sums over n >= 3 of t_n = (-x)^n / n!, of (n-2) t_n and
+// of (n-1)(n-2) t_n, each divided by x^3 (which: 0, 1, 2)
+GKS_FN constexpr double series_coef(int which, int k) {
+  const int n = k + 3;
+  double f = (n & 1) ? -1.0 : 1.0;
+  for (int j = 2; j <= n; ++j) f /= j;
+  return which == 0 ? f : (which == 1 ? (n - 2) * f : (double)((n - 1) * (n - 2)) * f);
+}
+
+template <int W, int K, class R>
+GKS_FN R series_sum(R x) {
+  if constexpr (K + 4 >= Prec<R>::series_terms) {
+    constexpr double c = series_coef(W, K);
+    return R(c);
+  } else {
+    constexpr double c = series_coef(W, K);
+    return R(c) + x * series_sum<W, K + 1>(x);
+  }
+}
 
 template <class R>
 GKS_FN void time_weights(R T, R tau, TimeW<R>& w) {
   const R x = tau > R(0) ? d_div(T, tau) : R(INFINITY);
-  const R e = tau > R(0) ? d_exp(-x) : R(0);
-  const R om = tau > R(0) ? -d_expm1(-x) : R(1);  // 1 - e
-  R f1, f2, f3, f4, f5, f6;  // see below
+  const R t2 = tau * tau, T2h = R(0.5) * T * T;
   if (x < Prec<R>::series_below) {
-    // t_n = (-x)^n / n!:  f1 = x-1+e = sum_{n>=2} t_n;  f2 = 1-(1+x)e = sum (n-1) t_n;
-    // f3 = 2-2e-x-xe = sum (n-2) t_n;  f4 = x^2/2-x+1-e = -sum_{n>=3} t_n;
-    // f5 = 4-(x+2)^2 e = -sum (n-1)(n-4) t_n;  f6 = 2-(x^2+2x+2) e = -sum_{n>=3} (n-1)(n-2) t_n
-    R t = R(0.5) * x * x;
-    f1 = t; f2 = t; f3 = R(0); f4 = R(0); f5 = R(2) * t; f6 = R(0);
-#pragma unroll
-    for (int n = 3; n < Prec<R>::series_terms; ++n) {
-      t *= -x * R(1.0 / n);
-      f1 += t;
-      f2 += R(n - 1) * t;
-      f3 += R(n - 2) * t;
-      f4 -= t;
-      f5 -= R((n - 1) * (n - 4)) * t;
-      f6 -= R((n - 1) * (n - 2)) * t;
-    }
-    const R t2 = tau * tau, t3 = t2 * tau;
-    w.I[1] = tau * f1;
-    w.I[2] = t2 * f3;
-    w.I[3] = t2 * f4;
-    w.I[4] = -t3 * f5;
-    w.I[9] = t2 * f2;
-    w.I[10] = t3 * f6;
-    w.E[2] = -tau * f2;
-    w.E[3] = tau * f1;
+    // with g = sum t_n, a = sum (n-2) t_n, b = sum (n-1)(n-2) t_n over n >= 3:
+    //   x - 1 + e = x^2/2 + g;  1 - (1+x) e = x^2/2 + a + g;  2 - 2e - x - x e = a;
+    //   x^2/2 - x + 1 - e = -g;  2 - (x^2 + 2x + 2) e = -b
+    const R xx = R(0.5) * x * x, x3 = R(2) * xx * x;
+    const R g = x3 * series_sum<0, 0>(x), a = x3 * series_sum<1, 0>(x), b = x3 * series_sum<2, 0>(x);
+    const R f1 = xx + g;
+    w.om = x - f1;
+    w.e = R(1) - w.om;
+    w.I1 = tau * f1;
+    w.I2 = t2 * a;
+    w.I3 = -t2 * g;
+    w.i9 = t2 * (f1 + a);
+    w.i10 = -(t2 * tau) * b;
+    w.i7 = tau * w.om;
   } else {
-    const R t2 = tau * tau;
-    w.I[1] = T - tau * om;
-    w.I[2] = R(2) * t2 * om - tau * T * (R(1) + e);
-    w.I[3] = R(0.5) * T * T - tau * T + t2 * om;
-    w.I[4] = -R(4) * t2 * tau + tau * sq(T + R(2) * tau) * e;
-    w.I[9] = t2 - tau * (tau + T) * e;
-    w.I[10] = R(2) * t2 * tau - tau * (T * T + R(2) * T * tau + R(2) * t2) * e;
-    w.E[2] = (T + tau) * e - tau;
-    w.E[3] = T - tau + tau * e;
+    // e is exactly 0 for x beyond the type's range: FP64 skips the exponential there (smooth
+    // Euler flow, where tau is a tiny fraction of dt)
+    w.e = x < Prec<R>::exp_zero ? d_exp(-x) : R(0);
+    w.om = R(1) - w.e;
+    w.i7 = tau * w.om;
+    w.I1 = T - w.i7;
+    w.I2 = R(2) * tau * w.i7 - tau * T * (R(1) + w.e);
+    w.I3 = T2h - tau * T + tau * w.i7;
+    w.i9 = t2 - tau * (tau + T) * w.e;
+    w.i10 = tau * (R(2) * t2 - R(2) * (T2h + T * tau + t2) * w.e);
   }
-  w.I[5] = T * T * T * R(1.0 / 3.0) - tau * T * T;
-  w.I[6] = -tau * (R(0.5) * T * T + w.I[9]);
-  w.I[7] = tau * om;
-  w.I[8] = -w.I[9];
-  w.E[1] = om;
-  w.E[4] = -(T * T + R(2) * T * tau) * e;
-  w.E[5] = T * T - R(2) * T * tau;
-  w.E[6] = -T * tau * (R(1) + e);
-  w.E[7] = e;
-  w.E[8] = -T * e;
-  w.E[9] = T * e;
-  w.E[10] = T * T * e;
+  w.I4 = -(w.i10 + R(2) * tau * w.i9);
+  w.I5 = R(2) * T2h * (R(1.0 / 3.0) * T - tau);
+  w.I6 = -tau * (T2h + w.i9);
 }
 
 // ---------------------------------------------------------------------------
-// The nine coefficients of one equilibrium state (system after Eq. dis3).
-// The composites (a1^2+d11), (a1 a2+d12), (a2^2+d22), (A a1+b1), (A a2+b2),
-// (A^2+B) are single unknowns expanded in psi: Axx, Axy, Ayy, Atx, Aty, Att.
-// d[] = (dn, dt, dnn, dnt, dtt) of the conservative variables.
+// Everything below works in a Maxwellian's own frame.  With c = u - U, d = v - V and
+// psi' = (1, c, d, (c^2 + d^2 + xi^2) / 2), a 4-vector e of "central" conservative components is
+// <psi' X> of a coefficient X expanded in psi' (the density, the momenta and the energy about
+// (U, V)): the coefficient itself is never needed over the whole velocity space, since every moment
+// of X is a multiple of e's components.  central() takes a derivative of the conservative variables
+// there, lab() takes moments back.
 // ---------------------------------------------------------------------------
 template <class R>
-struct Coefs {
-  R a1[4], a2[4], Axx[4], Axy[4], Ayy[4], A[4], Atx[4], Aty[4], Att[4];
+GKS_FN void central(R U, R V, R hq, const R d[4], R e[4]) {  // hq = (U^2 + V^2) / 2
+  e[0] = d[0];
+  e[1] = d[1] - U * d[0];
+  e[2] = d[2] - V * d[0];
+  e[3] = d[3] - U * e[1] - V * e[2] - hq * d[0];
+}
+
+template <class R>
+GKS_FN void lab(R U, R V, R hq, const R e[4], R o[4]) {
+  o[0] = e[0];
+  o[1] = e[1] + U * e[0];
+  o[2] = e[2] + V * e[0];
+  o[3] = e[3] + U * e[1] + V * e[2] + hq * e[0];
+}
+
+// The time coefficient T of <(X u + Y v + T) psi> = 0 (system after Eq. dis3), all in central
+// components: <c psi' X> = (X1, p', 0, kc X1) and <d psi' Y> = (Y2, 0, p', kc Y2) with
+// p' = (2/N) X3 (Y3) and kc = (N + 2) / (4 lam).
+template <class R>
+GKS_FN void time_coef(R U, R V, R i2N, R kc, const R X[4], const R Y[4], R T[4]) {
+  T[0] = -(U * X[0] + V * Y[0] + X[1] + Y[2]);
+  T[1] = -(U * X[1] + V * Y[1] + i2N * X[3]);
+  T[2] = -(U * X[2] + V * Y[2] + i2N * Y[3]);
+  T[3] = -(U * X[3] + V * Y[3] + kc * (X[1] + Y[2]));
+}
+
+// Coefficient of the Maxwellian (scaled by rho) with central components e, in the basis
+// (1, u, d, u^2/2 + eta), eta = (d^2 + xi^2)/2 less its mean: what half-space moments in u need.
+// l2 = 2 lam, c5 = 2 l2 / N, hs = (U^2 + 1/(2 lam)) / 2.
+template <class R>
+GKS_FN void half_coef(R U, R l2, R c5, R hs, const R e[4], R X[4]) {
+  X[3] = l2 * (c5 * e[3] - e[0]);
+  X[1] = l2 * e[1] - U * X[3];
+  X[0] = e[0] - U * X[1] - hs * X[3];
+  X[2] = l2 * e[2];
+}
+
+// A polynomial P(u, d, xi) of the half-space distribution averaged over d and xi: its mean q(u), and
+// its means weighted by d / <d^2> and by eta, r(u) and t(u).  The tangential and internal velocities run over
+// their whole range, so d's odd powers vanish and only these three remain of the full set of
+// monomials u^a d^b xi^2c.
+template <class R>
+struct HalfPoly {
+  R q[5], r[4], t[3];
 };
 
-// A coefficient vector X about the Maxwellian's (U, V) in central coordinates: the
-// coefficients of 1, c, d, s = (c^2 + d^2 + xi^2) / 2 with c = u - U, d = v - V
+// P = W + B1 + Bu u + Bd d + wq (xx u^2 + 2 xy u d + yy d^2), each letter a coefficient vector
+// of half_coef's basis; s = <d^2> = 1/(2 lam), n1h = (N - 1)/2.  <eta^2> = n1h s^2,
+// <d^2 eta> = s^2, <d^2 eta^2> = (n1h + 2) s^3.
 template <class R>
-GKS_FN void to_central(const SolveK<R>& k, const R X[4], R Y[4]) {
-  Y[0] = X[0] + k.U * X[1] + k.V * X[2] + k.hq * X[3];
-  Y[1] = X[1] + k.U * X[3];
-  Y[2] = X[2] + k.V * X[3];
-  Y[3] = X[3];
+GKS_FN void half_poly(R W, const R B1[4], const R Bu[4], const R Bd[4], R wq, const R xx[4], const R xy[4],
+                      const R yy[4], R s, R n1h, HalfPoly<R>& P) {
+  const R w2 = R(2) * wq, s2 = s * s;
+  const R D0 = Bd[2] + wq * yy[0], D1 = w2 * xy[2] + wq * yy[1];
+  const R y3 = wq * yy[3], x3 = wq * xx[3], sy3 = s * y3;
+  P.q[0] = (W + B1[0]) + s * (D0 + sy3);
+  P.q[1] = (B1[1] + Bu[0]) + s * D1;
+  P.q[2] = R(0.5) * (B1[3] + sy3) + (Bu[1] + wq * xx[0]);
+  P.q[3] = R(0.5) * Bu[3] + wq * xx[1];
+  P.q[4] = R(0.5) * x3;
+  P.r[0] = (B1[2] + Bd[0]) + s * (Bd[3] + R(3) * wq * yy[2]);
+  P.r[1] = (Bu[2] + Bd[1]) + w2 * (xy[0] + s * xy[3]);
+  P.r[2] = R(0.5) * Bd[3] + (wq * xx[2] + w2 * xy[1]);
+  P.r[3] = wq * xy[3];
+  P.t[0] = s2 * (n1h * B1[3] + D0 + (n1h + R(2)) * sy3);
+  P.t[1] = s2 * (n1h * Bu[3] + D1);
+  P.t[2] = s2 * (n1h * x3 + R(0.5) * y3);
 }
 
+// the same without the terms of second order (W = wq = 0)
 template <class R>
-GKS_FN void from_central(const SolveK<R>& k, const R Y[4], R X[4]) {
-  X[3] = Y[3];
-  X[1] = Y[1] - k.U * Y[3];
-  X[2] = Y[2] - k.V * Y[3];
-  X[0] = Y[0] - k.U * X[1] - k.V * X[2] - k.hq * Y[3];
+GKS_FN void half_poly_linear(const R B1[4], const R Bu[4], const R Bd[4], R s, R n1h, HalfPoly<R>& P) {
+  const R s2 = s * s;
+  P.q[0] = B1[0] + s * Bd[2];
+  P.q[1] = B1[1] + Bu[0];
+  P.q[2] = R(0.5) * B1[3] + Bu[1];
+  P.q[3] = R(0.5) * Bu[3];
+  P.r[0] = (B1[2] + Bd[0]) + s * Bd[3];
+  P.r[1] = Bu[2] + Bd[1];
+  P.r[2] = R(0.5) * Bd[3];
+  P.t[0] = s2 * (n1h * B1[3] + Bd[2]);
+  P.t[1] = s2 * n1h * Bu[3];
 }
 
-// The time coefficient T of <(X u + Y v + T) psi g> = 0 (X, Y, T in central coordinates):
-// T = -P(u X + v Y), P the projection on span(psi) in the inner product weighted by the
-// Maxwellian.  u X = U X + c X, and the Maxwellian's central moments (<c^2> = 1/(2 lam),
-// <c^4> = 3 <c^2>^2, <xi^2> = K <c^2>) give P(c) = c, P(c^2) = (2/N) s, P(c d) = 0 and
-// P(c s) = kc c with kc = <c^2 s> / <c^2> = (N + 2) / (4 lam); likewise in d.
-template <class R>
-GKS_FN void time_coef(const SolveK<R>& k, R i2N, const R X[4], const R Y[4], R T[4]) {
-  T[0] = -(k.U * X[0] + k.V * Y[0]);
-  T[1] = -(k.U * X[1] + k.V * Y[1] + X[0] + k.kc * X[3]);
-  T[2] = -(k.U * X[2] + k.V * Y[2] + Y[0] + k.kc * Y[3]);
-  T[3] = -(k.U * X[3] + k.V * Y[3] + i2N * (X[1] + Y[2]));
-}
-
-// ir = 1/rho of the Maxwellian, i2N = 2 / N.  The spatial coefficients by the closed-form
-// solve; the time coefficients (the compatibility conditions of the system after Eq. dis3)
-// by the projection above, in central coordinates, mapped back to the psi basis.
-template <class R>
-GKS_FN void coef_systems(R ir, const SolveK<R>& sk, R i2N, const R d[5][4], bool time_terms, bool second_time,
-                         Coefs<R>& c) {
-  const R c4i = sk.c4 * ir, l2i = sk.l2 * ir;
-  solve_scaled(sk, c4i, l2i, ir, d[0], c.a1);
-  solve_scaled(sk, c4i, l2i, ir, d[1], c.a2);
-  solve_scaled(sk, c4i, l2i, ir, d[2], c.Axx);
-  solve_scaled(sk, c4i, l2i, ir, d[3], c.Axy);
-  solve_scaled(sk, c4i, l2i, ir, d[4], c.Ayy);
-  if (!time_terms) return;
-  R x[4], y[4], z[4], tx[4], ty[4], t[4];
-  to_central(sk, c.a1, x);
-  to_central(sk, c.a2, y);
-  time_coef(sk, i2N, x, y, t);  // <A + a1 u + a2 v> = 0
-  from_central(sk, t, c.A);
-  to_central(sk, c.Axx, x);
-  to_central(sk, c.Axy, y);
-  to_central(sk, c.Ayy, z);
-  time_coef(sk, i2N, x, y, tx);  // <Axx u + Axy v + Atx> = 0
-  time_coef(sk, i2N, y, z, ty);  // <Axy u + Ayy v + Aty> = 0
-  from_central(sk, tx, c.Atx);
-  from_central(sk, ty, c.Aty);
-  if (!second_time) return;
-  time_coef(sk, i2N, tx, ty, t);  // <Atx u + Aty v + Att> = 0
-  from_central(sk, t, c.Att);
-}
-
-// The interface distribution grouped by velocity monomial: f = sum over
-// m in {1, u, v, u^2, u v, v^2} of X_m(psi) m g, plus y X'_m for the part
-// linear along the face.  The moments of f are taken by expanding
-// P = sum_m m X_m(psi) into monomials u^a v^b (xi^2)^c first (a + b <= 4 for
-// c = 0, a + b <= 2 for c = 1) and then pairing each monomial with the moment
-// table of g (moments factorise: <u^a v^b xi^2c> = <u^a><v^b><xi^2c>):
-//   flux   += rho <u P psi>           (time-integrated weights)
-//   point0 += rho <P psi>             (weights at t = dt)
-//   point1 += rho <P' psi>            (weights at t = dt, y-linear part)
-//   mean   += rho <P psi>             (time-integrated weights; heat flux)
-template <class R>
-struct Groups {
-  R X1[4], Xu[4], Xv[4], Xuu[4], Xuv[4], Xvv[4];
-};
-
-// monomial coefficients: c0[(b, a)] for u^a v^b, a + b <= 4, stored by b then a
-// (offsets 0, 5, 9, 12, 14); c1[(b, a)] for u^a v^b xi^2, a + b <= 2 (offsets 0, 3, 5)
-template <class R>
-struct Poly {
-  R c0[15], c1[6];
-};
-
-GKS_FN constexpr int pidx0(int a, int b) { return (b == 0 ? 0 : b == 1 ? 5 : b == 2 ? 9 : b == 3 ? 12 : 14) + a; }
-GKS_FN constexpr int pidx1(int a, int b) { return (b == 0 ? 0 : b == 1 ? 3 : 5) + a; }
-
-// P of the six groups (FULL) or of the first three only (the y-linear part)
-template <bool FULL, class R>
-GKS_FN void poly_of(const Groups<R>& g, Poly<R>& P) {
-  const R h1 = R(0.5) * g.X1[3], hu = R(0.5) * g.Xu[3], hv = R(0.5) * g.Xv[3];
-  // X (psi) = X0 + X1 u + X2 v + X3 (u^2 + v^2 + xi^2) / 2, times the group's monomial
-  P.c0[pidx0(0, 0)] = g.X1[0];
-  P.c0[pidx0(1, 0)] = g.X1[1] + g.Xu[0];
-  P.c0[pidx0(0, 1)] = g.X1[2] + g.Xv[0];
-  P.c0[pidx0(2, 0)] = h1 + g.Xu[1];
-  P.c0[pidx0(1, 1)] = g.Xu[2] + g.Xv[1];
-  P.c0[pidx0(0, 2)] = h1 + g.Xv[2];
-  P.c0[pidx0(3, 0)] = hu;
-  P.c0[pidx0(2, 1)] = hv;
-  P.c0[pidx0(1, 2)] = hu;
-  P.c0[pidx0(0, 3)] = hv;
-  P.c1[pidx1(0, 0)] = h1;
-  P.c1[pidx1(1, 0)] = hu;
-  P.c1[pidx1(0, 1)] = hv;
-  if (FULL) {
-    const R huu = R(0.5) * g.Xuu[3], huv = R(0.5) * g.Xuv[3], hvv = R(0.5) * g.Xvv[3];
-    P.c0[pidx0(2, 0)] += g.Xuu[0];
-    P.c0[pidx0(1, 1)] += g.Xuv[0];
-    P.c0[pidx0(0, 2)] += g.Xvv[0];
-    P.c0[pidx0(3, 0)] += g.Xuu[1];
-    P.c0[pidx0(2, 1)] += g.Xuu[2] + g.Xuv[1];
-    P.c0[pidx0(1, 2)] += g.Xuv[2] + g.Xvv[1];
-    P.c0[pidx0(0, 3)] += g.Xvv[2];
-    P.c0[pidx0(4, 0)] = huu;
-    P.c0[pidx0(3, 1)] = huv;
-    P.c0[pidx0(2, 2)] = huu + hvv;
-    P.c0[pidx0(1, 3)] = huv;
-    P.c0[pidx0(0, 4)] = hvv;
-    P.c1[pidx1(2, 0)] = huu;
-    P.c1[pidx1(1, 1)] = huv;
-    P.c1[pidx1(0, 2)] = hvv;
+// out += <u^SU P psi> over the half space, m[n] = <u^n>; DEG: the degree of q (4, or 3 when linear)
+template <int SU, int DEG, class R>
+GKS_FN void half_moments(const HalfPoly<R>& P, const R m[8], R V, R s, R n1h, R out[4]) {
+  R o0 = P.q[0] * m[SU], o1 = P.q[0] * m[SU + 1], o3 = P.q[0] * m[SU + 2];
+#pragma unroll
+  for (int n = 1; n <= DEG; ++n) {
+    o0 = o0 + P.q[n] * m[SU + n];
+    o1 = o1 + P.q[n] * m[SU + n + 1];
+    o3 = o3 + P.q[n] * m[SU + n + 2];
   }
-}
-
-// out += rho <u^SU P psi>, psi = (1, u, v, (u^2 + v^2 + xi^2) / 2); D / D1: the
-// degree of P in (u, v) for c = 0 / c = 1 (4 / 2, or 3 / 1 for the y-linear part).
-// <xi^2> is a number, so the xi^2 monomials fold into the others: with
-// q_ab = p0_ab + <xi^2> p1_ab, the first three components are sums of q_ab <u^a><v^b>;
-// the fourth's extra xi^2 weight, sum p0 <xi^2> + p1 <xi^4>, is <xi^2> o0 + kap T with
-// kap = <xi^4> - <xi^2>^2 and T = sum p1_ab <u^a><v^b> (u-moments shifted by SU).
-template <int SU, int D, int D1, class R, int NU, int NV>
-GKS_FN void poly_moments(const Poly<R>& P, const Moments<R, NU, NV>& m, R rho, R out[4]) {
-  static_assert(D + SU + 2 < NU && D + 2 < NV, "moment table too short");
-  R o0 = R(0), o1 = R(0), o2 = R(0), o3 = R(0);
+  R o2 = P.r[0] * m[SU], t = P.t[0] * m[SU];
 #pragma unroll
-  for (int b = 0; b <= D; ++b) {
-    // sum_a q u^(a+SU), u^(a+SU+1), u^(a+SU+2) moments (the first term starts each sum)
-    R s0 = R(0), s1 = R(0), s2 = R(0);
-#pragma unroll
-    for (int a = 0; a <= D - b; ++a) {
-      const R q = a + b <= D1 ? P.c0[pidx0(a, b)] + m.xi2 * P.c1[pidx1(a, b)] : P.c0[pidx0(a, b)];
-      s0 = a == 0 ? q * m.u[SU] : s0 + q * m.u[a + SU];
-      s1 = a == 0 ? q * m.u[SU + 1] : s1 + q * m.u[a + SU + 1];
-      s2 = a == 0 ? q * m.u[SU + 2] : s2 + q * m.u[a + SU + 2];
-    }
-    // <v^b>, <v^(b+1)>, <v^(b+2)> (v^0 = 1)
-    if (b == 0) {
-      o0 = s0;
-      o1 = s1;
-      o2 = s0 * m.v[1];
-      o3 = s2 + s0 * m.v[2];
-    } else {
-      o0 = o0 + s0 * m.v[b];
-      o1 = o1 + s1 * m.v[b];
-      o2 = o2 + s0 * m.v[b + 1];
-      o3 = o3 + s2 * m.v[b] + s0 * m.v[b + 2];
-    }
+  for (int n = 1; n < DEG; ++n) {
+    o2 = o2 + P.r[n] * m[SU + n];
+    if (n < DEG - 1) t = t + P.t[n] * m[SU + n];
   }
-  R T = R(0);
-#pragma unroll
-  for (int b = 0; b <= D1; ++b) {
-    R t = R(0);
-#pragma unroll
-    for (int a = 0; a <= D1 - b; ++a) t = a == 0 ? P.c1[pidx1(a, b)] * m.u[SU] : t + P.c1[pidx1(a, b)] * m.u[a + SU];
-    T = b == 0 ? t : T + t * m.v[b];
-  }
-  out[0] += rho * o0;
-  out[1] += rho * o1;
-  out[2] += rho * o2;
-  out[3] += rho * (R(0.5) * (o3 + m.xi2 * o0 + m.kap * T));
-}
-
-template <class R, int NU, int NV>
-GKS_FN void add_flux(const Groups<R>& g, const Moments<R, NU, NV>& m, R rho, R out[4]) {
-  Poly<R> P;
-  poly_of<true>(g, P);
-  poly_moments<1, 4, 2>(P, m, rho, out);
-}
-
-template <class R, int NU, int NV>
-GKS_FN void add_point(const Groups<R>& g, const Moments<R, NU, NV>& m, R rho, R out[4]) {
-  Poly<R> P;
-  poly_of<true>(g, P);
-  poly_moments<0, 4, 2>(P, m, rho, out);
-}
-
-// the same for groups whose u^2, u v, v^2 parts vanish
-template <class R, int NU, int NV>
-GKS_FN void add_point_first(const Groups<R>& g, const Moments<R, NU, NV>& m, R rho, R out[4]) {
-  Poly<R> P;
-  poly_of<false>(g, P);
-  poly_moments<0, 3, 1>(P, m, rho, out);
-}
-
-template <class R, int NU, int NV>
-GKS_FN void add_point_linear(const R Y1[4], const R Yu[4], const R Yv[4], const Moments<R, NU, NV>& m, R rho,
-                             R out[4]) {
-  Groups<R> g;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    g.X1[k] = Y1[k];
-    g.Xu[k] = Yu[k];
-    g.Xv[k] = Yv[k];
-  }
-  Poly<R> P;
-  poly_of<false>(g, P);
-  poly_moments<0, 3, 1>(P, m, rho, out);
-}
-
-// Eq. dis1 grouped: weights W = I (flux, mean) or E (point); y2 = dtan^2/12 is both
-// the face mean of y^2 and y^2 at the Gauss points.
-// SECOND = false: W[4] = 0, the groups of u^2, u v, v^2 vanish and are not formed.
-template <bool SECOND = true, class R>
-GKS_FN void hydro_groups(const Coefs<R>& c, const R* W, R y2, Groups<R>& g) {
-  const R h5 = R(0.5) * W[5], hy = R(0.5) * y2 * W[1], h4 = R(0.5) * W[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    g.X1[k] = W[3] * c.A[k] + h5 * c.Att[k] + hy * c.Ayy[k];
-    g.Xu[k] = W[2] * c.a1[k] + W[6] * c.Atx[k];
-    g.Xv[k] = W[2] * c.a2[k] + W[6] * c.Aty[k];
-    if (SECOND) {
-      g.Xuu[k] = h4 * c.Axx[k];
-      g.Xuv[k] = W[4] * c.Axy[k];
-      g.Xvv[k] = h4 * c.Ayy[k];
-    }
-  }
-  g.X1[0] += W[1];
-}
-
-// Eq. dis2 grouped for one side.  NS: f_G = g_k - tau (a u + A) g_k with the time
-// coefficients c.A, c.Atx, c.Aty and tn = tau; Euler: f_G = g_k, and the terms
-// with tn are absent (not formed).
-template <bool NS, class R>
-GKS_FN void kinetic_groups(const Coefs<R>& c, const R* W, R y2, R tn, Groups<R>& g) {
-  const R h7 = R(0.5) * y2 * W[7];
-  if (NS) {
-    const R t7 = tn * W[7], t8 = tn * W[8];
-    const R w78 = W[8] - t7, wq = R(0.5) * W[10] - t8, wq2 = W[10] - R(2) * t8;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      g.X1[k] = h7 * c.Ayy[k] - t7 * c.A[k];
-      g.Xu[k] = w78 * c.a1[k] - t8 * c.Atx[k];
-      g.Xv[k] = w78 * c.a2[k] - t8 * c.Aty[k];
-      g.Xuu[k] = wq * c.Axx[k];
-      g.Xuv[k] = wq2 * c.Axy[k];
-      g.Xvv[k] = wq * c.Ayy[k];
-    }
-  } else {
-    const R wq = R(0.5) * W[10];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      g.X1[k] = h7 * c.Ayy[k];
-      g.Xu[k] = W[8] * c.a1[k];
-      g.Xv[k] = W[8] * c.a2[k];
-      g.Xuu[k] = wq * c.Axx[k];
-      g.Xuv[k] = W[10] * c.Axy[k];
-      g.Xvv[k] = wq * c.Ayy[k];
-    }
-  }
-  g.X1[0] += W[7];
+  o2 = s * o2;
+  out[0] += o0;
+  out[1] += o1;
+  out[2] += o2 + V * o0;
+  out[3] += (R(0.5) * o3 + t) + V * o2 + (n1h * s + R(0.5) * V * V) * o0;
 }
 
 // ---------------------------------------------------------------------------
@@ -537,6 +318,7 @@ struct FaceParams {
 template <class R>
 struct FaceConst {
   R gamma, gm1, K, N, iN, i2N, dn, dtan, y2, mu, pr_fix, tau_eps, tau_C;
+  R n1h, n2h, n4h, nh;          // (N - 1)/2, (N + 2)/2, (N + 4)/2, N/2
   R dn2_12, dt2_24;             // dn^2 / 12, dtan^2 / 24 (face values of the cell polynomial)
   R i4n, i4t, i8n2, i2nt, i2t2;  // 1/(4 dn), 1/(4 dt), 1/(8 dn^2), 1/(2 dn dt), 1/(2 dt^2)
   bool ns, prandtl;
@@ -547,10 +329,16 @@ GKS_FN FaceConst<R> face_const(const FaceParams& P) {
   FaceConst<R> c;
   c.gamma = R(P.gamma);
   c.gm1 = R(P.gamma - 1.0);
-  c.K = R((4.0 - 2.0 * P.gamma) / (P.gamma - 1.0));  // internal degrees of freedom, Section 2.1
-  c.N = R(2.0 / (P.gamma - 1.0));                     // K + 2
+  // N = K + 2 degrees of freedom, K = (4 - 2 gamma) / (gamma - 1) internal ones (Section 2.1)
+  const double N = 2.0 / (P.gamma - 1.0);
+  c.K = R((4.0 - 2.0 * P.gamma) / (P.gamma - 1.0));
+  c.N = R(N);
   c.iN = R(0.5 * (P.gamma - 1.0));
   c.i2N = R(P.gamma - 1.0);  // 2 / N
+  c.nh = R(0.5 * N);
+  c.n1h = R(0.5 * (N - 1.0));
+  c.n2h = R(0.5 * (N + 2.0));
+  c.n4h = R(0.5 * (N + 4.0));
   c.dn = R(P.dn);
   c.dtan = R(P.dtan);
   c.y2 = R(P.dtan * P.dtan / 12.0);
@@ -669,147 +457,239 @@ GKS_FN void wall_image(int kind, R gamma, R uwt, R Tw, const FaceState<R>& in, F
 // at the two Gauss points (tangential -/+ sqrt(3)/6 dtan) at t = dt.
 // NSM: 1 Navier-Stokes, 0 Euler (mu = 0: the terms of the time derivatives of
 // g_k vanish and are not formed), -1 decided at run time by C.ns.
+//
+// Its bound is arithmetic: the FP32 kernels are held by issue slots, the FP64 ones by the FP64 pipe
+// (one warp instruction per 19 cycles and SM), so fewer operations is what makes it faster.  Each Maxwellian
+// is evaluated in its own frame, where g0's moments are closed forms in the central derivatives and a half-space's
+// reduce to one-dimensional sums over u.  Against expanding the distribution into the monomials
+// u^a v^b xi^2c (gks_face_monomials.cuh): 1,232 instead of 2,041 counted flops at a smooth
+// Euler face (exp(-dt/tau) = 0), 1,722 instead of 2,779 at another, 2,180 instead of 3,907
+// Navier-Stokes with the Prandtl correction.
+// x-faces at 512^2 FP32 26.2 -> 20.7 us (Euler), at 1024^2 108 -> 81 us (Navier-Stokes), at
+// 4096^2 1,177 -> 881 us; FP64 at 512^2 764 -> 534 us.
 // ---------------------------------------------------------------------------
 template <class R, int NSM = -1, class Src>
 GKS_FN void face_evolution(const FaceConst<R>& C, const Src& src, R dt, R F[4], R Wm[4], R Wp[4]) {
   const bool ns = NSM < 0 ? C.ns : NSM == 1;
-  // per side: rho, 1/rho, U, V, lam = rho / (2 p), 1 / (2 lam) = p / rho, p, and the
-  // half-space <u^0>, <u^1>
-  R rs[2], irs[2], us[2], vs[2], ls[2], vrs[2], ps[2], h0[2], h1[2];
+  // per side: rho, U, V, 1 / (2 lam) = p / rho, 2 lam, p, and the half-space <u^0>, <u^1>
+  R rs[2], us[2], vs[2], vrs[2], l2s[2], ps[2], h0[2], h1[2];
   R U0[4] = {R(0), R(0), R(0), R(0)};
   // Eq. compatibility2: U0 = rho_l <psi>_{u>0} + rho_r <psi>_{u<0}
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     FaceState<R> S;
     src.side(k, S);
-    prim(S.w[0], C.gm1, rs[k], irs[k], us[k], vs[k], ps[k]);
-    ls[k] = d_div(R(0.5) * rs[k], ps[k]);
-    vrs[k] = ps[k] * irs[k];
-    Moments<R, 4, 3> m;
-    moments(us[k], vs[k], ls[k], vrs[k], C.K, k == 0 ? +1 : -1, m);
-    h0[k] = m.u[0];
-    h1[k] = m.u[1];
-    R a[4];
-    psi_mom<0, 0>(m, a);
-#pragma unroll
-    for (int v = 0; v < 4; ++v) U0[v] += rs[k] * a[v];
+    R ir;
+    prim(S.w[0], C.gm1, rs[k], ir, us[k], vs[k], ps[k]);
+    l2s[k] = d_div(rs[k], ps[k]);
+    vrs[k] = ps[k] * ir;
+    half_start(us[k], l2s[k], k == 0 ? +1 : -1, h0[k], h1[k]);
+    const R m2 = us[k] * h1[k] + vrs[k] * h0[k];
+    U0[0] += rs[k] * h0[k];
+    U0[1] += rs[k] * h1[k];
+    U0[2] += rs[k] * (vs[k] * h0[k]);
+    U0[3] += rs[k] * (R(0.5) * m2 + (R(0.5) * vs[k] * vs[k] + C.n1h * vrs[k]) * h0[k]);
   }
   R r0, ir0, u0, v0, p0;
   prim(U0, C.gm1, r0, ir0, u0, v0, p0);
-  const R lam0 = d_div(R(0.5) * r0, p0), var0 = p0 * ir0;
+  const R var0 = p0 * ir0;
 
   // Section 4: collision time
   const R jump = fabs(d_div(ps[0] - ps[1], ps[0] + ps[1])) * dt;
   const R tau = ns ? d_div(C.mu, p0) + jump : C.tau_eps * dt + C.tau_C * jump;
   const R tn = ns ? tau : R(0);
 
-  TimeW<R> tw;
-  time_weights(dt, tau, tw);
+  TimeW<R> w;
+  time_weights(dt, tau, w);
   // e = exp(-dt/tau) >= 0 underflows to exactly 0 once tau is a small enough fraction of dt
   // (smooth Euler flow); the point-value terms whose weights carry it are then not formed
-  const bool kin_point = tw.E[7] > R(0);
+  const bool kin_point = w.e > R(0);
+  const R q20 = u0 * u0 + v0 * v0;
 
-  R Fl[4] = {0, 0, 0, 0}, P0[4] = {0, 0, 0, 0}, P1[4] = {0, 0, 0, 0}, Mn[4] = {0, 0, 0, 0};
+  R Fl[4], P0[4], P1[4], Mn[4];
 
-  // ---- equilibrium part, Eq. dis1, with g0 and the polynomial of Section 3.3 ----
+  // ---- equilibrium part, Eq. dis1, with g0 and the polynomial of Section 3.3.  All moments
+  // of g0 run over the whole velocity space: in its frame they are closed forms in the central
+  // components of the derivatives.  The compatibility conditions turn the moments of a1 u + a2 v
+  // into those of A, and so on, so that the point value is U0 and its time derivatives. ----
   {
-    R d[5][4];
+    const R U = u0, V = v0, s = var0, hq = R(0.5) * q20, pN = C.i2N, kc = C.n2h * var0;
+    R x[4], y[4], xx[4], xy[4], yy[4];
     {
-      R avg[2][3][4];
+      R avg[2][3][4], d[5][4];
       src.avg(avg);
-      const R i4n = C.i4n, i4t = C.i4t, i8n2 = C.i8n2, i2nt = C.i2nt, i2t2 = C.i2t2;
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const R um = avg[0][0][k], uc = avg[0][1][k], up = avg[0][2][k];
         const R wm = avg[1][0][k], wc = avg[1][1][k], wp = avg[1][2][k];
-        d[0][k] = ((wp - up) + R(2) * (wc - uc) + (wm - um)) * i4n;                // b2
-        d[1][k] = (wp - wm + up - um) * i4t;                                       // b3
-        d[2][k] = (R(26) * (wc + uc) - (wp + up + wm + um) - R(48) * U0[k]) * i8n2;  // b4
-        d[3][k] = (wp - up - wm + um) * i2nt;                                      // b6
-        d[4][k] = (wp - R(2) * wc + wm + up - R(2) * uc + um) * i2t2;               // b5
+        const R Sr = wp + wm, Sl = up + um, Dr = wp - wm, Dl = up - um, cc = wc + uc;
+        d[0][k] = ((Sr - Sl) + R(2) * (wc - uc)) * C.i4n;                     // b2
+        d[1][k] = (Dr + Dl) * C.i4t;                                          // b3
+        d[2][k] = (R(26) * cc - (Sr + Sl) - R(48) * U0[k]) * C.i8n2;          // b4
+        d[3][k] = (Dr - Dl) * C.i2nt;                                         // b6
+        d[4][k] = ((Sr + Sl) - R(2) * cc) * C.i2t2;                           // b5
       }
+      central(U, V, hq, d[0], x);
+      central(U, V, hq, d[1], y);
+      central(U, V, hq, d[2], xx);
+      central(U, V, hq, d[3], xy);
+      central(U, V, hq, d[4], yy);
     }
-    Moments<R, 8, 7> m;
-    moments(u0, v0, lam0, var0, C.K, 0, m);
-    Coefs<R> c;
-    coef_systems(ir0, solve_k(u0, v0, lam0, var0, C.N, C.iN), C.i2N, d, true, true, c);
-    Groups<R> g;
-    hydro_groups(c, tw.I, C.y2, g);
-    add_flux(g, m, r0, Fl);
-    if (C.prandtl) add_point(g, m, r0, Mn);
-    if (kin_point) {
-      hydro_groups(c, tw.E, C.y2, g);
-      add_point(g, m, r0, P0);
-    } else {
-      // e = exp(-dt/tau) = 0: the weight of the second-order groups at t = dt, -(dt^2 + 2 dt tau) e,
-      // is exactly 0
-      hydro_groups<false>(c, tw.E, C.y2, g);
-      add_point_first(g, m, r0, P0);
-    }
-    R Y1[4], Yu[4], Yv[4];
+    R A[4], tx[4], ty[4], tt[4], S[4], qx[4], qy[4];
+    const R px = pN * xx[3], pxy = pN * xy[3], pyy = pN * yy[3], pt = px + pyy;
+    const R dx = xx[1] + xy[2], dy = xy[1] + yy[2];
+    time_coef(U, V, pN, kc, x, y, A);  // <A + a1 u + a2 v> = 0
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      Y1[k] = tw.E[1] * c.a2[k] + tw.E[3] * c.Aty[k];
-      Yu[k] = tw.E[2] * c.Axy[k];
-      Yv[k] = tw.E[2] * c.Ayy[k];
+      qx[k] = U * xx[k] + V * xy[k];
+      qy[k] = U * xy[k] + V * yy[k];
     }
-    add_point_linear(Y1, Yu, Yv, m, r0, P1);
+    // <Axx u + Axy v + Atx> = 0, <Axy u + Ayy v + Aty> = 0
+    tx[0] = -(qx[0] + dx);
+    tx[1] = -(qx[1] + px);
+    tx[2] = -(qx[2] + pxy);
+    tx[3] = -(qx[3] + kc * dx);
+    ty[0] = -(qy[0] + dy);
+    ty[1] = -(qy[1] + pxy);
+    ty[2] = -(qy[2] + pyy);
+    ty[3] = -(qy[3] + kc * dy);
+    // <Atx u + Aty v + Att> = 0
+    const R qt0 = U * tx[0] + V * ty[0], qt1 = U * tx[1] + V * ty[1];
+    const R qt2 = U * tx[2] + V * ty[2], qt3 = U * tx[3] + V * ty[3], dt1 = tx[1] + ty[2];
+    tt[0] = -(qt0 + dt1);
+    tt[1] = -(qt1 + pN * tx[3]);
+    tt[2] = -(qt2 + pN * ty[3]);
+    tt[3] = -(qt3 + kc * dt1);
+    // S = <(Axx u^2 + 2 Axy u v + Ayy v^2) psi'>
+    const R gg = U * dx + V * dy, s1 = s * (R(3) * xx[1] + R(2) * xy[2] + yy[1]);
+    S[0] = (gg - qt0) + pt;
+    S[1] = (U * px + V * pxy - qt1) + s1;
+    S[2] = (U * pxy + V * pyy - qt2) + s * (xx[2] + R(2) * xy[1] + R(3) * yy[2]);
+    S[3] = kc * (gg + R(2) * pt - s * (xx[0] + yy[0])) - qt3;
+    // G0 = <psi' f> and G1 = <c psi' f>, time-integrated: the flux is U G0 + G1
+    const R y2h = R(0.5) * C.y2, h4 = R(0.5) * w.I4, h5 = R(0.5) * w.I5;
+    const R wA = w.I3 - w.I2, wyy = y2h * w.I1, wtt = h5 - w.I6, rI = r0 * w.I1;
+    R G0[4], f[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) G0[k] = wA * A[k] + wyy * yy[k] + wtt * tt[k] + h4 * S[k];
+    G0[0] += rI;
+    G0[3] += rI * (C.nh * s);
+    const R qa1 = U * x[1] + V * y[1], qa3 = U * x[3] + V * y[3];
+    const R b1 = w.I3 * A[1] + h5 * tt[1] + wyy * yy[1] + w.I2 * qa1 + w.I6 * qt1 + h4 * (U * qx[1] + V * qy[1]);
+    const R b3 = w.I3 * A[3] + h5 * tt[3] + wyy * yy[3] + w.I2 * qa3 + w.I6 * qt3 + h4 * (U * qx[3] + V * qy[3]);
+    const R c0 = w.I2 * x[0] + w.I6 * tx[0] + w.I4 * qx[0], c1 = w.I2 * x[1] + w.I6 * tx[1] + w.I4 * qx[1];
+    const R c2 = w.I2 * x[2] + w.I6 * tx[2] + w.I4 * qx[2], c3 = w.I2 * x[3] + w.I6 * tx[3] + w.I4 * qx[3];
+    const R d1 = w.I2 * y[1] + w.I6 * ty[1] + w.I4 * qy[1], d2 = w.I2 * y[2] + w.I6 * ty[2] + w.I4 * qy[2];
+    const R pB = pN * c3, z = h4 * s1, bz = b1 + pB;
+    f[0] = U * G0[0] + (bz + z);
+    f[1] = U * G0[1] + pN * b3 +
+           s * (rI + (R(3) * c1 + d2) + h4 * ((R(6) * px + R(2) * pyy) - s * (R(3) * xx[0] + yy[0])));
+    f[2] = U * G0[2] + s * ((c2 + d1) + w.I4 * (R(2) * pxy - s * xy[0]));
+    f[3] = U * G0[3] + kc * (bz + pB - s * c0) + C.n4h * s * z;
+    lab(U, V, hq, f, Fl);
+    if (C.prandtl) lab(U, V, hq, G0, Mn);
+    // values at t = dt: (1 - e) (U0 + dt U_t + ...), C_3 - C_2 = dt (1 - e),
+    // C_5 / 2 - C_6 = dt^2/2 + dt tau e, C_4 = -(dt^2 + 2 dt tau) e
+    const R pA = dt * w.om, pyw = y2h * w.om, te = tau * w.e, ptt = dt * (R(0.5) * dt + te);
+    const R pS = -dt * (R(0.5) * dt * w.e + te), rE = r0 * w.om;
+    R p[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) p[k] = pA * A[k] + pyw * yy[k] + ptt * tt[k] + pS * S[k];
+    p[0] += rE;
+    p[3] += rE * (C.nh * s);
+    lab(U, V, hq, p, P0);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) p[k] = w.om * y[k] + pA * ty[k];
+    lab(U, V, hq, p, P1);
   }
 
-  // ---- kinetic part, Eq. dis2, for both sides ----
+  // ---- kinetic part, Eq. dis2, for both sides: NS: f_G = g_k - tau (a u + A) g_k; Euler:
+  // f_G = g_k, the terms with tn are absent (not formed) ----
 #pragma unroll 1
   for (int side = 0; side < 2; ++side) {
     // selects, not indexing: a dynamic index would put these arrays in local memory
-    const R rho = side ? rs[1] : rs[0], U = side ? us[1] : us[0];
-    const R V = side ? vs[1] : vs[0], lam = side ? ls[1] : ls[0];
-    const R ir = side ? irs[1] : irs[0], var = side ? vrs[1] : vrs[0];
-    Coefs<R> c;
+    const R rho = side ? rs[1] : rs[0], U = side ? us[1] : us[0], V = side ? vs[1] : vs[0];
+    const R s = side ? vrs[1] : vrs[0], l2 = side ? l2s[1] : l2s[0];
+    R a1[4], a2[4], xx[4], xy[4], yy[4], A[4], tx[4], ty[4];
     {
-      R d[5][4];
-      {
-        FaceState<R> S;
-        src.side(side, S);
-#pragma unroll
-        for (int q = 0; q < 5; ++q)
-#pragma unroll
-          for (int k = 0; k < 4; ++k) d[q][k] = S.w[q + 1][k];
+      const R hq = R(0.5) * (U * U + V * V), hs = R(0.5) * (U * U + s), c5 = C.i2N * l2;
+      FaceState<R> S;
+      src.side(side, S);
+      R e1[4], e2[4], exx[4], exy[4], eyy[4];
+      central(U, V, hq, S.w[1], e1);
+      central(U, V, hq, S.w[2], e2);
+      central(U, V, hq, S.w[3], exx);
+      central(U, V, hq, S.w[4], exy);
+      central(U, V, hq, S.w[5], eyy);
+      half_coef(U, l2, c5, hs, e1, a1);
+      half_coef(U, l2, c5, hs, e2, a2);
+      half_coef(U, l2, c5, hs, exx, xx);
+      half_coef(U, l2, c5, hs, exy, xy);
+      half_coef(U, l2, c5, hs, eyy, yy);
+      if (ns) {
+        const R kc = C.n2h * s;
+        R t[4];
+        time_coef(U, V, C.i2N, kc, e1, e2, t);
+        half_coef(U, l2, c5, hs, t, A);
+        time_coef(U, V, C.i2N, kc, exx, exy, t);
+        half_coef(U, l2, c5, hs, t, tx);
+        time_coef(U, V, C.i2N, kc, exy, eyy, t);
+        half_coef(U, l2, c5, hs, t, ty);
       }
-      // the time coefficients of g_k (NS only)
-      coef_systems(ir, solve_k(U, V, lam, var, C.N, C.iN), C.i2N, d, ns, false, c);
     }
-    Moments<R, 8, 7> mh;
-    moments_from(U, V, var, C.K, side ? h0[1] : h0[0], side ? h1[1] : h1[0], mh);
-    Groups<R> g;
-    if (ns) kinetic_groups<true>(c, tw.I, C.y2, tn, g);
-    else kinetic_groups<false>(c, tw.I, C.y2, tn, g);
-    add_flux(g, mh, rho, Fl);
-    if (C.prandtl) add_point(g, mh, rho, Mn);
+    R m[8];
+    m[0] = side ? h0[1] : h0[0];
+    m[1] = side ? h1[1] : h1[0];
+#pragma unroll
+    for (int n = 2; n < 8; ++n) m[n] = U * m[n - 1] + (n == 2 ? s : R(n - 1) * s) * m[n - 2];
+
+    // P for the weights w7, w8 = -w9 and w10 of e^(-t/tau), -t e^(-t/tau) and t^2 e^(-t/tau):
+    // v = V + d takes the terms in v to V times themselves and d times themselves
+    auto poly = [&](R w7, R w9, R w10, HalfPoly<R>& P) {
+      R B1[4], Bu[4], Bd[4], wq = R(0.5) * w10, wu = -w9;
+      const R t7 = tn * w7, t8 = -tn * w9;
+      if (ns) {
+        wq -= t8;
+        wu -= t7;
+      }
+      const R wd = R(2) * wq * V, wyy = R(0.5) * C.y2 * w7 - wq * V * V;  // B1 takes V Bd, which holds wd yy
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        Bd[k] = wu * a2[k] + wd * yy[k];
+        Bu[k] = wu * a1[k] + wd * xy[k];
+        if (ns) {
+          Bd[k] = Bd[k] - t8 * ty[k];
+          Bu[k] = Bu[k] - t8 * tx[k];
+          B1[k] = V * Bd[k] + wyy * yy[k] - t7 * A[k];
+        } else {
+          B1[k] = V * Bd[k] + wyy * yy[k];
+        }
+      }
+      half_poly(w7 * rho, B1, Bu, Bd, wq, xx, xy, yy, s, C.n1h, P);
+    };
+    HalfPoly<R> P;
+    poly(w.i7, w.i9, w.i10, P);
+    half_moments<1, 4>(P, m, V, s, C.n1h, Fl);
+    if (C.prandtl) half_moments<0, 4>(P, m, V, s, C.n1h, Mn);
     // Every weight of the kinetic part at t = dt carries e = exp(-dt/tau), which underflows to
     // exactly 0 once tau is a small enough fraction of dt (smooth Euler flow): the point
     // values then get exactly nothing from this side
     if (kin_point) {
-      R Y1[4], Yu[4], Yv[4];
-      if (ns) {
-        kinetic_groups<true>(c, tw.E, C.y2, tn, g);
-        add_point(g, mh, rho, P0);
-        const R wy = -tn * tw.E[7] - tw.E[9];
+      const R e9 = dt * w.e;
+      poly(w.e, e9, dt * e9, P);
+      half_moments<0, 4>(P, m, V, s, C.n1h, P0);
+      // the part linear along the face: y (e (a2 - tau Aty) - (t + tau) e (Axy u + Ayy v))
+      const R wy = ns ? -tn * w.e - e9 : -e9, te = tn * w.e;
+      R B1[4], Bu[4], Bd[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          Y1[k] = tw.E[7] * (c.a2[k] - tn * c.Aty[k]);
-          Yu[k] = wy * c.Axy[k];
-          Yv[k] = wy * c.Ayy[k];
-        }
-      } else {
-        kinetic_groups<false>(c, tw.E, C.y2, tn, g);
-        add_point(g, mh, rho, P0);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          Y1[k] = tw.E[7] * c.a2[k];
-          Yu[k] = -tw.E[9] * c.Axy[k];
-          Yv[k] = -tw.E[9] * c.Ayy[k];
-        }
+      for (int k = 0; k < 4; ++k) {
+        Bd[k] = wy * yy[k];
+        Bu[k] = wy * xy[k];
+        B1[k] = w.e * a2[k] + V * Bd[k];
+        if (ns) B1[k] = B1[k] - te * ty[k];
       }
-      add_point_linear(Y1, Yu, Yv, mh, rho, P1);
+      half_poly_linear(B1, Bu, Bd, s, C.n1h, P);
+      half_moments<0, 3>(P, m, V, s, C.n1h, P1);
     }
   }
 
@@ -817,9 +697,8 @@ GKS_FN void face_evolution(const FaceConst<R>& C, const Src& src, R dt, R F[4], 
   // face-mean heat flux (1/2) int (u-U0)((u-U0)^2+(v-V0)^2+xi^2) f, written with the
   // flux and the time-integrated conservative moments.
   if (C.prandtl) {
-    const R q2 = u0 * u0 + v0 * v0;
-    const R q = Fl[3] - u0 * Fl[1] - v0 * Fl[2] + (R(0.5) * q2 + u0 * u0) * Fl[0] - u0 * Mn[3] +
-                u0 * v0 * Mn[2] - R(0.5) * u0 * q2 * Mn[0];
+    const R q = Fl[3] - u0 * Fl[1] - v0 * Fl[2] + (R(0.5) * q20 + u0 * u0) * Fl[0] - u0 * Mn[3] +
+                u0 * v0 * Mn[2] - R(0.5) * u0 * q20 * Mn[0];
     Fl[3] += C.pr_fix * q;
   }
   const R yg = R(0.28867513459481287) * C.dtan;  // sqrt(3)/6

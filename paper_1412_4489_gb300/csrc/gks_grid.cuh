@@ -8,6 +8,7 @@
 
 #include "../../include/gks.h"
 #include "gks_device.cuh"
+#include "gks_face_monomials.cuh"
 
 namespace gks {
 
@@ -694,8 +695,9 @@ __host__ __device__ inline FaceConst<R> grid_face_const(const Geo& g, int axis) 
 }
 
 // the evolution at face (i, j) of axis AX: flux F and new point values Wn
-// (NSM: Navier-Stokes 1, Euler 0, decided per grid at run time -1)
-template <int AX, class R, class TW, int NSM = -1>
+// (NSM: Navier-Stokes 1, Euler 0, decided per grid at run time -1; MONO: the routine in
+// velocity monomials, of FP32 batches)
+template <int AX, class R, class TW, int NSM = -1, bool MONO = false>
 __device__ __forceinline__ void flux_face(const Geo& g, const FaceConst<R>& C, const R* __restrict__ rec,
                                           TW* __restrict__ Wn, R* __restrict__ F, int i, int j, R dt) {
   const int nx = g.nx, ny = g.ny;
@@ -735,7 +737,8 @@ __device__ __forceinline__ void flux_face(const Geo& g, const FaceConst<R>& C, c
   src.first_order = false;
 
   R Fl[4], Wm[4], Wp[4];
-  face_evolution<R, NSM>(C, src, dt, Fl, Wm, Wp);
+  if constexpr (MONO) monomials::face_evolution<R, NSM>(C, src, dt, Fl, Wm, Wp);
+  else face_evolution<R, NSM>(C, src, dt, Fl, Wm, Wp);
   if (src.img_lo) wall_face_flux<R>(src.img_lo, src.uwt_lo, Fl);
   else if (src.img_hi) wall_face_flux<R>(src.img_hi, src.uwt_hi, Fl);
 
