@@ -7,6 +7,7 @@
 //              (block 0), and the compact reconstruction of every cell (Section 3.2)
 //   k_flux<0>  gas evolution at every x-face (Section 2.2, 3.3, 4)
 //   k_flux<1>  gas evolution at every y-face (frame rotated: n = y, t = x)
+//              (FP64: both axes in one launch, k_faces or k_faces_split)
 //   k_update   conservative update (Eq. finite) into FP64 averages, or in
 //              FP32-bulk mode into double-float (hi + lo FP32) averages, the
 //              ghost cells that are images of the updated cells, the next CFL
@@ -64,48 +65,66 @@ __global__ void k_ghost(Geo g, Cells<R> U0, Cells<R> U1, const Ctrl* c, int forc
 // begin = 1: block 0 also opens the step (ctrl_begin); the other blocks then do
 // not look at the skip flag it sets (coefficients of a skipped step go unused).
 // CHAR: reconstruction in characteristic variables.
-// resident 256-thread blocks per SM the reconstruction is compiled for: FP32 conservative 4
-// (64 registers; the kernel is latency-bound, so occupancy pays), FP64 characteristic 1
-// (it needs more than 128 registers), the others 2 (128)
+// block heights (of 32 cells) and resident blocks per SM the reconstruction is compiled for: FP32
+// conservative 8 and 4 (64 registers; the kernel is latency-bound, so occupancy pays), FP32
+// characteristic 8 and 2 (128); FP64 characteristic 1 and 8 (it needs more than 128, and one-warp blocks spread
+// over the SMs evenly)
+template <class R> struct ReconRows { static constexpr int value = 8; };
+template <> struct ReconRows<double> { static constexpr int value = 1; };
 template <class R, bool CHAR> struct ReconBlocks { static constexpr int value = 2; };
 template <> struct ReconBlocks<float, false> { static constexpr int value = 4; };
-template <> struct ReconBlocks<double, true> { static constexpr int value = 1; };
+template <> struct ReconBlocks<double, true> { static constexpr int value = 8; };
 
 template <class R, class TW, bool CHAR>
-__global__ void __launch_bounds__(256, ReconBlocks<R, CHAR>::value) k_recon(Geo g, const R* U0, const R* U1, const TW* Wx0, const TW* Wx1,
+__global__ void __launch_bounds__(32 * ReconRows<R>::value, ReconBlocks<R, CHAR>::value) k_recon(Geo g, const R* U0, const R* U1, const TW* Wx0, const TW* Wx1,
                                                const TW* Wy0, const TW* Wy1, R* __restrict__ rec, R dx, R dy,
                                                R weps, R wC, Ctrl* c, int force, int begin, double cfl,
                                                double dt_max, double t_end) {
   pdl_enter();
   if (begin) {
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0) ctrl_begin(c, cfl, dt_max, t_end);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0 && threadIdx.y == 0)
+      ctrl_begin(c, cfl, dt_max, t_end);
   } else if (!force && c->skip) {
     return;
   }
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
+  const int j = (sizeof(R) == 8 ? blockIdx.z * gridDim.y + blockIdx.y : blockIdx.y) * blockDim.y + threadIdx.y;
   if (i >= g.nx || j >= g.ny) return;
   const int par = (int)(c->steps & 1);
   recon_cell<R, TW, CHAR>(g, par ? U1 : U0, par ? Wx1 : Wx0, par ? Wy1 : Wy0, rec, i, j, dx, dy, weps, wC);
 }
 
+// FP64 in conservative variables: four lanes to a cell (recon_cell_lanes), eight cells to a one-warp block,
+// numbered through row by row
+__global__ void __launch_bounds__(32, 16) k_recon_lanes(Geo g, const double* U0, const double* U1, const double* Wx0,
+                                                        const double* Wx1, const double* Wy0, const double* Wy1,
+                                                        double* __restrict__ rec, Ctrl* c, int force, int begin,
+                                                        double cfl, double dt_max, double t_end) {
+  pdl_enter();
+  if (begin) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctrl_begin(c, cfl, dt_max, t_end);
+  } else if (!force && c->skip) {
+    return;
+  }
+  const unsigned long long n = (unsigned long long)g.nx * g.ny, k = (unsigned long long)blockIdx.x * 8 + (threadIdx.x >> 2);
+  const unsigned long long q = k < n ? k : n - 1;
+  const int j = (int)(q / (unsigned)g.nx), i = (int)(q - (unsigned long long)j * g.nx);
+  const int par = (int)(c->steps & 1);
+  recon_cell_lanes(g, par ? U1 : U0, par ? Wx1 : Wx0, par ? Wy1 : Wy0, rec, i, j, k < n);
+}
+
 // ---------------------------------------------------------------------------
 // face evolution
 // ---------------------------------------------------------------------------
-// resident 128-thread blocks per SM the face kernel is compiled for (register cap).
-// FP32: 4 blocks = 16 warps per SM at 128 registers (registers are allocated per SM
+// resident 128-thread blocks per SM the FP32 face kernel is compiled for (register cap): 4 blocks = 16 warps per SM at 128 registers (registers are allocated per SM
 // quarter, so more than 12 warps means at most 128); the Euler routine fits without
 // spilling, and the extra warps hide more of its latency than 3 blocks at 168 registers.
 #ifndef GKS_FLUX_MINB_F32
 #define GKS_FLUX_MINB_F32 4
 #endif
-template <class R> struct FluxBlocks;
-template <> struct FluxBlocks<double> { static constexpr int value = 1; };
-template <> struct FluxBlocks<float> { static constexpr int value = GKS_FLUX_MINB_F32; };
-
 // NS: Navier-Stokes (1) or Euler (0) face routine, chosen per grid by flux_kernel
 template <int AX, class R, class TW, int NS>
-__global__ void __launch_bounds__(128, FluxBlocks<R>::value) k_flux(Geo g, FaceConst<R> C, const R* __restrict__ rec,
+__global__ void __launch_bounds__(128, GKS_FLUX_MINB_F32) k_flux(Geo g, FaceConst<R> C, const R* __restrict__ rec,
                                                                     TW* Wn0, TW* Wn1, R* __restrict__ F,
                                                                     const Ctrl* c, int force) {
   pdl_enter();
@@ -130,6 +149,72 @@ template <int AX, class R, class TW>
 auto flux_kernel(const Geo& g) -> decltype(&k_flux<AX, R, TW, 1>) {
   return g.mu > 0.0 ? &k_flux<AX, R, TW, 1> : &k_flux<AX, R, TW, 0>;
 }
+
+// FP64: every face of the grid in one launch, 32 to a block, x-faces in blocks [0, nbx), y-faces after
+// them, numbered through row by row.  The FP64 pipe serves a warp instruction for a quarter of an SM in 64 cycles
+// whether its lanes are active or not, so what counts is full warps spread evenly over the quarters: one-warp
+// blocks without idle lanes at the rows' ends, and no second launch with a tail of its own.  (Instruction fetch,
+// which speaks against mixing the two axes' bodies in FP32, does not matter at this pace.)
+// first: the first block's number (a launch can take one axis alone).
+template <class R, class TW>
+struct FaceArgs {
+  FaceConst<R> Cx, Cy;
+  const R* rec;
+  TW *Wx0, *Wx1, *Wy0, *Wy1;
+  R *Fx, *Fy;
+  unsigned nbx, first;
+};
+
+template <int AX>
+__device__ __forceinline__ bool face_at(const Geo& g, unsigned block, int lane, int& i, int& j) {
+  const unsigned fx = AX == 0 ? g.nx + 1 : g.nx, fy = AX == 0 ? g.ny : g.ny + 1;
+  const unsigned long long f = (unsigned long long)block * 32 + lane, n = (unsigned long long)fx * fy;
+  const unsigned long long q = f < n ? f : n - 1;
+  j = (int)(q / fx);
+  i = (int)(q - (unsigned long long)j * fx);
+  return f < n;
+}
+
+template <class R, class TW, int NS>
+__global__ void __launch_bounds__(32, 8) k_faces(Geo g, FaceArgs<R, TW> a, const Ctrl* c, int force) {
+  pdl_enter();
+  if (!force && c->skip) return;
+  const unsigned b = blockIdx.x + a.first;
+  const int par = (int)(c->steps & 1);
+  const R dt = step_dt<R>(c);
+  int i, j;
+  if (b < a.nbx) {
+    if (face_at<0>(g, b, threadIdx.x, i, j))
+      flux_face<0, R, TW, NS>(g, a.Cx, a.rec, par ? a.Wx0 : a.Wx1, a.Fx, i, j, dt);
+  } else if (face_at<1>(g, b - a.nbx, threadIdx.x, i, j)) {
+    flux_face<1, R, TW, NS>(g, a.Cy, a.rec, par ? a.Wy0 : a.Wy1, a.Fy, i, j, dt);
+  }
+}
+
+// The same with three warps to 32 faces (flux_face_split): for grids whose face warps are too few to keep the
+// quarters of the SMs busy, where a face's serial time is the kernel's.
+template <class R, class TW, int NS>
+__global__ void __launch_bounds__(96, 2) k_faces_split(Geo g, FaceArgs<R, TW> a, const Ctrl* c, int force) {
+  __shared__ SplitShare<R> sh;
+  pdl_enter();
+  if (!force && c->skip) return;
+  const unsigned b = blockIdx.x + a.first;
+  const int par = (int)(c->steps & 1), lane = threadIdx.x & 31;
+  const R dt = step_dt<R>(c);
+  int i, j;
+  if (b < a.nbx) {
+    const bool active = face_at<0>(g, b, lane, i, j);
+    flux_face_split<0, R, TW, NS>(g, a.Cx, a.rec, par ? a.Wx0 : a.Wx1, a.Fx, i, j, active, dt, sh);
+  } else {
+    const bool active = face_at<1>(g, b - a.nbx, lane, i, j);
+    flux_face_split<1, R, TW, NS>(g, a.Cy, a.rec, par ? a.Wy0 : a.Wy1, a.Fy, i, j, active, dt, sh);
+  }
+}
+
+// Grids of at most kSplitWarps face warps per SM (both axes) take the split launch.  Step times, one warp / three
+// warps (us, Euler): 32^2 89 / 73, 64^2 (1.7 warps per SM) 90 / 80, 70^2 (2.0) 89 / 91, 100^2
+// 109 / 111; Navier-Stokes: 107 / 80, 107 / 91, 109 / 108, 140 / 149.
+constexpr unsigned kSplitWarps = 2;
 
 // ---------------------------------------------------------------------------
 // update, CFL bound of the new state, physical check
@@ -177,16 +262,21 @@ __global__ void __launch_bounds__(256, UpdateBlocks<R>::value) k_update(Geo g, C
   block_bound_to<R>(inv_max, &c->dtb[pass - 1]);
 }
 
-// launch grid of an update pass (32 x 8 tiles): pass 1 takes one wave of resident
+// launch grid of an update pass in tiles of 32 x rows cells: pass 1 takes one wave of resident
 // blocks (blocks_per_sm per SM), each walking ceil(tiles / wave) tiles along y, so
 // that the per-block work (control reads, the CFL reduction) is shared by its tiles;
-// the fallback passes at most 8 x (SMs / 2) blocks (usually no work)
-dim3 update_grid(const Geo& g, int pass, int sms, int blocks_per_sm) {
-  unsigned tx = (unsigned)((g.nx + 31) / 32), ty = (unsigned)((g.ny + 7) / 8);
+// the fallback passes at most 8 x (SMs / 2) blocks (usually no work).  Pass 1 of the FP64 form takes
+// one-warp blocks (rows = 1): its bound is the FP64 pipe, which wants the warps of a small grid spread over all SMs
+// (81^2 in 256-thread blocks keeps 33 of 152 SMs busy).
+constexpr int kUpdateRows = 8;
+template <class R> constexpr int update_rows(int pass) { return pass == 1 && sizeof(R) == 8 ? 1 : kUpdateRows; }
+
+dim3 update_grid(const Geo& g, int pass, int sms, int blocks_per_sm, int rows) {
+  unsigned tx = (unsigned)((g.nx + 31) / 32), ty = (unsigned)((g.ny + rows - 1) / rows);
   if (pass == 1 && sms > 0) {
-    const unsigned wave = (unsigned)sms * (unsigned)blocks_per_sm;
-    const unsigned rows = wave / tx > 0 ? wave / tx : 1;  // block rows that fit in one wave
-    const unsigned k = (ty + rows - 1) / rows;            // tiles per block
+    const unsigned wave = (unsigned)sms * (unsigned)(blocks_per_sm * (kUpdateRows / rows));
+    const unsigned fit = wave / tx > 0 ? wave / tx : 1;  // block rows that fit in one wave
+    const unsigned k = (ty + fit - 1) / fit;             // tiles per block
     ty = (ty + k - 1) / k;
   }
   if (pass > 1) {
@@ -366,7 +456,6 @@ cudaError_t launch(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block, cu
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
-// ev (optional, 10 events): recorded before each of the nine kernels and after the last
 template <class R>
 FaceConst<R> fconst(const Geo& g, int axis) {
   return grid_face_const<R>(g, axis);
@@ -383,14 +472,45 @@ void launch_ghost(gks_handle* h, int force) {
 }
 
 template <class R, class TW>
+cudaError_t launch_recon(bool pdl, cudaStream_t s, const Geo& g, const R* U0, const R* U1, const TW* Wx0, const TW* Wx1,
+                         const TW* Wy0, const TW* Wy1, R* rec, Ctrl* c, int force, int begin, double cfl, double dt_max,
+                         double t_end) {
+  if constexpr (sizeof(R) == 8) {
+    if (!g.characteristic)
+      return launch(pdl, k_recon_lanes, dim3((unsigned)(((unsigned long long)g.nx * g.ny + 7) / 8)), dim3(32), s, g, U0, U1,
+                    Wx0, Wx1, Wy0, Wy1, rec, c, force, begin, cfl, dt_max, t_end);
+    const dim3 b(32, ReconRows<R>::value);
+    // block rows beyond the grid's y limit continue in z
+    const unsigned rows = (unsigned)g.ny, gy = rows < 65535u ? rows : 65535u;
+    return launch(pdl, k_recon<R, TW, true>, dim3((unsigned)(g.nx + 31) / 32, gy, (rows + gy - 1) / gy), b, s, g, U0, U1, Wx0,
+                  Wx1, Wy0, Wy1, rec, R(g.dx), R(g.dy), R(g.weno_eps), R(g.weno_C), c, force, begin, cfl, dt_max, t_end);
+  } else {
+    const dim3 b(32, ReconRows<R>::value);
+    return launch(pdl, g.characteristic ? k_recon<R, TW, true> : k_recon<R, TW, false>, grid2(g.nx, g.ny, b), b, s, g, U0,
+                  U1, Wx0, Wx1, Wy0, Wy1, rec, R(g.dx), R(g.dy), R(g.weno_eps), R(g.weno_C), c, force, begin, cfl, dt_max,
+                  t_end);
+  }
+}
+
+template <class R, class TW>
 cudaError_t launch_recon(gks_handle* h, int force, int begin = 0, double cfl = 0, double dt_max = 0,
                          double t_end = 0, bool pdl = false) {
-  const Geo& g = h->g;
-  const dim3 b2(32, 8);
-  return launch(pdl, g.characteristic ? k_recon<R, TW, true> : k_recon<R, TW, false>, grid2(g.nx, g.ny, b2), b2,
-                h->stream, g, cells<R>(h, 0), cells<R>(h, 1),
-         (const TW*)h->Wx[0], (const TW*)h->Wx[1], (const TW*)h->Wy[0], (const TW*)h->Wy[1], (R*)h->rec, R(g.dx),
-         R(g.dy), R(g.weno_eps), R(g.weno_C), h->ctrl, force, begin, cfl, dt_max, t_end);
+  return launch_recon<R, TW>(pdl, h->stream, h->g, cells<R>(h, 0), cells<R>(h, 1), (const TW*)h->Wx[0], (const TW*)h->Wx[1],
+                             (const TW*)h->Wy[0], (const TW*)h->Wy[1], (R*)h->rec, h->ctrl, force, begin, cfl, dt_max, t_end);
+}
+
+// the FP64 face launch over both axes (axes 3) or one of them (1: x, 2: y)
+template <class R, class TW>
+cudaError_t launch_faces(bool pdl, cudaStream_t s, const Geo& g, int sms, const R* rec, TW* Wx0, TW* Wx1, TW* Wy0, TW* Wy1,
+                         R* Fx, R* Fy, const Ctrl* c, int force, int axes = 3) {
+  const unsigned nbx = (unsigned)(((unsigned long long)(g.nx + 1) * g.ny + 31) / 32);
+  const unsigned nby = (unsigned)(((unsigned long long)g.nx * (g.ny + 1) + 31) / 32);
+  const FaceArgs<R, TW> a{fconst<R>(g, 0), fconst<R>(g, 1), rec, Wx0, Wx1, Wy0, Wy1, Fx, Fy, nbx, axes == 2 ? nbx : 0};
+  const unsigned n = (axes & 1 ? nbx : 0) + (axes & 2 ? nby : 0);
+  const bool ns = g.mu > 0.0, split = (unsigned long long)nbx + nby <= (unsigned long long)kSplitWarps * sms;
+  if (split)
+    return launch(pdl, ns ? k_faces_split<R, TW, 1> : k_faces_split<R, TW, 0>, dim3(n), dim3(96), s, g, a, c, force);
+  return launch(pdl, ns ? k_faces<R, TW, 1> : k_faces<R, TW, 0>, dim3(n), dim3(32), s, g, a, c, force);
 }
 
 // ev (optional, kLaunchesPerStep + 1 events): recorded before each kernel and after the last.
@@ -415,32 +535,44 @@ gks_status launch_step_kernels(gks_handle* h, double cfl, double dt_max, double 
   mark(0);
   if (do_recon) keep(launch_recon<R, TW>(h, force, with_begin_end ? 1 : 0, cfl, dt_max, t_end, pdl));
   mark(1);
-  const dim3 b2(32, 8), bf(32, 4);
-  // the x- and y-face evolutions are independent: without per-kernel timing the y-faces run
-  // on a side stream (fork after the reconstruction, join before the update), so that each
-  // fills the other's tail wave
-  const bool fork = ev == nullptr;
-  if (fork) {
-    keep(cudaEventRecord(h->fork, s));
-    keep(cudaStreamWaitEvent(h->side, h->fork, 0));
-    keep(launch(false, flux_kernel<1, R, TW>(g), grid2(g.nx, g.ny + 1, bf), bf, h->side, g, fconst<R>(g, 1),
-                (const R*)h->rec, (TW*)h->Wy[0], (TW*)h->Wy[1], (R*)h->Fy, (const Ctrl*)h->ctrl, force));
-    keep(cudaEventRecord(h->join, h->side));
-  }
-  keep(launch(pdl, flux_kernel<0, R, TW>(g), grid2(g.nx + 1, g.ny, bf), bf, s, g, fconst<R>(g, 0), (const R*)h->rec,
-              (TW*)h->Wx[0], (TW*)h->Wx[1], (R*)h->Fx, (const Ctrl*)h->ctrl, force));
-  mark(2);
-  if (fork) {
-    keep(cudaStreamWaitEvent(s, h->join, 0));
+  const dim3 bf(32, 4);
+  bool fork = false;
+  if constexpr (sizeof(R) == 8) {
+    auto faces = [&](int axes) {
+      keep(launch_faces<R, TW>(pdl, s, g, h->sms, (const R*)h->rec, (TW*)h->Wx[0], (TW*)h->Wx[1], (TW*)h->Wy[0],
+                               (TW*)h->Wy[1], (R*)h->Fx, (R*)h->Fy, (const Ctrl*)h->ctrl, force, axes));
+    };
+    if (ev) faces(1);
+    mark(2);
+    faces(ev ? 2 : 3);
   } else {
-    keep(launch(pdl, flux_kernel<1, R, TW>(g), grid2(g.nx, g.ny + 1, bf), bf, s, g, fconst<R>(g, 1),
-                (const R*)h->rec, (TW*)h->Wy[0], (TW*)h->Wy[1], (R*)h->Fy, (const Ctrl*)h->ctrl, force));
+    // the x- and y-face evolutions are independent: without per-kernel timing the y-faces run
+    // on a side stream (fork after the reconstruction, join before the update), so that each
+    // fills the other's tail wave
+    fork = ev == nullptr;
+    if (fork) {
+      keep(cudaEventRecord(h->fork, s));
+      keep(cudaStreamWaitEvent(h->side, h->fork, 0));
+      keep(launch(false, flux_kernel<1, R, TW>(g), grid2(g.nx, g.ny + 1, bf), bf, h->side, g, fconst<R>(g, 1),
+                  (const R*)h->rec, (TW*)h->Wy[0], (TW*)h->Wy[1], (R*)h->Fy, (const Ctrl*)h->ctrl, force));
+      keep(cudaEventRecord(h->join, h->side));
+    }
+    keep(launch(pdl, flux_kernel<0, R, TW>(g), grid2(g.nx + 1, g.ny, bf), bf, s, g, fconst<R>(g, 0), (const R*)h->rec,
+                (TW*)h->Wx[0], (TW*)h->Wx[1], (R*)h->Fx, (const Ctrl*)h->ctrl, force));
+    mark(2);
+    if (fork) {
+      keep(cudaStreamWaitEvent(s, h->join, 0));
+    } else {
+      keep(launch(pdl, flux_kernel<1, R, TW>(g), grid2(g.nx, g.ny + 1, bf), bf, s, g, fconst<R>(g, 1),
+                  (const R*)h->rec, (TW*)h->Wy[0], (TW*)h->Wy[1], (R*)h->Fy, (const Ctrl*)h->ctrl, force));
+    }
   }
   mark(3);
   for (int pass = 1; pass <= 3; ++pass) {
     if (do_update)
       // pass 1 follows the join (two predecessors): an ordinary launch
-      keep(launch(pdl && !(fork && pass == 1), k_update<R, TW>, update_grid(g, pass, h->sms, UpdateBlocks<R>::value), b2, s, g,
+      keep(launch(pdl && !(fork && pass == 1), k_update<R, TW>, update_grid(g, pass, h->sms, UpdateBlocks<R>::value, update_rows<R>(pass)),
+                  dim3(32, update_rows<R>(pass)), s, g,
                   cellbuf<R>(h, 0), cellbuf<R>(h, 1),
                   (const R*)h->Fx, (const R*)h->Fy, (TW*)h->Wx[0], (TW*)h->Wx[1], (TW*)h->Wy[0], (TW*)h->Wy[1],
                   h->bad, h->ctrl, pass));
@@ -857,8 +989,7 @@ gks_status gks_profile_step(gks_handle* h, double CFL, float* ms) {
 }
 
 int gks_launches_per_step(const gks_handle* h) {
-  (void)h;
-  return kLaunchesPerStep;
+  return h && h->prec == GKS_FP64 ? kLaunchesPerStep - 1 : kLaunchesPerStep;  // FP64: both face axes in one
 }
 
 gks_status gks_debug_recon(gks_handle* h, double* coef) {
@@ -1105,6 +1236,9 @@ extern "C" gks_status gks_step_noalloc(int nx, int ny, double Lx, double Ly, dou
   int device = 0;
   cudaError_t e = cudaGetDevice(&device);
   if (e != cudaSuccess) { g_create_err = std::string("cudaGetDevice: ") + cudaGetErrorString(e); return GKS_ECUDA; }
+  int sms = 0;
+  e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+  if (e != cudaSuccess) { g_create_err = std::string("cudaDeviceGetAttribute: ") + cudaGetErrorString(e); return GKS_ECUDA; }
   unsigned char* base = (unsigned char*)noalloc_base(device, why);
   if (!base) { g_create_err = "gks_step_noalloc: " + why; return GKS_ECUDA; }
   Ctrl* ctrl = (Ctrl*)base;
@@ -1115,7 +1249,7 @@ extern "C" gks_status gks_step_noalloc(int nx, int ny, double Lx, double Ly, dou
   double* Fy = (double*)(base + b_ctrl + 2 * b_u + b_rec + b_fx);
   unsigned char* bad = base + b_ctrl + 2 * b_u + b_rec + b_fx + b_fy;
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  const dim3 b2(32, 8), bf(32, 4);
+  const dim3 b2(32, 8);
   const int per = perimeter(g);
   const Cells<double> C0{U0}, C1{U1};
   // the control block must start from zero state; the rest is fully written before it is read
@@ -1123,16 +1257,14 @@ extern "C" gks_status gks_step_noalloc(int nx, int ny, double Lx, double Ly, dou
   k_scatter_U<double><<<grid2(nx, ny, b2), b2, 0, s>>>(g, dU, C0, C1, ctrl, 1);
   k_ghost<double><<<(per + 127) / 128, 128, 0, s>>>(g, C0, C1, ctrl, 1);
   k_dtbound<double><<<grid2(nx, ny, b2), b2, 0, s>>>(g, C0, C1, ctrl);
-  (g.characteristic ? k_recon<double, double, true> : k_recon<double, double, false>)<<<grid2(nx, ny, b2), b2, 0, s>>>(
-      g, U0, U1, dWx, dWx_out, dWy, dWy_out, rec, g.dx, g.dy,
-                                                            g.weno_eps, g.weno_C, ctrl, 0, 1, CFL,
-                                                            dt_max, INFINITY);
-  flux_kernel<0, double, double>(g)<<<grid2(nx + 1, ny, bf), bf, 0, s>>>(g, fconst<double>(g, 0), rec,
-                                                                  const_cast<double*>(dWx), dWx_out, Fx, ctrl, 0);
-  flux_kernel<1, double, double>(g)<<<grid2(nx, ny + 1, bf), bf, 0, s>>>(g, fconst<double>(g, 1), rec,
-                                                                  const_cast<double*>(dWy), dWy_out, Fy, ctrl, 0);
+  e = launch_recon<double, double>(false, s, g, U0, U1, dWx, dWx_out, dWy, dWy_out, rec, ctrl, 0, 1, CFL, dt_max, INFINITY);
+  if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
+  e = launch_faces<double, double>(false, s, g, sms, rec, const_cast<double*>(dWx), dWx_out, const_cast<double*>(dWy),
+                                   dWy_out, Fx, Fy, ctrl, 0);
+  if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
   for (int pass = 1; pass <= 3; ++pass)
-    k_update<double, double><<<update_grid(g, pass, 0, UpdateBlocks<double>::value), b2, 0, s>>>(g, C0, C1, Fx, Fy, const_cast<double*>(dWx), dWx_out,
+    k_update<double, double><<<update_grid(g, pass, sms, UpdateBlocks<double>::value, update_rows<double>(pass)),
+                               dim3(32, update_rows<double>(pass)), 0, s>>>(g, C0, C1, Fx, Fy, const_cast<double*>(dWx), dWx_out,
                                                               const_cast<double*>(dWy), dWy_out, bad, ctrl, pass);
   k_end<<<1, 1, 0, s>>>(ctrl);
   k_scatter_U<double><<<grid2(nx, ny, b2), b2, 0, s>>>(g, dU_out, C0, C1, ctrl, 0);

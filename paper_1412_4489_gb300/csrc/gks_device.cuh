@@ -12,6 +12,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "gks_half_normal.cuh"
+
 #ifndef GKS_FN
 #define GKS_FN __host__ __device__ __forceinline__
 #endif
@@ -55,6 +57,8 @@ __device__ __forceinline__ float d_rsqrt(float x) { return rsqrtf(x); }
 // 2 ulps for divisors below 2^126), far inside the FP32 path's error budget
 __device__ __forceinline__ double d_div(double a, double b) { return a / b; }
 __device__ __forceinline__ float d_div(float a, float b) { return __fdividef(a, b); }
+__device__ __forceinline__ double d_rcp(double a) { return 1.0 / a; }
+__device__ __forceinline__ float d_rcp(float a) { return __fdividef(1.0f, a); }
 
 template <class R> GKS_FN R sq(R a) { return a * a; }
 
@@ -79,6 +83,13 @@ GKS_FN void half_start(R U, R l2, int kind, R& h, R& g) {
   // boundary term of the integration by parts at u = 0
   const R b = d_exp(-lam * U * U) * R(0.28209479177387814) * rs;  // 1/(2 sqrt(pi lam))
   g = U * h + R(kind) * b;
+}
+__device__ __forceinline__ void half_start(double U, double l2, int kind, double& h, double& g) {
+  const double lam = 0.5 * l2, rs = rsqrt(lam), a = kind * (lam * rs) * U;
+  double t, e;
+  half_normal(fabs(a), t, e);
+  h = a > 0.0 ? 1.0 - t : t;
+  g = U * h + kind * (e * (0.28209479177387814 * rs));
 }
 
 // moments over u > 0 (kind +1) or u < 0 (kind -1); var = 1/(2 lam) = p/rho, formed once per
@@ -117,7 +128,7 @@ template <class R>
 struct TimeW {
   R I1, I2, I3, I4, I5, I6;  // integrals of C_1..C_6
   R i7, i9, i10;             // integrals of e^(-t/tau) (C_7), t e^(-t/tau) (-C_8), t^2 e^(-t/tau)
-  R e, om;                   // exp(-x), 1 - exp(-x)
+  R e, om, te;               // exp(-x), 1 - exp(-x), tau exp(-x)
 };
 
 // Coefficients of x^k, k = n - 3, in the sums over n >= 3 of t_n = (-x)^n / n!, of (n-2) t_n and
@@ -142,7 +153,7 @@ GKS_FN R series_sum(R x) {
 
 template <class R>
 GKS_FN void time_weights(R T, R tau, TimeW<R>& w) {
-  const R x = tau > R(0) ? d_div(T, tau) : R(INFINITY);
+  const R x = tau > R(0) ? T * d_rcp(tau) : R(INFINITY);
   const R t2 = tau * tau, T2h = R(0.5) * T * T;
   if (x < Prec<R>::series_below) {
     // with g = sum t_n, a = sum (n-2) t_n, b = sum (n-1)(n-2) t_n over n >= 3:
@@ -171,6 +182,7 @@ GKS_FN void time_weights(R T, R tau, TimeW<R>& w) {
     w.i9 = t2 - tau * (tau + T) * w.e;
     w.i10 = tau * (R(2) * t2 - R(2) * (T2h + T * tau + t2) * w.e);
   }
+  w.te = tau * w.e;
   w.I4 = -(w.i10 + R(2) * tau * w.i9);
   w.I5 = R(2) * T2h * (R(1.0 / 3.0) * T - tau);
   w.I6 = -tau * (T2h + w.i9);
@@ -307,6 +319,29 @@ GKS_FN void prim(const R w[4], R gm1, R& rho, R& ir, R& U, R& V, R& p) {
   U = w[1] * ir;
   V = w[2] * ir;
   p = gm1 * (w[3] - R(0.5) * (w[1] * U + w[2] * V));
+}
+
+// the same with 2 lam = rho / p and 1 / (2 lam).  FP64: both quotients from one reciprocal (a
+// reciprocal takes 5.4 FP64 instructions, a quotient 8.6); FP32: a reciprocal is one instruction, and the
+// product rho p would leave FP32's range earlier than rho and p do.
+template <class R>
+GKS_FN void prim_lam(const R w[4], R gm1, R& rho, R& U, R& V, R& p, R& l2, R& var) {
+  R ir;
+  if constexpr (sizeof(R) == 8) {
+    rho = w[0];
+    const R rp = gm1 * (rho * w[3] - R(0.5) * (w[1] * w[1] + w[2] * w[2]));  // rho p
+    const R t = d_rcp(rho * rp);
+    ir = t * rp;
+    U = w[1] * ir;
+    V = w[2] * ir;
+    p = rp * ir;
+    l2 = rho * rho * (rho * t);
+    var = p * ir;
+  } else {
+    prim(w, gm1, rho, ir, U, V, p);
+    l2 = d_div(rho, p);
+    var = p * ir;
+  }
 }
 
 struct FaceParams {
@@ -448,6 +483,242 @@ GKS_FN void wall_image(int kind, R gamma, R uwt, R Tw, const FaceState<R>& in, F
   out.w[5][3] += hess(in.w[2], in.w[2]);
 }
 
+// One side of the face: its value as a Maxwellian (s = 1 / (2 lam) = p / rho, l2 = 2 lam) and the
+// half-space <u^0>, <u^1>
+template <class R>
+struct SideData {
+  R rho, U, V, s, l2, p, h, g;
+};
+
+// the side's Maxwellian from its value w (side 0: u > 0, side 1: u < 0) and its share of
+// Eq. compatibility2, U0 += rho <psi>
+template <class R>
+GKS_FN void side_start(const FaceConst<R>& C, const R w[4], int side, SideData<R>& d, R U0[4]) {
+  prim_lam(w, C.gm1, d.rho, d.U, d.V, d.p, d.l2, d.s);
+  half_start(d.U, d.l2, side == 0 ? +1 : -1, d.h, d.g);
+  const R m2 = d.U * d.g + d.s * d.h;
+  U0[0] += d.rho * d.h;
+  U0[1] += d.rho * d.g;
+  U0[2] += d.rho * (d.V * d.h);
+  U0[3] += d.rho * (R(0.5) * m2 + (R(0.5) * d.V * d.V + C.n1h * d.s) * d.h);
+}
+
+// Section 4: collision time, from the pressures of the two sides and of g0
+template <class R>
+GKS_FN R collision_time(const FaceConst<R>& C, bool ns, R pl, R pr, R p0, R dt) {
+  const R jump = fabs((pl - pr) * d_rcp(pl + pr)) * dt;
+  return ns ? C.mu * d_rcp(p0) + jump : C.tau_eps * dt + C.tau_C * jump;
+}
+
+// Equilibrium part, Eq. dis1, with g0 and the polynomial of Section 3.3.  All moments of g0 run over the
+// whole velocity space: in its frame they are closed forms in the central components of the
+// derivatives.  The compatibility conditions turn the moments of a1 u + a2 v into those of A,
+// and so on, so that the point value is U0 and its time derivatives.  (r0, u0, v0, var0): g0's
+// density, velocity and 1 / (2 lam).
+template <class R, class Src>
+GKS_FN void equilibrium_part(const FaceConst<R>& C, const Src& src, const R U0[4], R r0, R u0, R v0, R var0,
+                             const TimeW<R>& w, R dt, R Fl[4], R P0[4], R P1[4], R Mn[4]) {
+  const R U = u0, V = v0, s = var0, hq = R(0.5) * (u0 * u0 + v0 * v0), pN = C.i2N, kc = C.n2h * var0;
+  R x[4], y[4], xx[4], xy[4], yy[4];
+  {
+    R avg[2][3][4], d[5][4];
+    src.avg(avg);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const R um = avg[0][0][k], uc = avg[0][1][k], up = avg[0][2][k];
+      const R wm = avg[1][0][k], wc = avg[1][1][k], wp = avg[1][2][k];
+      const R Sr = wp + wm, Sl = up + um, Dr = wp - wm, Dl = up - um, cc = wc + uc;
+      d[0][k] = ((Sr - Sl) + R(2) * (wc - uc)) * C.i4n;                     // b2
+      d[1][k] = (Dr + Dl) * C.i4t;                                          // b3
+      d[2][k] = (R(26) * cc - (Sr + Sl) - R(48) * U0[k]) * C.i8n2;          // b4
+      d[3][k] = (Dr - Dl) * C.i2nt;                                         // b6
+      d[4][k] = ((Sr + Sl) - R(2) * cc) * C.i2t2;                           // b5
+    }
+    central(U, V, hq, d[0], x);
+    central(U, V, hq, d[1], y);
+    central(U, V, hq, d[2], xx);
+    central(U, V, hq, d[3], xy);
+    central(U, V, hq, d[4], yy);
+  }
+  R A[4], tx[4], ty[4], tt[4], S[4], qx[4], qy[4];
+  const R px = pN * xx[3], pxy = pN * xy[3], pyy = pN * yy[3], pt = px + pyy;
+  const R dx = xx[1] + xy[2], dy = xy[1] + yy[2];
+  time_coef(U, V, pN, kc, x, y, A);  // <A + a1 u + a2 v> = 0
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    qx[k] = U * xx[k] + V * xy[k];
+    qy[k] = U * xy[k] + V * yy[k];
+  }
+  // <Axx u + Axy v + Atx> = 0, <Axy u + Ayy v + Aty> = 0
+  tx[0] = -(qx[0] + dx);
+  tx[1] = -(qx[1] + px);
+  tx[2] = -(qx[2] + pxy);
+  tx[3] = -(qx[3] + kc * dx);
+  ty[0] = -(qy[0] + dy);
+  ty[1] = -(qy[1] + pxy);
+  ty[2] = -(qy[2] + pyy);
+  ty[3] = -(qy[3] + kc * dy);
+  // <Atx u + Aty v + Att> = 0
+  const R qt0 = U * tx[0] + V * ty[0], qt1 = U * tx[1] + V * ty[1];
+  const R qt2 = U * tx[2] + V * ty[2], qt3 = U * tx[3] + V * ty[3], dt1 = tx[1] + ty[2];
+  tt[0] = -(qt0 + dt1);
+  tt[1] = -(qt1 + pN * tx[3]);
+  tt[2] = -(qt2 + pN * ty[3]);
+  tt[3] = -(qt3 + kc * dt1);
+  // S = <(Axx u^2 + 2 Axy u v + Ayy v^2) psi'>
+  const R gg = U * dx + V * dy, s1 = s * (R(3) * xx[1] + R(2) * xy[2] + yy[1]);
+  S[0] = (gg - qt0) + pt;
+  S[1] = (U * px + V * pxy - qt1) + s1;
+  S[2] = (U * pxy + V * pyy - qt2) + s * (xx[2] + R(2) * xy[1] + R(3) * yy[2]);
+  S[3] = kc * (gg + R(2) * pt - s * (xx[0] + yy[0])) - qt3;
+  // G0 = <psi' f> and G1 = <c psi' f>, time-integrated: the flux is U G0 + G1
+  const R y2h = R(0.5) * C.y2, h4 = R(0.5) * w.I4, h5 = R(0.5) * w.I5;
+  const R wA = w.I3 - w.I2, wyy = y2h * w.I1, wtt = h5 - w.I6, rI = r0 * w.I1;
+  R G0[4], f[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) G0[k] = wA * A[k] + wyy * yy[k] + wtt * tt[k] + h4 * S[k];
+  G0[0] += rI;
+  G0[3] += rI * (C.nh * s);
+  const R qa1 = U * x[1] + V * y[1], qa3 = U * x[3] + V * y[3];
+  const R b1 = w.I3 * A[1] + h5 * tt[1] + wyy * yy[1] + w.I2 * qa1 + w.I6 * qt1 + h4 * (U * qx[1] + V * qy[1]);
+  const R b3 = w.I3 * A[3] + h5 * tt[3] + wyy * yy[3] + w.I2 * qa3 + w.I6 * qt3 + h4 * (U * qx[3] + V * qy[3]);
+  const R c0 = w.I2 * x[0] + w.I6 * tx[0] + w.I4 * qx[0], c1 = w.I2 * x[1] + w.I6 * tx[1] + w.I4 * qx[1];
+  const R c2 = w.I2 * x[2] + w.I6 * tx[2] + w.I4 * qx[2], c3 = w.I2 * x[3] + w.I6 * tx[3] + w.I4 * qx[3];
+  const R d1 = w.I2 * y[1] + w.I6 * ty[1] + w.I4 * qy[1], d2 = w.I2 * y[2] + w.I6 * ty[2] + w.I4 * qy[2];
+  const R pB = pN * c3, z = h4 * s1, bz = b1 + pB;
+  f[0] = U * G0[0] + (bz + z);
+  f[1] = U * G0[1] + pN * b3 +
+         s * (rI + (R(3) * c1 + d2) + h4 * ((R(6) * px + R(2) * pyy) - s * (R(3) * xx[0] + yy[0])));
+  f[2] = U * G0[2] + s * ((c2 + d1) + w.I4 * (R(2) * pxy - s * xy[0]));
+  f[3] = U * G0[3] + kc * (bz + pB - s * c0) + C.n4h * s * z;
+  lab(U, V, hq, f, Fl);
+  if (C.prandtl) lab(U, V, hq, G0, Mn);
+  // values at t = dt: (1 - e) (U0 + dt U_t + ...), C_3 - C_2 = dt (1 - e),
+  // C_5 / 2 - C_6 = dt^2/2 + dt tau e, C_4 = -(dt^2 + 2 dt tau) e
+  const R pA = dt * w.om, pyw = y2h * w.om, te = w.te, ptt = dt * (R(0.5) * dt + te);
+  const R pS = -dt * (R(0.5) * dt * w.e + te), rE = r0 * w.om;
+  R p[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) p[k] = pA * A[k] + pyw * yy[k] + ptt * tt[k] + pS * S[k];
+  p[0] += rE;
+  p[3] += rE * (C.nh * s);
+  lab(U, V, hq, p, P0);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) p[k] = w.om * y[k] + pA * ty[k];
+  lab(U, V, hq, p, P1);
+}
+
+// Kinetic part, Eq. dis2, of one side, added to Fl, P0, P1 and Mn: NS: f_G = g_k - tau (a u + A) g_k;
+// Euler: f_G = g_k, the terms with tn are absent (not formed).  kin_point: e > 0.
+template <class R, class Src>
+GKS_FN void kinetic_part(const FaceConst<R>& C, const Src& src, int side, const SideData<R>& sd, bool ns, bool kin_point,
+                         const TimeW<R>& w, R tn, R dt, R Fl[4], R P0[4], R P1[4], R Mn[4]) {
+  const R rho = sd.rho, U = sd.U, V = sd.V, s = sd.s, l2 = sd.l2;
+  R a1[4], a2[4], xx[4], xy[4], yy[4], A[4], tx[4], ty[4];
+  {
+    const R hq = R(0.5) * (U * U + V * V), hs = R(0.5) * (U * U + s), c5 = C.i2N * l2;
+    FaceState<R> S;
+    src.side(side, S);
+    R e1[4], e2[4], exx[4], exy[4], eyy[4];
+    central(U, V, hq, S.w[1], e1);
+    central(U, V, hq, S.w[2], e2);
+    central(U, V, hq, S.w[3], exx);
+    central(U, V, hq, S.w[4], exy);
+    central(U, V, hq, S.w[5], eyy);
+    half_coef(U, l2, c5, hs, e1, a1);
+    half_coef(U, l2, c5, hs, e2, a2);
+    half_coef(U, l2, c5, hs, exx, xx);
+    half_coef(U, l2, c5, hs, exy, xy);
+    half_coef(U, l2, c5, hs, eyy, yy);
+    if (ns) {
+      const R kc = C.n2h * s;
+      R t[4];
+      time_coef(U, V, C.i2N, kc, e1, e2, t);
+      half_coef(U, l2, c5, hs, t, A);
+      time_coef(U, V, C.i2N, kc, exx, exy, t);
+      half_coef(U, l2, c5, hs, t, tx);
+      time_coef(U, V, C.i2N, kc, exy, eyy, t);
+      half_coef(U, l2, c5, hs, t, ty);
+    }
+  }
+  R m[8];
+  m[0] = sd.h;
+  m[1] = sd.g;
+#pragma unroll
+  for (int n = 2; n < 8; ++n) m[n] = U * m[n - 1] + (n == 2 ? s : R(n - 1) * s) * m[n - 2];
+
+  // P for the weights w7, w8 = -w9 and w10 of e^(-t/tau), -t e^(-t/tau) and t^2 e^(-t/tau):
+  // v = V + d takes the terms in v to V times themselves and d times themselves
+  auto poly = [&](R w7, R w9, R w10, HalfPoly<R>& P) {
+    R B1[4], Bu[4], Bd[4], wq = R(0.5) * w10, wu = -w9;
+    const R t7 = tn * w7, t8 = -tn * w9;
+    if (ns) {
+      wq -= t8;
+      wu -= t7;
+    }
+    const R wd = R(2) * wq * V, wyy = R(0.5) * C.y2 * w7 - wq * V * V;  // B1 takes V Bd, which holds wd yy
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      Bd[k] = wu * a2[k] + wd * yy[k];
+      Bu[k] = wu * a1[k] + wd * xy[k];
+      if (ns) {
+        Bd[k] = Bd[k] - t8 * ty[k];
+        Bu[k] = Bu[k] - t8 * tx[k];
+        B1[k] = V * Bd[k] + wyy * yy[k] - t7 * A[k];
+      } else {
+        B1[k] = V * Bd[k] + wyy * yy[k];
+      }
+    }
+    half_poly(w7 * rho, B1, Bu, Bd, wq, xx, xy, yy, s, C.n1h, P);
+  };
+  HalfPoly<R> P;
+  poly(w.i7, w.i9, w.i10, P);
+  half_moments<1, 4>(P, m, V, s, C.n1h, Fl);
+  if (C.prandtl) half_moments<0, 4>(P, m, V, s, C.n1h, Mn);
+  // Every weight of the kinetic part at t = dt carries e = exp(-dt/tau), which underflows to
+  // exactly 0 once tau is a small enough fraction of dt (smooth Euler flow): the point
+  // values then get exactly nothing from this side
+  if (kin_point) {
+    const R e9 = dt * w.e;
+    poly(w.e, e9, dt * e9, P);
+    half_moments<0, 4>(P, m, V, s, C.n1h, P0);
+    // the part linear along the face: y (e (a2 - tau Aty) - (t + tau) e (Axy u + Ayy v))
+    const R wy = ns ? -tn * w.e - e9 : -e9, te = tn * w.e;
+    R B1[4], Bu[4], Bd[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      Bd[k] = wy * yy[k];
+      Bu[k] = wy * xy[k];
+      B1[k] = w.e * a2[k] + V * Bd[k];
+      if (ns) B1[k] = B1[k] - te * ty[k];
+    }
+    half_poly_linear(B1, Bu, Bd, s, C.n1h, P);
+    half_moments<0, 3>(P, m, V, s, C.n1h, P1);
+  }
+}
+
+// the Prandtl-number fix, and the face's results from the accumulated moments
+template <class R>
+GKS_FN void finish_face(const FaceConst<R>& C, R u0, R v0, R Fl[4], const R P0[4], const R P1[4], const R Mn[4], R F[4],
+                        R Wm[4], R Wp[4]) {
+  // Prandtl-number fix: energy flux += (1/Pr - 1) q, q the time-integrated
+  // face-mean heat flux (1/2) int (u-U0)((u-U0)^2+(v-V0)^2+xi^2) f, written with the
+  // flux and the time-integrated conservative moments.
+  if (C.prandtl) {
+    const R q20 = u0 * u0 + v0 * v0;
+    const R q = Fl[3] - u0 * Fl[1] - v0 * Fl[2] + (R(0.5) * q20 + u0 * u0) * Fl[0] - u0 * Mn[3] +
+                u0 * v0 * Mn[2] - R(0.5) * u0 * q20 * Mn[0];
+    Fl[3] += C.pr_fix * q;
+  }
+  const R yg = R(0.28867513459481287) * C.dtan;  // sqrt(3)/6
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    F[k] = Fl[k];
+    Wm[k] = P0[k] - yg * P1[k];
+    Wp[k] = P0[k] + yg * P1[k];
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Section 2.2 at one face centre.  The two sides (value and derivatives in the
 // face frame) and the six cell averages of Section 3.3 (avg[m][k], m = 0 left,
@@ -471,243 +742,33 @@ GKS_FN void wall_image(int kind, R gamma, R uwt, R Tw, const FaceState<R>& in, F
 template <class R, int NSM = -1, class Src>
 GKS_FN void face_evolution(const FaceConst<R>& C, const Src& src, R dt, R F[4], R Wm[4], R Wp[4]) {
   const bool ns = NSM < 0 ? C.ns : NSM == 1;
-  // per side: rho, U, V, 1 / (2 lam) = p / rho, 2 lam, p, and the half-space <u^0>, <u^1>
-  R rs[2], us[2], vs[2], vrs[2], l2s[2], ps[2], h0[2], h1[2];
+  SideData<R> sd[2];
   R U0[4] = {R(0), R(0), R(0), R(0)};
-  // Eq. compatibility2: U0 = rho_l <psi>_{u>0} + rho_r <psi>_{u<0}
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     FaceState<R> S;
     src.side(k, S);
-    R ir;
-    prim(S.w[0], C.gm1, rs[k], ir, us[k], vs[k], ps[k]);
-    l2s[k] = d_div(rs[k], ps[k]);
-    vrs[k] = ps[k] * ir;
-    half_start(us[k], l2s[k], k == 0 ? +1 : -1, h0[k], h1[k]);
-    const R m2 = us[k] * h1[k] + vrs[k] * h0[k];
-    U0[0] += rs[k] * h0[k];
-    U0[1] += rs[k] * h1[k];
-    U0[2] += rs[k] * (vs[k] * h0[k]);
-    U0[3] += rs[k] * (R(0.5) * m2 + (R(0.5) * vs[k] * vs[k] + C.n1h * vrs[k]) * h0[k]);
+    side_start(C, S.w[0], k, sd[k], U0);
   }
   R r0, ir0, u0, v0, p0;
   prim(U0, C.gm1, r0, ir0, u0, v0, p0);
-  const R var0 = p0 * ir0;
-
-  // Section 4: collision time
-  const R jump = fabs(d_div(ps[0] - ps[1], ps[0] + ps[1])) * dt;
-  const R tau = ns ? d_div(C.mu, p0) + jump : C.tau_eps * dt + C.tau_C * jump;
-  const R tn = ns ? tau : R(0);
-
+  const R tau = collision_time(C, ns, sd[0].p, sd[1].p, p0, dt);
   TimeW<R> w;
   time_weights(dt, tau, w);
   // e = exp(-dt/tau) >= 0 underflows to exactly 0 once tau is a small enough fraction of dt
   // (smooth Euler flow); the point-value terms whose weights carry it are then not formed
   const bool kin_point = w.e > R(0);
-  const R q20 = u0 * u0 + v0 * v0;
-
   R Fl[4], P0[4], P1[4], Mn[4];
-
-  // ---- equilibrium part, Eq. dis1, with g0 and the polynomial of Section 3.3.  All moments
-  // of g0 run over the whole velocity space: in its frame they are closed forms in the central
-  // components of the derivatives.  The compatibility conditions turn the moments of a1 u + a2 v
-  // into those of A, and so on, so that the point value is U0 and its time derivatives. ----
-  {
-    const R U = u0, V = v0, s = var0, hq = R(0.5) * q20, pN = C.i2N, kc = C.n2h * var0;
-    R x[4], y[4], xx[4], xy[4], yy[4];
-    {
-      R avg[2][3][4], d[5][4];
-      src.avg(avg);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const R um = avg[0][0][k], uc = avg[0][1][k], up = avg[0][2][k];
-        const R wm = avg[1][0][k], wc = avg[1][1][k], wp = avg[1][2][k];
-        const R Sr = wp + wm, Sl = up + um, Dr = wp - wm, Dl = up - um, cc = wc + uc;
-        d[0][k] = ((Sr - Sl) + R(2) * (wc - uc)) * C.i4n;                     // b2
-        d[1][k] = (Dr + Dl) * C.i4t;                                          // b3
-        d[2][k] = (R(26) * cc - (Sr + Sl) - R(48) * U0[k]) * C.i8n2;          // b4
-        d[3][k] = (Dr - Dl) * C.i2nt;                                         // b6
-        d[4][k] = ((Sr + Sl) - R(2) * cc) * C.i2t2;                           // b5
-      }
-      central(U, V, hq, d[0], x);
-      central(U, V, hq, d[1], y);
-      central(U, V, hq, d[2], xx);
-      central(U, V, hq, d[3], xy);
-      central(U, V, hq, d[4], yy);
-    }
-    R A[4], tx[4], ty[4], tt[4], S[4], qx[4], qy[4];
-    const R px = pN * xx[3], pxy = pN * xy[3], pyy = pN * yy[3], pt = px + pyy;
-    const R dx = xx[1] + xy[2], dy = xy[1] + yy[2];
-    time_coef(U, V, pN, kc, x, y, A);  // <A + a1 u + a2 v> = 0
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      qx[k] = U * xx[k] + V * xy[k];
-      qy[k] = U * xy[k] + V * yy[k];
-    }
-    // <Axx u + Axy v + Atx> = 0, <Axy u + Ayy v + Aty> = 0
-    tx[0] = -(qx[0] + dx);
-    tx[1] = -(qx[1] + px);
-    tx[2] = -(qx[2] + pxy);
-    tx[3] = -(qx[3] + kc * dx);
-    ty[0] = -(qy[0] + dy);
-    ty[1] = -(qy[1] + pxy);
-    ty[2] = -(qy[2] + pyy);
-    ty[3] = -(qy[3] + kc * dy);
-    // <Atx u + Aty v + Att> = 0
-    const R qt0 = U * tx[0] + V * ty[0], qt1 = U * tx[1] + V * ty[1];
-    const R qt2 = U * tx[2] + V * ty[2], qt3 = U * tx[3] + V * ty[3], dt1 = tx[1] + ty[2];
-    tt[0] = -(qt0 + dt1);
-    tt[1] = -(qt1 + pN * tx[3]);
-    tt[2] = -(qt2 + pN * ty[3]);
-    tt[3] = -(qt3 + kc * dt1);
-    // S = <(Axx u^2 + 2 Axy u v + Ayy v^2) psi'>
-    const R gg = U * dx + V * dy, s1 = s * (R(3) * xx[1] + R(2) * xy[2] + yy[1]);
-    S[0] = (gg - qt0) + pt;
-    S[1] = (U * px + V * pxy - qt1) + s1;
-    S[2] = (U * pxy + V * pyy - qt2) + s * (xx[2] + R(2) * xy[1] + R(3) * yy[2]);
-    S[3] = kc * (gg + R(2) * pt - s * (xx[0] + yy[0])) - qt3;
-    // G0 = <psi' f> and G1 = <c psi' f>, time-integrated: the flux is U G0 + G1
-    const R y2h = R(0.5) * C.y2, h4 = R(0.5) * w.I4, h5 = R(0.5) * w.I5;
-    const R wA = w.I3 - w.I2, wyy = y2h * w.I1, wtt = h5 - w.I6, rI = r0 * w.I1;
-    R G0[4], f[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) G0[k] = wA * A[k] + wyy * yy[k] + wtt * tt[k] + h4 * S[k];
-    G0[0] += rI;
-    G0[3] += rI * (C.nh * s);
-    const R qa1 = U * x[1] + V * y[1], qa3 = U * x[3] + V * y[3];
-    const R b1 = w.I3 * A[1] + h5 * tt[1] + wyy * yy[1] + w.I2 * qa1 + w.I6 * qt1 + h4 * (U * qx[1] + V * qy[1]);
-    const R b3 = w.I3 * A[3] + h5 * tt[3] + wyy * yy[3] + w.I2 * qa3 + w.I6 * qt3 + h4 * (U * qx[3] + V * qy[3]);
-    const R c0 = w.I2 * x[0] + w.I6 * tx[0] + w.I4 * qx[0], c1 = w.I2 * x[1] + w.I6 * tx[1] + w.I4 * qx[1];
-    const R c2 = w.I2 * x[2] + w.I6 * tx[2] + w.I4 * qx[2], c3 = w.I2 * x[3] + w.I6 * tx[3] + w.I4 * qx[3];
-    const R d1 = w.I2 * y[1] + w.I6 * ty[1] + w.I4 * qy[1], d2 = w.I2 * y[2] + w.I6 * ty[2] + w.I4 * qy[2];
-    const R pB = pN * c3, z = h4 * s1, bz = b1 + pB;
-    f[0] = U * G0[0] + (bz + z);
-    f[1] = U * G0[1] + pN * b3 +
-           s * (rI + (R(3) * c1 + d2) + h4 * ((R(6) * px + R(2) * pyy) - s * (R(3) * xx[0] + yy[0])));
-    f[2] = U * G0[2] + s * ((c2 + d1) + w.I4 * (R(2) * pxy - s * xy[0]));
-    f[3] = U * G0[3] + kc * (bz + pB - s * c0) + C.n4h * s * z;
-    lab(U, V, hq, f, Fl);
-    if (C.prandtl) lab(U, V, hq, G0, Mn);
-    // values at t = dt: (1 - e) (U0 + dt U_t + ...), C_3 - C_2 = dt (1 - e),
-    // C_5 / 2 - C_6 = dt^2/2 + dt tau e, C_4 = -(dt^2 + 2 dt tau) e
-    const R pA = dt * w.om, pyw = y2h * w.om, te = tau * w.e, ptt = dt * (R(0.5) * dt + te);
-    const R pS = -dt * (R(0.5) * dt * w.e + te), rE = r0 * w.om;
-    R p[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) p[k] = pA * A[k] + pyw * yy[k] + ptt * tt[k] + pS * S[k];
-    p[0] += rE;
-    p[3] += rE * (C.nh * s);
-    lab(U, V, hq, p, P0);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) p[k] = w.om * y[k] + pA * ty[k];
-    lab(U, V, hq, p, P1);
-  }
-
-  // ---- kinetic part, Eq. dis2, for both sides: NS: f_G = g_k - tau (a u + A) g_k; Euler:
-  // f_G = g_k, the terms with tn are absent (not formed) ----
+  equilibrium_part(C, src, U0, r0, u0, v0, p0 * ir0, w, dt, Fl, P0, P1, Mn);
 #pragma unroll 1
   for (int side = 0; side < 2; ++side) {
-    // selects, not indexing: a dynamic index would put these arrays in local memory
-    const R rho = side ? rs[1] : rs[0], U = side ? us[1] : us[0], V = side ? vs[1] : vs[0];
-    const R s = side ? vrs[1] : vrs[0], l2 = side ? l2s[1] : l2s[0];
-    R a1[4], a2[4], xx[4], xy[4], yy[4], A[4], tx[4], ty[4];
-    {
-      const R hq = R(0.5) * (U * U + V * V), hs = R(0.5) * (U * U + s), c5 = C.i2N * l2;
-      FaceState<R> S;
-      src.side(side, S);
-      R e1[4], e2[4], exx[4], exy[4], eyy[4];
-      central(U, V, hq, S.w[1], e1);
-      central(U, V, hq, S.w[2], e2);
-      central(U, V, hq, S.w[3], exx);
-      central(U, V, hq, S.w[4], exy);
-      central(U, V, hq, S.w[5], eyy);
-      half_coef(U, l2, c5, hs, e1, a1);
-      half_coef(U, l2, c5, hs, e2, a2);
-      half_coef(U, l2, c5, hs, exx, xx);
-      half_coef(U, l2, c5, hs, exy, xy);
-      half_coef(U, l2, c5, hs, eyy, yy);
-      if (ns) {
-        const R kc = C.n2h * s;
-        R t[4];
-        time_coef(U, V, C.i2N, kc, e1, e2, t);
-        half_coef(U, l2, c5, hs, t, A);
-        time_coef(U, V, C.i2N, kc, exx, exy, t);
-        half_coef(U, l2, c5, hs, t, tx);
-        time_coef(U, V, C.i2N, kc, exy, eyy, t);
-        half_coef(U, l2, c5, hs, t, ty);
-      }
-    }
-    R m[8];
-    m[0] = side ? h0[1] : h0[0];
-    m[1] = side ? h1[1] : h1[0];
-#pragma unroll
-    for (int n = 2; n < 8; ++n) m[n] = U * m[n - 1] + (n == 2 ? s : R(n - 1) * s) * m[n - 2];
-
-    // P for the weights w7, w8 = -w9 and w10 of e^(-t/tau), -t e^(-t/tau) and t^2 e^(-t/tau):
-    // v = V + d takes the terms in v to V times themselves and d times themselves
-    auto poly = [&](R w7, R w9, R w10, HalfPoly<R>& P) {
-      R B1[4], Bu[4], Bd[4], wq = R(0.5) * w10, wu = -w9;
-      const R t7 = tn * w7, t8 = -tn * w9;
-      if (ns) {
-        wq -= t8;
-        wu -= t7;
-      }
-      const R wd = R(2) * wq * V, wyy = R(0.5) * C.y2 * w7 - wq * V * V;  // B1 takes V Bd, which holds wd yy
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        Bd[k] = wu * a2[k] + wd * yy[k];
-        Bu[k] = wu * a1[k] + wd * xy[k];
-        if (ns) {
-          Bd[k] = Bd[k] - t8 * ty[k];
-          Bu[k] = Bu[k] - t8 * tx[k];
-          B1[k] = V * Bd[k] + wyy * yy[k] - t7 * A[k];
-        } else {
-          B1[k] = V * Bd[k] + wyy * yy[k];
-        }
-      }
-      half_poly(w7 * rho, B1, Bu, Bd, wq, xx, xy, yy, s, C.n1h, P);
-    };
-    HalfPoly<R> P;
-    poly(w.i7, w.i9, w.i10, P);
-    half_moments<1, 4>(P, m, V, s, C.n1h, Fl);
-    if (C.prandtl) half_moments<0, 4>(P, m, V, s, C.n1h, Mn);
-    // Every weight of the kinetic part at t = dt carries e = exp(-dt/tau), which underflows to
-    // exactly 0 once tau is a small enough fraction of dt (smooth Euler flow): the point
-    // values then get exactly nothing from this side
-    if (kin_point) {
-      const R e9 = dt * w.e;
-      poly(w.e, e9, dt * e9, P);
-      half_moments<0, 4>(P, m, V, s, C.n1h, P0);
-      // the part linear along the face: y (e (a2 - tau Aty) - (t + tau) e (Axy u + Ayy v))
-      const R wy = ns ? -tn * w.e - e9 : -e9, te = tn * w.e;
-      R B1[4], Bu[4], Bd[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        Bd[k] = wy * yy[k];
-        Bu[k] = wy * xy[k];
-        B1[k] = w.e * a2[k] + V * Bd[k];
-        if (ns) B1[k] = B1[k] - te * ty[k];
-      }
-      half_poly_linear(B1, Bu, Bd, s, C.n1h, P);
-      half_moments<0, 3>(P, m, V, s, C.n1h, P1);
-    }
+    // selects, not indexing: a dynamic index would put the sides in local memory
+    const SideData<R> d{side ? sd[1].rho : sd[0].rho, side ? sd[1].U : sd[0].U, side ? sd[1].V : sd[0].V,
+                        side ? sd[1].s : sd[0].s, side ? sd[1].l2 : sd[0].l2, side ? sd[1].p : sd[0].p,
+                        side ? sd[1].h : sd[0].h, side ? sd[1].g : sd[0].g};
+    kinetic_part(C, src, side, d, ns, kin_point, w, ns ? tau : R(0), dt, Fl, P0, P1, Mn);
   }
-
-  // Prandtl-number fix: energy flux += (1/Pr - 1) q, q the time-integrated
-  // face-mean heat flux (1/2) int (u-U0)((u-U0)^2+(v-V0)^2+xi^2) f, written with the
-  // flux and the time-integrated conservative moments.
-  if (C.prandtl) {
-    const R q = Fl[3] - u0 * Fl[1] - v0 * Fl[2] + (R(0.5) * q20 + u0 * u0) * Fl[0] - u0 * Mn[3] +
-                u0 * v0 * Mn[2] - R(0.5) * u0 * q20 * Mn[0];
-    Fl[3] += C.pr_fix * q;
-  }
-  const R yg = R(0.28867513459481287) * C.dtan;  // sqrt(3)/6
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    F[k] = Fl[k];
-    Wm[k] = P0[k] - yg * P1[k];
-    Wp[k] = P0[k] + yg * P1[k];
-  }
+  finish_face(C, u0, v0, Fl, P0, P1, Mn, F, Wm, Wp);
 }
 
 // ---------------------------------------------------------------------------
@@ -797,6 +858,50 @@ GKS_FN void recon_var(R c, R e, R w, R n, R s, R em, R ep, R wm, R wp, R nm, R n
   const R b2 = K.weps + I2, b2sq = b2 * b2;
   // w1 = (1/b1^2) / (1/b1^2 + 1/b2^2) = b2^2 / (b1^2 + b2^2); a = c + w1 (a_one-sided - c)
   const R w1 = d_div(b2sq, K.b1sq + b2sq);
+  a[0] = c2 + w1 * (a2 - c2);
+  a[1] = c3 + w1 * (a3 - c3);
+  a[2] = c4 + w1 * (a4 - c4);
+  a[3] = c5 + w1 * (a5 - c5);
+  a[4] = c6 + w1 * (a6 - c6);
+}
+
+// ---------------------------------------------------------------------------
+// The FP64 form of the same reconstruction of one variable, in units of the cell size: the
+// coefficients come out as (a2 dx, a3 dy, a4 dx^2, a5 dy^2, a6 dx dy).  It is bound by the FP64 pipe,
+// so the cell size enters once at the end, comparisons of magnitudes and signs run on the integer pipe
+// (|a| < |b| as the ordering of their bits), and the weight's quotient is a reciprocal: 86 FP64
+// instructions instead of about 115.  Infinities and NaN among the stencil values reach the smoothness
+// indicator and make every coefficient NaN, as before.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ bool abs_less(double a, double b) {
+  return (__double_as_longlong(a) & 0x7fffffffffffffffll) < (__double_as_longlong(b) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double minmod_bits(double a, double b) {
+  return (__double2hiint(a) ^ __double2hiint(b)) < 0 ? 0.0 : (abs_less(a, b) ? a : b);
+}
+
+__device__ __forceinline__ void recon_var_scaled(double c, double e, double w, double n, double s, double em, double ep,
+                                                 double wm, double wp, double nm, double np, double sm, double sp,
+                                                 double weps, double b1sq, double a[5]) {
+  constexpr double r3 = 1.7320508075688772, sixth = 1.0 / 6.0;
+  const double se = em + ep, sw = wm + wp, sn = nm + np, ss = sm + sp, cc = c + c;
+  const double ce = c + e, cw = c + w, cn = c + n, cs = c + s;
+  const double a4 = 3.0 * minmod_bits(cw - sw, ce - se), a5 = 3.0 * minmod_bits(cs - ss, cn - sn);
+  const double a2 = minmod_bits((cc - sw) + sixth * a4, (se - cc) - sixth * a4);
+  const double a3 = minmod_bits((cc - ss) + sixth * a5, (sn - cc) - sixth * a5);
+  const double de = ep - em, dw = wp - wm, dn = np - nm, ds = sp - sm;
+  const double xe = r3 * de - a3, xw = r3 * dw - a3, yn = r3 * dn - a2, ys = r3 * ds - a2;
+  constexpr double keep = 1.0 - Prec<double>::tie;
+  double a6 = xe + yn, cand = yn - xw;
+  if (abs_less(cand, a6 * keep)) a6 = cand;
+  cand = -xw - ys;
+  if (abs_less(cand, a6 * keep)) a6 = cand;
+  cand = xe - ys;
+  if (abs_less(cand, a6 * keep)) a6 = cand;
+  const double c2 = 0.5 * (e - w), c3 = 0.5 * (n - s), c4 = (ce + cw) - 2.0 * cc, c5 = (cn + cs) - 2.0 * cc;
+  const double c6 = (0.5 * r3) * ((de - dw) + (dn - ds));
+  const double I2 = c2 * c2 + c3 * c3 + (13.0 / 12.0) * (c4 * c4 + c5 * c5) + (7.0 / 6.0) * (c6 * c6);
+  const double b2 = weps + I2, b2sq = b2 * b2, w1 = b2sq * d_rcp(b1sq + b2sq);
   a[0] = c2 + w1 * (a2 - c2);
   a[1] = c3 + w1 * (a3 - c3);
   a[2] = c4 + w1 * (a4 - c4);

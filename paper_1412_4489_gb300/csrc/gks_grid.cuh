@@ -36,6 +36,8 @@ struct Geo {
   size_t plane;       // (ny+2) * pitch
   double dx, dy;
   double idx, idy;                  // 1/dx, 1/dy
+  double idx2, idy2, idxy;          // 1/dx^2, 1/dy^2, 1/(dx dy)
+  double b1sq;                      // (eps + C dx dy)^2 of the reconstruction's weights
   float idx_hi, idx_lo, idy_hi, idy_lo;  // the same as FP32 pairs hi + lo
   double visc;                      // viscous rate bound 2 mu max(4/3, gamma/Pr) / min(dx, dy)^2
   float gamma_f, gm1_f, K_f, visc_f;  // gamma, gamma - 1, K = (4 - 2 gamma) / (gamma - 1), visc in FP32
@@ -125,6 +127,11 @@ inline void geo_finish(Geo& g) {
   g.plane = (size_t)(g.ny + 2) * g.pitch;
   g.idx = 1.0 / g.dx;
   g.idy = 1.0 / g.dy;
+  g.idx2 = g.idx * g.idx;
+  g.idy2 = g.idy * g.idy;
+  g.idxy = g.idx * g.idy;
+  const double b1 = g.weno_eps + g.weno_C * g.dx * g.dy;
+  g.b1sq = b1 * b1;
   g.idx_hi = (float)g.idx;
   g.idx_lo = (float)(g.idx - (double)g.idx_hi);
   g.idy_hi = (float)g.idy;
@@ -555,6 +562,53 @@ __device__ __forceinline__ void recon_cell(const Geo& g, const R* __restrict__ U
   });
 }
 
+// Reconstruction of cell (i, j) in FP64 and conservative variables by four neighbouring lanes, one
+// variable each (lane & 3); every lane of the warp calls it, active: the cell exists.  Same loads and record as
+// recon_cell.  Four times the warps of one thread per cell: the FP64 pipe's interval of 64 cycles
+// per warp instruction makes a cell's serial time the kernel's on grids of up to some 10,000 cells, and
+// on larger ones the register need of one variable lets twice the warps be resident.  81^2 46 -> 15 us
+// (with the event's ~4), 200 x 1 25 -> 11 us, 512^2 276 -> 259 us.
+__device__ __forceinline__ void recon_cell_lanes(const Geo& g, const double* __restrict__ U, const double* __restrict__ Wx,
+                                                 const double* __restrict__ Wy, double* __restrict__ rec, int i, int j,
+                                                 bool active) {
+  const int nx = g.nx, v = threadIdx.x & 3;
+  const size_t fxp = (size_t)g.ny * (nx + 1), fyp = (size_t)(g.ny + 1) * nx;
+  const double* wx = Wx + (size_t)v * 2 * fxp + (size_t)j * (nx + 1) + i;
+  const double* ws = Wy + (size_t)v * 2 * fyp + (size_t)j * nx + i;
+  const double* wn = ws + nx;
+  const double* u = U + ci(g, v, i, j);
+  const double c = u[0];
+  double a[5];
+  recon_var_scaled(c, u[1], u[-1], u[g.pitch], u[-g.pitch], wx[1], wx[fxp + 1], wx[0], wx[fxp], wn[0], wn[fyp], ws[0],
+                   ws[fyp], g.weno_eps, g.b1sq, a);
+  // the polynomial at the four face centres: positive density and pressure
+  // (2 rho rho E > |rho u|^2), else the constant average
+  const double p4 = (1.0 / 12.0) * a[2], p5 = (1.0 / 12.0) * a[3];
+  const double e0 = c + (p4 - 0.5 * p5), n0 = c + (p5 - 0.5 * p4);
+  const double f[4] = {e0 + 0.5 * a[0], e0 - 0.5 * a[0], n0 + 0.5 * a[1], n0 - 0.5 * a[1]};
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    // lane 0: 2 rho rho E, lanes 1 and 2: minus their momentum squared; the sum over the four
+    const double E = __shfl_down_sync(0xffffffffu, f[k], 3, 4);
+    double t = f[k] * (v == 0 ? E + E : (v == 3 ? 0.0 : -f[k]));
+    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    t += __shfl_xor_sync(0xffffffffu, t, 2);
+    // t > 0 and (lane 0) the density > 0, as orderings of their bits: NaN lies above infinity
+    auto positive = [](double x) { return (unsigned long long)(__double_as_longlong(x) - 1) < 0x7ff0000000000000ull; };
+    ok = ok && positive(t) && (v != 0 || positive(f[k]));
+  }
+  const bool bad = !__shfl_sync(0xffffffffu, (int)ok, 0, 4);
+  if (!active) return;
+  double* r = rec + ri(g, i, j) + v;
+  const double scale[5] = {g.idx, g.idy, g.idx2, g.idy2, g.idxy};
+  r[0] = c;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) r[4 + 4 * k] = bad ? 0.0 : scale[k] * a[k];
+  // the ghost ring's averages (boundary images written by the last update)
+  for_each_ghost_of(g, i, j, [&](int gi, int gj) { rec[ri(g, gi, gj) + v] = U[ci(g, v, gi, gj)]; });
+}
+
 // ---------------------------------------------------------------------------
 // face evolution
 // ---------------------------------------------------------------------------
@@ -694,22 +748,17 @@ __host__ __device__ inline FaceConst<R> grid_face_const(const Geo& g, int axis) 
   return face_const<R>(P);
 }
 
-// the evolution at face (i, j) of axis AX: flux F and new point values Wn
-// (NSM: Navier-Stokes 1, Euler 0, decided per grid at run time -1; MONO: the routine in
-// velocity monomials, of FP32 batches)
-template <int AX, class R, class TW, int NSM = -1, bool MONO = false>
-__device__ __forceinline__ void flux_face(const Geo& g, const FaceConst<R>& C, const R* __restrict__ rec,
-                                          TW* __restrict__ Wn, R* __restrict__ F, int i, int j, R dt) {
-  const int nx = g.nx, ny = g.ny;
-  const int fx = AX == 0 ? nx + 1 : nx, fy = AX == 0 ? ny : ny + 1;
+// the inputs of face (i, j) of axis AX; U (may be null) serves constant states only
+template <int AX, class R>
+__device__ __forceinline__ GridFaceSource<AX, R> face_source(const Geo& g, const R* U, const R* rec, int i, int j) {
   GridFaceSource<AX, R> src;
   src.g = &g;
-  src.U = nullptr;
+  src.U = U;
   src.rec = rec;
   src.i = i;
   src.j = j;
-  const int f = AX == 0 ? i : j;     // face index along the normal
-  const int nf = AX == 0 ? nx : ny;  // faces 0 and nf are on the boundary
+  const int f = AX == 0 ? i : j;         // face index along the normal
+  const int nf = AX == 0 ? g.nx : g.ny;  // faces 0 and nf are on the boundary
   const int lo_side = AX == 0 ? 0 : 2, hi_side = lo_side + 1;
   // the two cells along the normal: across a periodic side the wrapped cell, across an
   // exchange side the neighbouring slab's (its record in the halo row), across any other
@@ -725,30 +774,123 @@ __device__ __forceinline__ void flux_face(const Geo& g, const FaceConst<R>& C, c
     if (g.bc.kind[hi_side] == GKS_BC_PERIODIC) src.cr = 0;
     else if (g.bc.kind[hi_side] != GKS_BC_EXCHANGE) src.img_hi = g.bc.kind[hi_side];
   }
-  src.hn = C.dn;
-  src.ht = C.dtan;
-  src.hn2_12 = C.dn2_12;
-  src.ht2_24 = C.dt2_24;
-  src.gamma = C.gamma;
+  src.gamma = GeoR<R>::gamma(g);
   src.uwt_lo = GeoR<R>::uwt(g, lo_side);
   src.Tw_lo = GeoR<R>::Tw(g, lo_side);
   src.uwt_hi = GeoR<R>::uwt(g, hi_side);
   src.Tw_hi = GeoR<R>::Tw(g, hi_side);
   src.first_order = false;
+  return src;
+}
 
-  R Fl[4], Wm[4], Wp[4];
-  if constexpr (MONO) monomials::face_evolution<R, NSM>(C, src, dt, Fl, Wm, Wp);
-  else face_evolution<R, NSM>(C, src, dt, Fl, Wm, Wp);
+// the same with the cell sizes that a polynomial's face state needs
+template <int AX, class R>
+__device__ __forceinline__ GridFaceSource<AX, R> face_source(const Geo& g, const FaceConst<R>& C, const R* rec, int i, int j) {
+  GridFaceSource<AX, R> src = face_source<AX, R>(g, (const R*)nullptr, rec, i, j);
+  src.hn = C.dn;
+  src.ht = C.dtan;
+  src.hn2_12 = C.dn2_12;
+  src.ht2_24 = C.dt2_24;
+  src.gamma = C.gamma;
+  return src;
+}
+
+// the wall's flux rule, then flux and point values to memory in physical components
+template <int AX, class R, class TW>
+__device__ __forceinline__ void store_face(const Geo& g, const GridFaceSource<AX, R>& src, TW* __restrict__ Wn,
+                                           R* __restrict__ F, R Fl[4], const R Wm[4], const R Wp[4]) {
   if (src.img_lo) wall_face_flux<R>(src.img_lo, src.uwt_lo, Fl);
   else if (src.img_hi) wall_face_flux<R>(src.img_hi, src.uwt_hi, Fl);
-
-  const size_t nfaces = (size_t)fx * fy, o = (size_t)j * fx + i;
+  const int fx = AX == 0 ? g.nx + 1 : g.nx, fy = AX == 0 ? g.ny : g.ny + 1;
+  const size_t nfaces = (size_t)fx * fy, o = (size_t)src.j * fx + src.i;
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     const int k = slot<AX>(v);
     F[(size_t)v * nfaces + o] = Fl[k];
     Wn[(size_t)(v * 2 + 0) * nfaces + o] = TW(Wm[k]);
     Wn[(size_t)(v * 2 + 1) * nfaces + o] = TW(Wp[k]);
+  }
+}
+
+// the evolution at face (i, j) of axis AX: flux F and new point values Wn
+// (NSM: Navier-Stokes 1, Euler 0, decided per grid at run time -1; MONO: the routine in
+// velocity monomials, of FP32 batches)
+template <int AX, class R, class TW, int NSM = -1, bool MONO = false>
+__device__ __forceinline__ void flux_face(const Geo& g, const FaceConst<R>& C, const R* __restrict__ rec,
+                                          TW* __restrict__ Wn, R* __restrict__ F, int i, int j, R dt) {
+  const GridFaceSource<AX, R> src = face_source<AX, R>(g, C, rec, i, j);
+  R Fl[4], Wm[4], Wp[4];
+  if constexpr (MONO) monomials::face_evolution<R, NSM>(C, src, dt, Fl, Wm, Wp);
+  else face_evolution<R, NSM>(C, src, dt, Fl, Wm, Wp);
+  store_face<AX, R, TW>(g, src, Wn, F, Fl, Wm, Wp);
+}
+
+// What the three warps of a split face group exchange: the sides' shares of U0 and pressures, then
+// their kinetic parts of flux, point values and time-integrated means.
+template <class R>
+struct SplitShare {
+  R u0[2][4][32], p[2][32], part[2][16][32];
+};
+
+// The evolution at 32 faces by three warps: the left side (warp 0), the right side (warp 1) and the equilibrium
+// part (warp 2), each with the same arithmetic as face_evolution.  Every thread of the 96 calls it; active: the
+// lane has a face.
+template <int AX, class R, class TW, int NSM>
+__device__ __forceinline__ void flux_face_split(const Geo& g, const FaceConst<R>& C, const R* __restrict__ rec,
+                                                TW* __restrict__ Wn, R* __restrict__ F, int i, int j, bool active, R dt,
+                                                SplitShare<R>& sh) {
+  const int role = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool ns = NSM < 0 ? C.ns : NSM == 1;
+  const GridFaceSource<AX, R> src = face_source<AX, R>(g, C, rec, i, j);
+  SideData<R> sd;
+  if (active && role < 2) {
+    FaceState<R> S;
+    src.side(role, S);
+    R u[4] = {R(0), R(0), R(0), R(0)};
+    side_start(C, S.w[0], role, sd, u);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) sh.u0[role][k][lane] = u[k];
+    sh.p[role][lane] = sd.p;
+  }
+  __syncthreads();
+  R r0, ir0, u0, v0, p0, Fl[4], P0[4], P1[4], Mn[4];
+  if (active) {
+    R U0[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) U0[k] = sh.u0[0][k][lane] + sh.u0[1][k][lane];
+    prim(U0, C.gm1, r0, ir0, u0, v0, p0);
+    const R tau = collision_time(C, ns, sh.p[0][lane], sh.p[1][lane], p0, dt);
+    TimeW<R> w;
+    time_weights(dt, tau, w);
+    if (role == 2) {
+      equilibrium_part(C, src, U0, r0, u0, v0, p0 * ir0, w, dt, Fl, P0, P1, Mn);
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) Fl[k] = P0[k] = P1[k] = Mn[k] = R(0);
+      kinetic_part(C, src, role, sd, ns, w.e > R(0), w, ns ? tau : R(0), dt, Fl, P0, P1, Mn);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        sh.part[role][k][lane] = Fl[k];
+        sh.part[role][4 + k][lane] = P0[k];
+        sh.part[role][8 + k][lane] = P1[k];
+        sh.part[role][12 + k][lane] = Mn[k];
+      }
+    }
+  }
+  __syncthreads();
+  if (active && role == 2) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        Fl[k] += sh.part[q][k][lane];
+        P0[k] += sh.part[q][4 + k][lane];
+        P1[k] += sh.part[q][8 + k][lane];
+        if (C.prandtl) Mn[k] += sh.part[q][12 + k][lane];
+      }
+    R Fo[4], Wm[4], Wp[4];
+    finish_face(C, u0, v0, Fl, P0, P1, Mn, Fo, Wm, Wp);
+    store_face<AX, R, TW>(g, src, Wn, F, Fo, Wm, Wp);
   }
 }
 
@@ -808,30 +950,7 @@ __device__ __forceinline__ void block_bound_to(R inv, unsigned long long* slot) 
 template <int AX, class R>
 __device__ __forceinline__ void kfvs_face(const Geo& g, const R* U, R gm1, R K, int i, int j, R dt, R F[4],
                                           R W[4]) {
-  GridFaceSource<AX, R> src;
-  src.g = &g;
-  src.U = U;
-  src.rec = nullptr;
-  src.i = i;
-  src.j = j;
-  const int f = AX == 0 ? i : j, nf = AX == 0 ? g.nx : g.ny;
-  const int lo_side = AX == 0 ? 0 : 2, hi_side = lo_side + 1;
-  src.cl = f - 1;
-  src.cr = f;
-  src.img_lo = src.img_hi = 0;
-  if (f == 0) {
-    if (g.bc.kind[lo_side] == GKS_BC_PERIODIC) src.cl = nf - 1;
-    else if (g.bc.kind[lo_side] != GKS_BC_EXCHANGE) src.img_lo = g.bc.kind[lo_side];
-  }
-  if (f == nf) {
-    if (g.bc.kind[hi_side] == GKS_BC_PERIODIC) src.cr = 0;
-    else if (g.bc.kind[hi_side] != GKS_BC_EXCHANGE) src.img_hi = g.bc.kind[hi_side];
-  }
-  src.gamma = GeoR<R>::gamma(g);
-  src.uwt_lo = GeoR<R>::uwt(g, lo_side);
-  src.Tw_lo = GeoR<R>::Tw(g, lo_side);
-  src.uwt_hi = GeoR<R>::uwt(g, hi_side);
-  src.Tw_hi = GeoR<R>::Tw(g, hi_side);
+  GridFaceSource<AX, R> src = face_source<AX, R>(g, U, (const R*)nullptr, i, j);
   src.first_order = true;
   R Ff[4] = {R(0), R(0), R(0), R(0)}, Wf[4] = {R(0), R(0), R(0), R(0)};
 #pragma unroll
