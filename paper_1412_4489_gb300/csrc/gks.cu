@@ -37,10 +37,6 @@ namespace {
 
 constexpr int kLaunchesPerStep = 7;
 
-template <class T> struct Store;
-template <> struct Store<double> { static __device__ __forceinline__ double to(double x) { return x; } };
-template <> struct Store<float> { static __device__ __forceinline__ float to(double x) { return (float)x; } };
-
 // ---------------------------------------------------------------------------
 // control kernels
 // ---------------------------------------------------------------------------
@@ -65,14 +61,29 @@ __global__ void k_ghost(Geo g, Cells<R> U0, Cells<R> U1, const Ctrl* c, int forc
 // begin = 1: block 0 also opens the step (ctrl_begin); the other blocks then do
 // not look at the skip flag it sets (coefficients of a skipped step go unused).
 // CHAR: reconstruction in characteristic variables.
-// block heights (of 32 cells) and resident blocks per SM the reconstruction is compiled for: FP32
-// conservative 8 and 4 (64 registers; the kernel is latency-bound, so occupancy pays), FP32
-// characteristic 8 and 2 (128); FP64 characteristic 1 and 8 (it needs more than 128, and one-warp blocks spread
-// over the SMs evenly)
+
+// bytes (a multiple of 16, both addresses too) that the warp's lanes wrote to shared memory, to
+// global memory in one bulk copy; complete on return.  Every lane of the warp calls it.
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, unsigned bytes) {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst),
+                 "r"((unsigned)__cvta_generic_to_shared(src)), "r"(bytes)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+    asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+  }
+}
+
+// block heights (of 32 cells) and resident blocks per SM the reconstruction is compiled for.  FP32
+// conservative 8 and 3 (80 registers hold a cell's 13 stencil vectors without spills; 4 blocks at 64 spill: 512^2
+// step 49.5 against 48.4 us, 5 blocks 55), FP32 characteristic 8 and 2 (128; 1 and 3 are slower); FP64
+// characteristic 1 and 8 (it needs more than 128, and one-warp blocks spread over the SMs evenly)
 template <class R> struct ReconRows { static constexpr int value = 8; };
 template <> struct ReconRows<double> { static constexpr int value = 1; };
 template <class R, bool CHAR> struct ReconBlocks { static constexpr int value = 2; };
-template <> struct ReconBlocks<float, false> { static constexpr int value = 4; };
+template <> struct ReconBlocks<float, false> { static constexpr int value = 3; };
 template <> struct ReconBlocks<double, true> { static constexpr int value = 8; };
 
 template <class R, class TW, bool CHAR>
@@ -89,9 +100,26 @@ __global__ void __launch_bounds__(32 * ReconRows<R>::value, ReconBlocks<R, CHAR>
   }
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = (sizeof(R) == 8 ? blockIdx.z * gridDim.y + blockIdx.y : blockIdx.y) * blockDim.y + threadIdx.y;
-  if (i >= g.nx || j >= g.ny) return;
   const int par = (int)(c->steps & 1);
-  recon_cell<R, TW, CHAR>(g, par ? U1 : U0, par ? Wx1 : Wx0, par ? Wy1 : Wy0, rec, i, j, dx, dy, weps, wC);
+  if constexpr (sizeof(R) == 8) {
+    if (i >= g.nx || j >= g.ny) return;
+    recon_cell<R, CHAR>(g, par ? U1 : U0, par ? Wx1 : Wx0, par ? Wy1 : Wy0, rec, i, j, dx, dy, weps, wC);
+  } else {
+    // FP32: a warp's 32 records are 3,072 contiguous bytes.  Written by its lanes they would go out as 16-byte
+    // pieces at a stride of 96; they are laid down in shared memory and leave in one bulk copy
+    // (2048^2: 156 -> 139 us).
+    __shared__ __align__(16) R stage[ReconRows<R>::value][32 * kRec];
+    if (j >= g.ny) return;  // whole warps: a block row is a row of cells
+    R* mine = stage[threadIdx.y];
+    if (i < g.nx) {
+      R r[kRec];
+      recon_record<R, CHAR>(g, par ? U1 : U0, par ? Wx1 : Wx0, par ? Wy1 : Wy0, i, j, dx, dy, weps, wC, r);
+      Lay<R>::store_rec(mine, threadIdx.x, r);
+      ghost_records(g, par ? U1 : U0, rec, i, j);
+    }
+    const int i0 = blockIdx.x * blockDim.x, count = g.nx - i0 < 32 ? g.nx - i0 : 32;
+    bulk_store(rec + rec_at(g, i0, j) * kRec, mine, (unsigned)(count * kRec * sizeof(R)));
+  }
 }
 
 // FP64 in conservative variables: four lanes to a cell (recon_cell_lanes), eight cells to a one-warp block,
@@ -116,15 +144,15 @@ __global__ void __launch_bounds__(32, 16) k_recon_lanes(Geo g, const double* U0,
 // ---------------------------------------------------------------------------
 // face evolution
 // ---------------------------------------------------------------------------
-// resident 128-thread blocks per SM the FP32 face kernel is compiled for (register cap): 4 blocks = 16 warps per SM at 128 registers (registers are allocated per SM
-// quarter, so more than 12 warps means at most 128); the Euler routine fits without
-// spilling, and the extra warps hide more of its latency than 3 blocks at 168 registers.
-#ifndef GKS_FLUX_MINB_F32
-#define GKS_FLUX_MINB_F32 4
-#endif
+// resident 128-thread blocks per SM the FP32 face kernel is compiled for: Euler 5 (96 registers,
+// 20 warps per SM; 16-52 bytes of spill), Navier-Stokes 4 (128 registers; at 96 it spills 100-144 bytes).
+// x-faces at 2048^2, 4 / 5 blocks: Euler 222 / 207 us; Navier-Stokes at 1024^2 79.5 / 80.4 us.  6 blocks (80
+// registers) are slower for both, 3 slower for Navier-Stokes.
+template <int NS> struct FluxBlocks { static constexpr int value = NS ? 4 : 5; };
+
 // NS: Navier-Stokes (1) or Euler (0) face routine, chosen per grid by flux_kernel
 template <int AX, class R, class TW, int NS>
-__global__ void __launch_bounds__(128, GKS_FLUX_MINB_F32) k_flux(Geo g, FaceConst<R> C, const R* __restrict__ rec,
+__global__ void __launch_bounds__(128, FluxBlocks<NS>::value) k_flux(Geo g, FaceConst<R> C, const R* __restrict__ rec,
                                                                     TW* Wn0, TW* Wn1, R* __restrict__ F,
                                                                     const Ctrl* c, int force) {
   pdl_enter();
@@ -325,13 +353,13 @@ __global__ void k_scatter_U(Geo g, const double* __restrict__ src, Cells<R> U0, 
   }
 }
 
+// face values between the caller's planes [4][2][faces] (n = 8 x faces values) and the layout of the type
 template <class TW>
 __global__ void k_copy_W(const double* __restrict__ src, TW* W0, TW* W1, size_t n, const Ctrl* c, int to_dev) {
   const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   TW* W = (c->steps & 1) ? W1 : W0;
-  if (to_dev) W[k] = Store<TW>::to(src[k]);
-  else const_cast<double*>(src)[k] = (double)W[k];
+  copy_w(src, W, n / 8, k, to_dev);
 }
 
 // face values = mean of the two adjacent averages (ghosts included)
@@ -348,8 +376,7 @@ __global__ void k_init_W(Geo g, Cells<TW> U0, Cells<TW> U1, TW* W0, TW* W1, cons
   for (int v = 0; v < 4; ++v) {
     const double a = U.get(g, v, AX == 0 ? i - 1 : i, AX == 0 ? j : j - 1);
     const double b = U.get(g, v, i, j);
-    W[(size_t)(v * 2) * n + o] = Store<TW>::to(0.5 * (a + b));
-    W[(size_t)(v * 2 + 1) * n + o] = Store<TW>::to(0.5 * (a + b));
+    W[Lay<TW>::w(n, v, 0, o)] = W[Lay<TW>::w(n, v, 1, o)] = TW(0.5 * (a + b));
   }
 }
 
@@ -360,17 +387,18 @@ __global__ void k_coef_out(Geo g, Cells<R> U0, Cells<R> U1, const R* rec, double
   if (i >= g.nx || j >= g.ny) return;
   const Cells<R> U = (c->steps & 1) ? U1 : U0;
   const size_t N = (size_t)g.nx * g.ny, o = (size_t)j * g.nx + i;
-  const R* r = rec + ri(g, i, j);
+  const R* r = rec + rec_at(g, i, j) * kRec;
   for (int v = 0; v < 4; ++v) {
     out[(size_t)(v * 6) * N + o] = U.get(g, v, i, j);
     for (int k = 0; k < 5; ++k) out[(size_t)(v * 6 + k + 1) * N + o] = (double)r[4 + 4 * k + v];
   }
 }
 
+// fluxes as planes [4][faces]
 template <class R>
-__global__ void k_to_double(const R* src, double* dst, size_t n) {
+__global__ void k_flux_out(const R* F, double* dst, size_t faces) {
   const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n) dst[k] = (double)src[k];
+  if (k < 4 * faces) dst[k] = (double)F[Lay<R>::f(faces, (int)(k / faces), k % faces)];
 }
 
 // opens a step of the partitioned form with the dt the caller reduced over all slabs
@@ -1024,17 +1052,23 @@ gks_status gks_debug_flux(gks_handle* h, double dt, double* Fx, double* Fy, doub
   if (st != GKS_OK) return st;
   st = read_ctrl(h);
   if (st != GKS_OK) return st;
-  const int par = (int)(h->hctrl->steps & 1) ^ 1;  // new values were written to the other buffer
-  const size_t nfx = (size_t)4 * g.ny * (g.nx + 1), nfy = (size_t)4 * (g.ny + 1) * g.nx;
-  struct { void* src; double* dst; size_t n; } parts[4] = {
-      {h->Fx, Fx, nfx}, {h->Fy, Fy, nfy}, {h->Wx[par], Wxn, n_wx(g)}, {h->Wy[par], Wyn, n_wy(g)}};
+  // new face values were written to the buffer that is not in use: as k_copy_W's other one
+  const size_t nfx = (size_t)g.ny * (g.nx + 1), nfy = (size_t)(g.ny + 1) * g.nx;
+  struct { void *a, *b; double* dst; size_t faces; bool w; } parts[4] = {
+      {h->Fx, h->Fx, Fx, nfx, false}, {h->Fy, h->Fy, Fy, nfy, false}, {h->Wx[1], h->Wx[0], Wxn, nfx, true}, {h->Wy[1], h->Wy[0], Wyn, nfy, true}};
   for (auto& p : parts) {
     if (!p.dst) continue;
-    if (h->prec == GKS_FP64)
-      k_to_double<double><<<(unsigned)((p.n + 255) / 256), 256, 0, h->stream>>>((const double*)p.src, h->staging, p.n);
-    else
-      k_to_double<float><<<(unsigned)((p.n + 255) / 256), 256, 0, h->stream>>>((const float*)p.src, h->staging, p.n);
-    CK(cudaMemcpyAsync(p.dst, h->staging, p.n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    const size_t n = (p.w ? 8 : 4) * p.faces;
+    const unsigned blocks = (unsigned)((n + 255) / 256);
+    if (h->prec == GKS_FP64) {
+      if (p.w) k_copy_W<double><<<blocks, 256, 0, h->stream>>>(h->staging, (double*)p.a, (double*)p.b, n, h->ctrl, 0);
+      else k_flux_out<double><<<blocks, 256, 0, h->stream>>>((const double*)p.a, h->staging, p.faces);
+    } else {
+      if (p.w) k_copy_W<float><<<blocks, 256, 0, h->stream>>>(h->staging, (float*)p.a, (float*)p.b, n, h->ctrl, 0);
+      else k_flux_out<float><<<blocks, 256, 0, h->stream>>>((const float*)p.a, h->staging, p.faces);
+    }
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(p.dst, h->staging, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   }
   CK(cudaStreamSynchronize(h->stream));
   return GKS_OK;
@@ -1099,12 +1133,14 @@ gks_status part_row(gks_handle* h, int side, int what, bool halo, char** p, size
   const size_t es = h->prec == GKS_FP64 ? sizeof(double) : sizeof(float);
   if (what == GKS_PART_STATE) {
     const int par = (int)(h->hctrl->steps & 1);
-    *p = (char*)h->U[par] + ((size_t)(j + 1) * g.pitch) * es;
-    *pitch = g.plane * es;
-    *rows = h->prec == GKS_FP64 ? 4 : 8;
-    *width = (size_t)(g.nx + 2) * es;
+    // FP64: the row of each of the four planes; FP32: of the hi and of the lo vectors
+    const int per = h->prec == GKS_FP64 ? 1 : 4;
+    *p = (char*)h->U[par] + ((size_t)(j + 1) * g.pitch) * per * es;
+    *pitch = g.plane * per * es;
+    *rows = h->prec == GKS_FP64 ? 4 : 2;
+    *width = (size_t)(g.nx + 2) * per * es;
   } else {
-    *p = (char*)h->rec + ri(g, -1, j) * es;
+    *p = (char*)h->rec + rec_at(g, -1, j) * kRec * es;
     *pitch = 0;
     *rows = 1;
     *width = (size_t)(g.nx + 2) * kRec * es;

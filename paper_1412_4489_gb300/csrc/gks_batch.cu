@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kThreads, BatchBlocks<R>::value) k_batch(Args<
         for (int r = 0; r < kCellsPerThread; ++r) {
           const int i = w.y + tid % a.cell_tw, j = w.z + tid / a.cell_tw + r * (kThreads / a.cell_tw);
           if (i < g.nx && j < g.ny)
-            recon_cell<R, TW, CHAR>(g, U, a.Wx[par] + o.wx, a.Wy[par] + o.wy, a.rec + o.rec, i, j, GeoR<R>::dx(g),
+            recon_cell<R, CHAR>(g, U, a.Wx[par] + o.wx, a.Wy[par] + o.wy, a.rec + o.rec, i, j, GeoR<R>::dx(g),
                                     GeoR<R>::dy(g), GeoR<R>::weps(g), GeoR<R>::wC(g));
         }
       }
@@ -271,8 +271,7 @@ template <class TW>
 __global__ void kb_copyW(const double* src, TW* W, size_t n, int to_dev) {
   const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
-  if (to_dev) W[k] = (TW)src[k];
-  else const_cast<double*>(src)[k] = (double)W[k];
+  copy_w(src, W, n / 8, k, to_dev);
 }
 
 template <class R>

@@ -760,14 +760,9 @@ GKS_FN void face_evolution(const FaceConst<R>& C, const Src& src, R dt, R F[4], 
   const bool kin_point = w.e > R(0);
   R Fl[4], P0[4], P1[4], Mn[4];
   equilibrium_part(C, src, U0, r0, u0, v0, p0 * ir0, w, dt, Fl, P0, P1, Mn);
-#pragma unroll 1
-  for (int side = 0; side < 2; ++side) {
-    // selects, not indexing: a dynamic index would put the sides in local memory
-    const SideData<R> d{side ? sd[1].rho : sd[0].rho, side ? sd[1].U : sd[0].U, side ? sd[1].V : sd[0].V,
-                        side ? sd[1].s : sd[0].s, side ? sd[1].l2 : sd[0].l2, side ? sd[1].p : sd[0].p,
-                        side ? sd[1].h : sd[0].h, side ? sd[1].g : sd[0].g};
-    kinetic_part(C, src, side, d, ns, kin_point, w, ns ? tau : R(0), dt, Fl, P0, P1, Mn);
-  }
+#pragma unroll
+  for (int side = 0; side < 2; ++side)
+    kinetic_part(C, src, side, sd[side], ns, kin_point, w, ns ? tau : R(0), dt, Fl, P0, P1, Mn);
   finish_face(C, u0, v0, Fl, P0, P1, Mn, F, Wm, Wp);
 }
 

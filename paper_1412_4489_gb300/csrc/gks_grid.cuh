@@ -51,73 +51,108 @@ struct Geo {
   BCs bc;
 };
 
-__host__ __device__ __forceinline__ size_t ci(const Geo& g, int v, int i, int j) {
-  return (size_t)v * g.plane + (size_t)(j + 1) * g.pitch + (i + 1);
-}
-
 // ---------------------------------------------------------------------------
-// Reconstruction records.  Per cell, ghost ring included, the compute-type cell
-// average and the coefficient vectors a2..a6 of Section 3.2, four variables each:
-// 24 contiguous values (96 bytes in FP32, 192 in FP64), so that a face reads each
-// of its two cells with 16-byte loads from one address instead of gathering 24
-// values from separate planes.  Ghost records hold only the average (the images
-// of the ghost ring), which the equilibrium polynomial of Section 3.3 reads.
+// Layouts by compute type.  FP64: one plane per variable (and Gauss point) of cell averages, face values and
+// fluxes; those kernels are bound by the FP64 pipe, and the allocation-free step works on the caller's
+// planes in place.  FP32: the four variables of a cell, Gauss point or face are one 16-byte vector: a
+// cell's reconstruction takes 13 loads instead of 52, a face 3 stores instead of 12, an update 6
+// loads and 2 stores instead of 24 and 8.  At 2048^2 reconstruction 177 -> 139 us (79% of copy
+// bandwidth, with bulk-stored records), update 96 -> 76 us (79%).
+// Reconstruction records hold, per cell, ghost ring included, the compute-type cell average
+// and the coefficient vectors a2..a6 of Section 3.2, four variables each.  Ghost records hold only
+// the average (the images of the ghost ring), which the equilibrium polynomial of Section 3.3 reads.
 //   [0..3] average, [4 + 4 (k - 2) + v] = a_k of variable v, k = 2..6
+// A face reads each of its two cells' 24 contiguous values from one address (six planes of vectors, the
+// same bytes at six addresses, cost the face kernels 10% and give the reconstruction 5%: 2048^2 x-faces 207 -> 227 us).
 // ---------------------------------------------------------------------------
 constexpr int kRec = 24;
 
-__host__ __device__ __forceinline__ size_t rec_count(const Geo& g) { return (size_t)(g.nx + 2) * (g.ny + 2) * kRec; }
-__host__ __device__ __forceinline__ size_t ri(const Geo& g, int i, int j) {
-  return ((size_t)(j + 1) * (g.nx + 2) + (i + 1)) * kRec;
+__host__ __device__ __forceinline__ size_t cell_at(const Geo& g, int i, int j) {
+  return (size_t)(j + 1) * g.pitch + (i + 1);
+}
+__host__ __device__ __forceinline__ size_t rec_cells(const Geo& g) { return (size_t)(g.nx + 2) * (g.ny + 2); }
+__host__ __device__ __forceinline__ size_t rec_count(const Geo& g) { return rec_cells(g) * kRec; }
+__host__ __device__ __forceinline__ size_t rec_at(const Geo& g, int i, int j) {
+  return (size_t)(j + 1) * (g.nx + 2) + (i + 1);
 }
 
-template <class R> struct RecIO;
-template <> struct RecIO<float> {
-  static __device__ __forceinline__ void load(const float* __restrict__ p, float r[kRec]) {
-    const float4* q = reinterpret_cast<const float4*>(p);
+template <class R> struct Lay;
+template <> struct Lay<double> {
+  // average of variable v in padded cell arrays; point value of variable v at Gauss point p and flux of variable
+  // v of face o (of n)
+  static __host__ __device__ __forceinline__ size_t u(const Geo& g, int v, int i, int j) { return (size_t)v * g.plane + cell_at(g, i, j); }
+  static __host__ __device__ __forceinline__ size_t w(size_t n, int v, int p, size_t o) { return (size_t)(v * 2 + p) * n + o; }
+  static __host__ __device__ __forceinline__ size_t f(size_t n, int v, size_t o) { return (size_t)v * n + o; }
+  static __device__ __forceinline__ void load_u(const Geo& g, const double* p, int i, int j, double o[4]) {
 #pragma unroll
-    for (int k = 0; k < kRec / 4; ++k) {
-      const float4 t = q[k];
-      r[4 * k] = t.x; r[4 * k + 1] = t.y; r[4 * k + 2] = t.z; r[4 * k + 3] = t.w;
-    }
+    for (int v = 0; v < 4; ++v) o[v] = p[u(g, v, i, j)];
   }
-  static __device__ __forceinline__ void load_avg(const float* __restrict__ p, float r[4]) {
-    const float4 t = *reinterpret_cast<const float4*>(p);
-    r[0] = t.x; r[1] = t.y; r[2] = t.z; r[3] = t.w;
-  }
-  static __device__ __forceinline__ void store(float* p, const float r[kRec]) {
-    float4* q = reinterpret_cast<float4*>(p);
+  static __device__ __forceinline__ void load_w(const double* p, size_t n, int q, size_t o, double x[4]) {
 #pragma unroll
-    for (int k = 0; k < kRec / 4; ++k) q[k] = make_float4(r[4 * k], r[4 * k + 1], r[4 * k + 2], r[4 * k + 3]);
+    for (int v = 0; v < 4; ++v) x[v] = p[w(n, v, q, o)];
   }
-  static __device__ __forceinline__ void store_avg(float* p, const float r[4]) {
-    *reinterpret_cast<float4*>(p) = make_float4(r[0], r[1], r[2], r[3]);
+  static __device__ __forceinline__ void load_f(const double* p, size_t n, size_t o, double x[4]) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) x[v] = p[f(n, v, o)];
   }
-};
-template <> struct RecIO<double> {
-  static __device__ __forceinline__ void load(const double* __restrict__ p, double r[kRec]) {
-    const double2* q = reinterpret_cast<const double2*>(p);
+  static __device__ __forceinline__ void store_w(double* p, size_t n, int q, size_t o, const double x[4]) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) p[w(n, v, q, o)] = x[v];
+  }
+  static __device__ __forceinline__ void store_f(double* p, size_t n, size_t o, const double x[4]) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) p[f(n, v, o)] = x[v];
+  }
+  static __device__ __forceinline__ void load_rec(const double* p, size_t c, double r[kRec]) {
+    const double2* q = reinterpret_cast<const double2*>(p + c * kRec);
 #pragma unroll
     for (int k = 0; k < kRec / 2; ++k) {
       const double2 t = q[k];
       r[2 * k] = t.x; r[2 * k + 1] = t.y;
     }
   }
-  static __device__ __forceinline__ void load_avg(const double* __restrict__ p, double r[4]) {
-    const double2* q = reinterpret_cast<const double2*>(p);
+  static __device__ __forceinline__ void load_avg(const double* p, size_t c, double r[4]) {
+    const double2* q = reinterpret_cast<const double2*>(p + c * kRec);
     const double2 a = q[0], b = q[1];
     r[0] = a.x; r[1] = a.y; r[2] = b.x; r[3] = b.y;
   }
-  static __device__ __forceinline__ void store(double* p, const double r[kRec]) {
-    double2* q = reinterpret_cast<double2*>(p);
+  static __device__ __forceinline__ void store_rec(double* p, size_t c, const double r[kRec]) {
+    double2* q = reinterpret_cast<double2*>(p + c * kRec);
 #pragma unroll
     for (int k = 0; k < kRec / 2; ++k) q[k] = make_double2(r[2 * k], r[2 * k + 1]);
   }
-  static __device__ __forceinline__ void store_avg(double* p, const double r[4]) {
-    double2* q = reinterpret_cast<double2*>(p);
+  static __device__ __forceinline__ void store_avg(double* p, size_t c, const double r[4]) {
+    double2* q = reinterpret_cast<double2*>(p + c * kRec);
     q[0] = make_double2(r[0], r[1]);
     q[1] = make_double2(r[2], r[3]);
   }
+};
+template <> struct Lay<float> {
+  static __host__ __device__ __forceinline__ size_t u(const Geo& g, int v, int i, int j) { return 4 * cell_at(g, i, j) + v; }
+  static __host__ __device__ __forceinline__ size_t w(size_t n, int v, int p, size_t o) { return 4 * (p * n + o) + v; }
+  static __host__ __device__ __forceinline__ size_t f(size_t, int v, size_t o) { return 4 * o + v; }
+  static __device__ __forceinline__ void get(const float* p, size_t k, float o[4]) {
+    const float4 t = reinterpret_cast<const float4*>(p)[k];
+    o[0] = t.x; o[1] = t.y; o[2] = t.z; o[3] = t.w;
+  }
+  static __device__ __forceinline__ void put(float* p, size_t k, const float o[4]) {
+    reinterpret_cast<float4*>(p)[k] = make_float4(o[0], o[1], o[2], o[3]);
+  }
+  static __device__ __forceinline__ void load_u(const Geo& g, const float* p, int i, int j, float o[4]) { get(p, cell_at(g, i, j), o); }
+  static __device__ __forceinline__ void load_w(const float* p, size_t n, int q, size_t o, float x[4]) { get(p, q * n + o, x); }
+  static __device__ __forceinline__ void load_f(const float* p, size_t, size_t o, float x[4]) { get(p, o, x); }
+  static __device__ __forceinline__ void store_w(float* p, size_t n, int q, size_t o, const float x[4]) { put(p, q * n + o, x); }
+  static __device__ __forceinline__ void store_f(float* p, size_t, size_t o, const float x[4]) { put(p, o, x); }
+  static __device__ __forceinline__ void load_rec(const float* p, size_t c, float r[kRec]) {
+#pragma unroll
+    for (int k = 0; k < kRec / 4; ++k) get(p, c * (kRec / 4) + k, r + 4 * k);
+  }
+  static __device__ __forceinline__ void load_avg(const float* p, size_t c, float r[4]) { get(p, c * (kRec / 4), r); }
+  static __device__ __forceinline__ void store_rec(float* p, size_t c, const float r[kRec]) {
+#pragma unroll
+    for (int k = 0; k < kRec / 4; ++k) put(p, c * (kRec / 4) + k, r + 4 * k);
+  }
+  static __device__ __forceinline__ void store_avg(float* p, size_t c, const float r[4]) { put(p, c * (kRec / 4), r); }
 };
 
 // derived fields: sizes of the padded arrays, reciprocal cell sizes and FP32
@@ -196,34 +231,34 @@ template <> __device__ __forceinline__ float step_dt<float>(const Ctrl* c) { ret
 // into (get / set in FP64; put stores a compute-type value).  One allocation of 4 * plane doubles per buffer either way:
 //  * FP64 mode: four FP64 planes;
 //  * FP32-bulk mode: each average is an unevaluated sum hi + lo of two FP32
-//    numbers (a double-float pair), hi planes in the first half and lo planes
-//    in the second.  hi is the FP32 rounding of hi + lo, so the hi planes are
+//    numbers (a double-float pair), the hi vectors in the first half and the lo vectors
+//    in the second.  hi is the FP32 rounding of hi + lo, so the hi vectors are
 //    the FP32 cell averages every FP32 kernel reads.
 // view() is the compute-type array of the averages.
 // ---------------------------------------------------------------------------
 template <class R> struct Cells;
 template <> struct Cells<double> {
   double* p;
-  __device__ __forceinline__ double get(const Geo& g, int v, int i, int j) const { return p[ci(g, v, i, j)]; }
-  __device__ __forceinline__ void set(const Geo& g, int v, int i, int j, double w) const { p[ci(g, v, i, j)] = w; }
-  __device__ __forceinline__ void put(const Geo& g, int v, int i, int j, double w) const { p[ci(g, v, i, j)] = w; }
+  __device__ __forceinline__ double get(const Geo& g, int v, int i, int j) const { return p[Lay<double>::u(g, v, i, j)]; }
+  __device__ __forceinline__ void set(const Geo& g, int v, int i, int j, double w) const { p[Lay<double>::u(g, v, i, j)] = w; }
+  __device__ __forceinline__ void put(const Geo& g, int v, int i, int j, double w) const { p[Lay<double>::u(g, v, i, j)] = w; }
   __host__ __device__ __forceinline__ const double* view() const { return p; }
 };
 template <> struct Cells<float> {
-  float* p;  // hi planes; lo planes at p + 4 * plane
+  float* p;  // hi vectors; lo vectors at p + 4 * plane
   __device__ __forceinline__ double get(const Geo& g, int v, int i, int j) const {
-    const size_t o = ci(g, v, i, j);
+    const size_t o = Lay<float>::u(g, v, i, j);
     return (double)p[o] + (double)p[o + 4 * g.plane];
   }
   __device__ __forceinline__ void set(const Geo& g, int v, int i, int j, double w) const {
-    const size_t o = ci(g, v, i, j);
+    const size_t o = Lay<float>::u(g, v, i, j);
     const float hi = (float)w;
     p[o] = hi;
     p[o + 4 * g.plane] = (float)(w - (double)hi);
   }
   // a value known only in FP32 (ghost images): lo = 0
   __device__ __forceinline__ void put(const Geo& g, int v, int i, int j, float w) const {
-    const size_t o = ci(g, v, i, j);
+    const size_t o = Lay<float>::u(g, v, i, j);
     p[o] = w;
     p[o + 4 * g.plane] = 0.0f;
   }
@@ -242,6 +277,15 @@ __device__ __forceinline__ void df_add_product(float& hi, float& lo, float f, fl
   const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
   hi = s;
   lo = __fadd_rn(lo, __fadd_rn(e, pe));
+}
+
+// value k of the caller's face-value planes [4][2][faces] to (to_dev) or from the layout of the type
+template <class TW>
+__device__ __forceinline__ void copy_w(const double* src, TW* W, size_t faces, size_t k, int to_dev) {
+  const size_t q = k / faces;
+  const size_t at = Lay<TW>::w(faces, (int)(q >> 1), (int)(q & 1), k - q * faces);
+  if (to_dev) W[at] = (TW)src[k];
+  else const_cast<double*>(src)[k] = (double)W[at];
 }
 
 // Programmatic dependent launch: a step kernel launched with programmatic stream
@@ -329,7 +373,7 @@ __device__ __forceinline__ void ghost_cell(const Geo& g, const R* U, int i, int 
   if (i < 0) { xs = 0; is = g.bc.kind[0] == GKS_BC_PERIODIC ? g.nx - 1 : 0; }
   if (i >= g.nx) { xs = 1; is = g.bc.kind[1] == GKS_BC_PERIODIC ? 0 : g.nx - 1; }
   R w[4], t[4];
-  for (int v = 0; v < 4; ++v) w[v] = U[ci(g, v, is, js)];
+  Lay<R>::load_u(g, U, is, js, w);
   if (ys >= 0) {
     bc_value<R>(g.bc.kind[ys], GeoR<R>::gamma(g), GeoR<R>::uwt(g, ys), GeoR<R>::Tw(g, ys), 1, w, t);
     for (int v = 0; v < 4; ++v) w[v] = t[v];
@@ -479,54 +523,33 @@ __device__ __forceinline__ void recon_vectors(const R in[13][4], const ReconK<R>
   }
 }
 
-template <class R, class TW, bool CHAR = false>
-__device__ __forceinline__ void recon_cell(const Geo& g, const R* __restrict__ U, const TW* __restrict__ Wx,
-                                           const TW* __restrict__ Wy, R* __restrict__ rec, int i, int j, R dx,
-                                           R dy, R weps, R wC) {
+// the record of cell (i, j)
+template <class R, bool CHAR = false>
+__device__ __forceinline__ void recon_record(const Geo& g, const R* __restrict__ U, const R* __restrict__ Wx,
+                                             const R* __restrict__ Wy, int i, int j, R dx, R dy, R weps, R wC,
+                                             R r[kRec]) {
   const int nx = g.nx, ny = g.ny;
   const size_t fxp = (size_t)ny * (nx + 1), fyp = (size_t)(ny + 1) * nx;
   const ReconK<R> K = recon_k(dx, dy, GeoR<R>::idx(g), GeoR<R>::idy(g), weps, wC);
   R a[4][5], cbar[4];
-  // stencil vector k of variable v: c, e, w, n, s; east face y-/y+, west y-/y+, north x-/x+,
-  // south x-/x+
-  auto load = [&](int v, R in[13]) {
-    const TW* wx = Wx + (size_t)v * 2 * fxp + (size_t)j * (nx + 1);
-    const TW* wy = Wy + (size_t)v * 2 * fyp;
-    in[0] = U[ci(g, v, i, j)];
-    in[1] = U[ci(g, v, i + 1, j)];
-    in[2] = U[ci(g, v, i - 1, j)];
-    in[3] = U[ci(g, v, i, j + 1)];
-    in[4] = U[ci(g, v, i, j - 1)];
-    in[5] = R(wx[i + 1]);
-    in[6] = R(wx[fxp + i + 1]);
-    in[7] = R(wx[i]);
-    in[8] = R(wx[fxp + i]);
-    in[9] = R(wy[(size_t)(j + 1) * nx + i]);
-    in[10] = R(wy[fyp + (size_t)(j + 1) * nx + i]);
-    in[11] = R(wy[(size_t)j * nx + i]);
-    in[12] = R(wy[fyp + (size_t)j * nx + i]);
-  };
-  if constexpr (CHAR) {
-    R in[13][4];
+  // stencil vector k: c, e, w, n, s; east face y-/y+, west y-/y+, north x-/x+, south x-/x+
+  const size_t ox = (size_t)j * (nx + 1) + i, oy = (size_t)j * nx + i;
+  R in[13][4];
+  Lay<R>::load_u(g, U, i, j, in[0]);
+  Lay<R>::load_u(g, U, i + 1, j, in[1]);
+  Lay<R>::load_u(g, U, i - 1, j, in[2]);
+  Lay<R>::load_u(g, U, i, j + 1, in[3]);
+  Lay<R>::load_u(g, U, i, j - 1, in[4]);
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      R t[13];
-      load(v, t);
-#pragma unroll
-      for (int k = 0; k < 13; ++k) in[k][v] = t[k];
-      cbar[v] = t[0];
-    }
-    recon_vectors<true, R>(in, K, GeoR<R>::gm1(g), GeoR<R>::gamma(g), a);
-  } else {
-    // one variable at a time: only its 13 stencil values are live
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      R t[13];
-      load(v, t);
-      cbar[v] = t[0];
-      recon_var<R>(t[0], t[1], t[2], t[3], t[4], t[5], t[6], t[7], t[8], t[9], t[10], t[11], t[12], K, a[v]);
-    }
+  for (int p = 0; p < 2; ++p) {
+    Lay<R>::load_w(Wx, fxp, p, ox + 1, in[5 + p]);
+    Lay<R>::load_w(Wx, fxp, p, ox, in[7 + p]);
+    Lay<R>::load_w(Wy, fyp, p, oy + nx, in[9 + p]);
+    Lay<R>::load_w(Wy, fyp, p, oy, in[11 + p]);
   }
+#pragma unroll
+  for (int v = 0; v < 4; ++v) cbar[v] = in[0][v];
+  recon_vectors<CHAR, R>(in, K, GeoR<R>::gm1(g), GeoR<R>::gamma(g), a);
   // the polynomial at the four face centres (x = +-dx/2, y = 0 and x = 0, y = +-dy/2):
   // value = e0 +- a2 dx/2 on x-faces, n0 +- a3 dy/2 on y-faces
   R ve[4], vw[4], vn[4], vs[4];
@@ -545,21 +568,32 @@ __device__ __forceinline__ void recon_cell(const Geo& g, const R* __restrict__ U
   // else the constant average
   auto ok = [](const R w[4]) { return w[0] > R(0) && R(2) * w[0] * w[3] > w[1] * w[1] + w[2] * w[2]; };
   const bool bad = !(ok(ve) && ok(vw) && ok(vn) && ok(vs));
-  R r[kRec];
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     r[v] = cbar[v];
 #pragma unroll
     for (int k = 0; k < 5; ++k) r[4 + 4 * k + v] = bad ? R(0) : a[v][k];
   }
-  RecIO<R>::store(rec + ri(g, i, j), r);
-  // the ghost ring's averages (boundary images written by the last update)
+}
+
+// the ghost records' averages that are boundary images of cell (i, j) (written by the last update)
+template <class R>
+__device__ __forceinline__ void ghost_records(const Geo& g, const R* __restrict__ U, R* __restrict__ rec, int i, int j) {
   for_each_ghost_of(g, i, j, [&](int gi, int gj) {
     R w[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) w[v] = U[ci(g, v, gi, gj)];
-    RecIO<R>::store_avg(rec + ri(g, gi, gj), w);
+    Lay<R>::load_u(g, U, gi, gj, w);
+    Lay<R>::store_avg(rec, rec_at(g, gi, gj), w);
   });
+}
+
+template <class R, bool CHAR = false>
+__device__ __forceinline__ void recon_cell(const Geo& g, const R* __restrict__ U, const R* __restrict__ Wx,
+                                           const R* __restrict__ Wy, R* __restrict__ rec, int i, int j, R dx,
+                                           R dy, R weps, R wC) {
+  R r[kRec];
+  recon_record<R, CHAR>(g, U, Wx, Wy, i, j, dx, dy, weps, wC, r);
+  Lay<R>::store_rec(rec, rec_at(g, i, j), r);
+  ghost_records(g, U, rec, i, j);
 }
 
 // Reconstruction of cell (i, j) in FP64 and conservative variables by four neighbouring lanes, one
@@ -576,7 +610,7 @@ __device__ __forceinline__ void recon_cell_lanes(const Geo& g, const double* __r
   const double* wx = Wx + (size_t)v * 2 * fxp + (size_t)j * (nx + 1) + i;
   const double* ws = Wy + (size_t)v * 2 * fyp + (size_t)j * nx + i;
   const double* wn = ws + nx;
-  const double* u = U + ci(g, v, i, j);
+  const double* u = U + Lay<double>::u(g, v, i, j);
   const double c = u[0];
   double a[5];
   recon_var_scaled(c, u[1], u[-1], u[g.pitch], u[-g.pitch], wx[1], wx[fxp + 1], wx[0], wx[fxp], wn[0], wn[fyp], ws[0],
@@ -600,13 +634,13 @@ __device__ __forceinline__ void recon_cell_lanes(const Geo& g, const double* __r
   }
   const bool bad = !__shfl_sync(0xffffffffu, (int)ok, 0, 4);
   if (!active) return;
-  double* r = rec + ri(g, i, j) + v;
+  double* r = rec + rec_at(g, i, j) * kRec + v;
   const double scale[5] = {g.idx, g.idy, g.idx2, g.idy2, g.idxy};
   r[0] = c;
 #pragma unroll
   for (int k = 0; k < 5; ++k) r[4 + 4 * k] = bad ? 0.0 : scale[k] * a[k];
   // the ghost ring's averages (boundary images written by the last update)
-  for_each_ghost_of(g, i, j, [&](int gi, int gj) { rec[ri(g, gi, gj) + v] = U[ci(g, v, gi, gj)]; });
+  for_each_ghost_of(g, i, j, [&](int gi, int gj) { rec[rec_at(g, gi, gj) * kRec + v] = U[Lay<double>::u(g, v, gi, gj)]; });
 }
 
 // ---------------------------------------------------------------------------
@@ -621,7 +655,7 @@ template <int AX, class R>
 __device__ __forceinline__ void side_state(const Geo& g, const R* __restrict__ rec, int i, int j, int s, R hn,
                                            R hn2_12, R ht2_24, FaceState<R>& S) {
   R r[kRec];
-  RecIO<R>::load(rec + ri(g, i, j), r);
+  Lay<R>::load_rec(rec, rec_at(g, i, j), r);
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     const R c = r[v];
@@ -664,7 +698,7 @@ struct GridFaceSource {
   __device__ __forceinline__ void const_state(int n, FaceState<R>& S) const {
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
-      S.w[0][slot<AX>(v)] = U[ci(*g, v, cx(n), cy(n))];
+      S.w[0][slot<AX>(v)] = U[Lay<R>::u(*g, v, cx(n), cy(n))];
 #pragma unroll
       for (int d = 1; d < 6; ++d) S.w[d][v] = R(0);
     }
@@ -719,7 +753,7 @@ struct GridFaceSource {
         const int ii = AX == 0 ? i - 1 + m : i - 1 + k;
         const int jj = AX == 0 ? j - 1 + k : j - 1 + m;
         R w[4];
-        RecIO<R>::load_avg(rec + ri(*g, ii, jj), w);
+        Lay<R>::load_avg(rec, rec_at(*g, ii, jj), w);
 #pragma unroll
         for (int v = 0; v < 4; ++v) a[m][k][slot<AX>(v)] = w[v];
       }
@@ -803,13 +837,16 @@ __device__ __forceinline__ void store_face(const Geo& g, const GridFaceSource<AX
   else if (src.img_hi) wall_face_flux<R>(src.img_hi, src.uwt_hi, Fl);
   const int fx = AX == 0 ? g.nx + 1 : g.nx, fy = AX == 0 ? g.ny : g.ny + 1;
   const size_t nfaces = (size_t)fx * fy, o = (size_t)src.j * fx + src.i;
+  R f[4], m[4], p[4];
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
-    const int k = slot<AX>(v);
-    F[(size_t)v * nfaces + o] = Fl[k];
-    Wn[(size_t)(v * 2 + 0) * nfaces + o] = TW(Wm[k]);
-    Wn[(size_t)(v * 2 + 1) * nfaces + o] = TW(Wp[k]);
+    f[v] = Fl[slot<AX>(v)];
+    m[v] = Wm[slot<AX>(v)];
+    p[v] = Wp[slot<AX>(v)];
   }
+  Lay<R>::store_f(F, nfaces, o, f);
+  Lay<R>::store_w(Wn, nfaces, 0, o, m);
+  Lay<R>::store_w(Wn, nfaces, 1, o, p);
 }
 
 // the evolution at face (i, j) of axis AX: flux F and new point values Wn
@@ -999,16 +1036,19 @@ template <> struct CellState<double> { double w[4]; };
 template <> struct CellState<float> { float hi[4], lo[4]; };
 
 __device__ __forceinline__ void load_state(const Geo& g, Cells<double> U, int i, int j, CellState<double>& s) {
-#pragma unroll
-  for (int v = 0; v < 4; ++v) s.w[v] = U.p[ci(g, v, i, j)];
+  Lay<double>::load_u(g, U.p, i, j, s.w);
 }
 __device__ __forceinline__ void load_state(const Geo& g, Cells<float> U, int i, int j, CellState<float>& s) {
+  Lay<float>::load_u(g, U.p, i, j, s.hi);
+  Lay<float>::load_u(g, U.p + 4 * g.plane, i, j, s.lo);
+}
+__device__ __forceinline__ void store_state(const Geo& g, Cells<double> U, int i, int j, const CellState<double>& s) {
 #pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    const size_t o = ci(g, v, i, j);
-    s.hi[v] = U.p[o];
-    s.lo[v] = U.p[o + 4 * g.plane];
-  }
+  for (int v = 0; v < 4; ++v) U.p[Lay<double>::u(g, v, i, j)] = s.w[v];
+}
+__device__ __forceinline__ void store_state(const Geo& g, Cells<float> U, int i, int j, const CellState<float>& s) {
+  Lay<float>::put(U.p, cell_at(g, i, j), s.hi);
+  Lay<float>::put(U.p + 4 * g.plane, cell_at(g, i, j), s.lo);
 }
 
 // Eq. finite for one variable: FP64 planes take the FP32 or FP64 fluxes in
@@ -1017,17 +1057,13 @@ __device__ __forceinline__ void load_state(const Geo& g, Cells<float> U, int i, 
 // Either way each face flux enters both neighbours with the same rounding, so
 // the sum over cells telescopes to roundoff of the accumulation type.
 template <class R>
-__device__ __forceinline__ R update_var(const Geo& g, const CellState<double>& S, Cells<double> Un, const R f[4][4], int v,
-                                        int i, int j, bool& finite) {
-  const size_t o = ci(g, v, i, j);
+__device__ __forceinline__ R update_var(const Geo& g, CellState<double>& S, const R f[4][4], int v, bool& finite) {
   const double w = S.w[v] + ((double)f[0][v] - (double)f[1][v]) * g.idx + ((double)f[2][v] - (double)f[3][v]) * g.idy;
-  Un.p[o] = w;
+  S.w[v] = w;
   finite = isfinite(w);
   return R(w);
 }
-__device__ __forceinline__ float update_var(const Geo& g, const CellState<float>& S, Cells<float> Un, const float f[4][4],
-                                            int v, int i, int j, bool& finite) {
-  const size_t o = ci(g, v, i, j), lo_off = 4 * g.plane;
+__device__ __forceinline__ float update_var(const Geo& g, CellState<float>& S, const float f[4][4], int v, bool& finite) {
   float hi = S.hi[v], lo = S.lo[v];
   df_add_product(hi, lo, f[0][v], g.idx_hi, g.idx_lo);
   df_add_product(hi, lo, -f[1][v], g.idx_hi, g.idx_lo);
@@ -1037,8 +1073,8 @@ __device__ __forceinline__ float update_var(const Geo& g, const CellState<float>
   const float s = __fadd_rn(hi, lo);
   lo = __fsub_rn(lo, __fsub_rn(s, hi));
   hi = s;
-  Un.p[o] = hi;
-  Un.p[o + lo_off] = lo;
+  S.hi[v] = hi;
+  S.lo[v] = lo;
   finite = isfinite(hi) && isfinite(lo);
   return hi;
 }
@@ -1060,13 +1096,10 @@ __device__ __forceinline__ R update_cell(const Geo& g, Cells<R> U, Cells<R> Un, 
   const R* Ur = U.view();
   // the four face fluxes: west, east, south, north
   R f[4][4];
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    f[0][v] = Fx[v * nfx + (size_t)j * (nx + 1) + i];
-    f[1][v] = Fx[v * nfx + (size_t)j * (nx + 1) + i + 1];
-    f[2][v] = Fy[v * nfy + (size_t)j * nx + i];
-    f[3][v] = Fy[v * nfy + (size_t)(j + 1) * nx + i];
-  }
+  Lay<R>::load_f(Fx, nfx, (size_t)j * (nx + 1) + i, f[0]);
+  Lay<R>::load_f(Fx, nfx, (size_t)j * (nx + 1) + i + 1, f[1]);
+  Lay<R>::load_f(Fy, nfy, (size_t)j * nx + i, f[2]);
+  Lay<R>::load_f(Fy, nfy, (size_t)(j + 1) * nx + i, f[3]);
   CellState<R> S;
   load_state(g, U, i, j, S);
   if (pass > 1) {
@@ -1091,11 +1124,8 @@ __device__ __forceinline__ R update_cell(const Geo& g, Cells<R> U, Cells<R> Un, 
         TW* Wn = x ? Wxn : Wyn;
         const size_t nf = x ? nfx : nfy;
         const size_t o = x ? (size_t)fj * (nx + 1) + fi : (size_t)fj * nx + fi;
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          Wn[(size_t)(v * 2 + 0) * nf + o] = TW(W[v]);
-          Wn[(size_t)(v * 2 + 1) * nf + o] = TW(W[v]);
-        }
+        Lay<R>::store_w(Wn, nf, 0, o, W);
+        Lay<R>::store_w(Wn, nf, 1, o, W);
       }
     }
   }
@@ -1104,9 +1134,10 @@ __device__ __forceinline__ R update_cell(const Geo& g, Cells<R> U, Cells<R> Un, 
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     bool fv;
-    wr[v] = update_var(g, S, Un, f, v, i, j, fv);
+    wr[v] = update_var(g, S, f, v, fv);
     finite = finite && fv;
   }
+  store_state(g, Un, i, j, S);
   ghosts_of_cell<R>(g, Un, i, j);
   bool ok;
   R inv = inv_bound<R>(g, wr, ok);
