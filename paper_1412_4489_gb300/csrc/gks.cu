@@ -1,19 +1,20 @@
 // GB300 (sm_103a) kernels and C ABI of the compact third-order gas-kinetic
 // scheme (Pan & Xu, arXiv:1412.4489).  See include/gks.h for the interface.
 //
-// One step = seven launches on the handle's stream, all reading a device-resident
+// One step = four or five launches on the handle's stream, all reading a device-resident
 // control block so that the sequence can be captured once in a CUDA graph:
 //   k_recon    dt = min(CFL * dt_cfl, dt_max, t_end - t) from the running min
 //              (block 0), and the compact reconstruction of every cell (Section 3.2)
-//   k_flux<0>  gas evolution at every x-face (Section 2.2, 3.3, 4)
-//   k_flux<1>  gas evolution at every y-face (frame rotated: n = y, t = x)
-//              (FP64: both axes in one launch, k_faces or k_faces_split)
+//              (FP64 in conservative variables: k_recon_lanes)
+//   faces      gas evolution at every x-face and y-face (frame rotated: n = y, t = x; Section 2.2, 3.3, 4):
+//              FP64 k_faces or k_faces_split, FP32 Euler k_flux_euler, FP32 Navier-Stokes
+//              k_flux<0> and k_flux<1> on two streams
 //   k_update   conservative update (Eq. finite) into FP64 averages, or in
 //              FP32-bulk mode into double-float (hi + lo FP32) averages, the
 //              ghost cells that are images of the updated cells, the next CFL
-//              bound (warp-shuffle / block / atomic min) and the physical check;
-//              three passes, the second and third only for the positivity fallback
-//   k_end      advance t and the step counter
+//              bound (warp-shuffle / block / atomic min) and the physical check
+//   k_finish   the update's second and third pass, only for the positivity fallback; advances t and
+//              the step counter
 // The ghost ring of a newly set state is filled by k_ghost.
 // Cell averages and face values are double-buffered; the buffer in use is the
 // parity of the device step counter, so a failed step leaves the last good
@@ -35,15 +36,7 @@ using namespace gks;
 
 namespace {
 
-constexpr int kLaunchesPerStep = 7;
-
-// ---------------------------------------------------------------------------
-// control kernels
-// ---------------------------------------------------------------------------
-__global__ void k_end(Ctrl* c) {
-  pdl_enter();
-  ctrl_end(c);
-}
+constexpr int kProfileParts = 7;  // gks_profile_step's times: the fallback passes' and the end's are one kernel's
 
 // ---------------------------------------------------------------------------
 // ghost ring: perimeter of the padded cell array of the current buffer
@@ -145,16 +138,16 @@ __global__ void __launch_bounds__(32, 16) k_recon_lanes(Geo g, const double* U0,
 // face evolution
 // ---------------------------------------------------------------------------
 // resident 128-thread blocks per SM the FP32 face kernel is compiled for: Euler 5 (96 registers,
-// 20 warps per SM; 16-52 bytes of spill), Navier-Stokes 4 (128 registers; at 96 it spills 100-144 bytes).
-// x-faces at 2048^2, 4 / 5 blocks: Euler 222 / 207 us; Navier-Stokes at 1024^2 79.5 / 80.4 us.  6 blocks (80
+// 20 warps per SM; 4 bytes of spill), Navier-Stokes 4 (128 registers; at 96 it spills 100-144 bytes).
+// x-faces at 2048^2, 4 / 5 blocks: Euler 222 / 207 us (195 with fewer spills); Navier-Stokes at 1024^2 79.5 / 80.4 us.  6 blocks (80
 // registers) are slower for both, 3 slower for Navier-Stokes.
 template <int NS> struct FluxBlocks { static constexpr int value = NS ? 4 : 5; };
 
-// NS: Navier-Stokes (1) or Euler (0) face routine, chosen per grid by flux_kernel
-template <int AX, class R, class TW, int NS>
-__global__ void __launch_bounds__(128, FluxBlocks<NS>::value) k_flux(Geo g, FaceConst<R> C, const R* __restrict__ rec,
-                                                                    TW* Wn0, TW* Wn1, R* __restrict__ F,
-                                                                    const Ctrl* c, int force) {
+// Navier-Stokes faces of one axis (FP32)
+template <int AX, class R, class TW>
+__global__ void __launch_bounds__(128, FluxBlocks<1>::value) k_flux(Geo g, FaceConst<R> C, const R* __restrict__ rec,
+                                                                   TW* Wn0, TW* Wn1, R* __restrict__ F,
+                                                                   const Ctrl* c, int force) {
   pdl_enter();
   if (!force && c->skip) return;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -170,20 +163,9 @@ __global__ void __launch_bounds__(128, FluxBlocks<NS>::value) k_flux(Geo g, Face
   if (i >= fx || j >= fy) return;
   const int par = (int)(c->steps & 1);
   // new face values go to the other buffer
-  flux_face<AX, R, TW, NS>(g, C, rec, par ? Wn0 : Wn1, F, i, j, step_dt<R>(c));
+  flux_face<AX, R, TW, 1>(g, C, rec, par ? Wn0 : Wn1, F, i, j, step_dt<R>(c));
 }
 
-template <int AX, class R, class TW>
-auto flux_kernel(const Geo& g) -> decltype(&k_flux<AX, R, TW, 1>) {
-  return g.mu > 0.0 ? &k_flux<AX, R, TW, 1> : &k_flux<AX, R, TW, 0>;
-}
-
-// FP64: every face of the grid in one launch, 32 to a block, x-faces in blocks [0, nbx), y-faces after
-// them, numbered through row by row.  The FP64 pipe serves a warp instruction for a quarter of an SM in 64 cycles
-// whether its lanes are active or not, so what counts is full warps spread evenly over the quarters: one-warp
-// blocks without idle lanes at the rows' ends, and no second launch with a tail of its own.  (Instruction fetch,
-// which speaks against mixing the two axes' bodies in FP32, does not matter at this pace.)
-// first: the first block's number (a launch can take one axis alone).
 template <class R, class TW>
 struct FaceArgs {
   FaceConst<R> Cx, Cy;
@@ -193,6 +175,39 @@ struct FaceArgs {
   unsigned nbx, first;
 };
 
+// FP32 Euler faces of both axes in one launch: blocks [0, nbx) take x-faces, the others y-faces, 32 x 4 to a
+// block in tiles (tx tiles to a row); with nx a multiple of 32 the x-tiles' last column as in k_flux.  No second stream to
+// fork to and join: 48^2 12.2 -> 10.9 us a step, 512^2 44.6 -> 43.8, from 1024^2 on the same.  (Navier-Stokes faces stay two
+// kernels on two streams: mixing the larger bodies costs 2% at 1024^2.)
+__global__ void __launch_bounds__(128, FluxBlocks<0>::value) k_flux_euler(Geo g, FaceArgs<float, float> a, const Ctrl* c, int force) {
+  pdl_enter();
+  if (!force && c->skip) return;
+  const int par = (int)(c->steps & 1);
+  const float dt = step_dt<float>(c);
+  const unsigned b = blockIdx.x + a.first, tx = (unsigned)(g.nx + 31) / 32, ny4 = (unsigned)(g.ny + 3) / 4;
+  if (b < a.nbx) {
+    int i, j;
+    if (b < tx * ny4) {
+      i = (int)(b % tx) * 32 + threadIdx.x;
+      j = (int)(b / tx) * 4 + threadIdx.y;
+    } else {  // the last faces of 128 rows
+      i = g.nx;
+      j = (int)(b - tx * ny4) * 128 + threadIdx.y * 32 + threadIdx.x;
+    }
+    if (i <= g.nx && j < g.ny) flux_face<0, float, float, 0>(g, a.Cx, a.rec, par ? a.Wx0 : a.Wx1, a.Fx, i, j, dt);
+  } else {
+    const unsigned q = b - a.nbx;
+    const int i = (int)(q % tx) * 32 + threadIdx.x, j = (int)(q / tx) * 4 + threadIdx.y;
+    if (i < g.nx && j <= g.ny) flux_face<1, float, float, 0>(g, a.Cy, a.rec, par ? a.Wy0 : a.Wy1, a.Fy, i, j, dt);
+  }
+}
+
+// FP64: every face of the grid in one launch, 32 to a block, x-faces in blocks [0, nbx), y-faces after
+// them, numbered through row by row.  The FP64 pipe serves a warp instruction for a quarter of an SM in 64 cycles
+// whether its lanes are active or not, so what counts is full warps spread evenly over the quarters: one-warp
+// blocks without idle lanes at the rows' ends, and no second launch with a tail of its own.  (Instruction fetch,
+// which speaks against mixing the two axes' bodies in FP32, does not matter at this pace.)
+// first: the first block's number (a launch can take one axis alone).
 template <int AX>
 __device__ __forceinline__ bool face_at(const Geo& g, unsigned block, int lane, int& i, int& j) {
   const unsigned fx = AX == 0 ? g.nx + 1 : g.nx, fy = AX == 0 ? g.ny : g.ny + 1;
@@ -260,11 +275,15 @@ template <> struct UpdateBlocks<double> { static constexpr int value = 2; };
 template <> struct UpdateBlocks<float> { static constexpr int value = 4; };
 
 template <class R, class TW>
-__global__ void __launch_bounds__(256, UpdateBlocks<R>::value) k_update(Geo g, Cells<R> U0, Cells<R> U1, const R* __restrict__ Fx,
-                                                const R* __restrict__ Fy, TW* Wx0, TW* Wx1, TW* Wy0, TW* Wy1,
-                                                unsigned char* __restrict__ bad, Ctrl* c, int pass) {
-  pdl_enter();
-  if (c->skip || (pass == 2 && !c->bad_found[0]) || (pass == 3 && !c->bad_found[1])) return;
+struct UpdateArgs {
+  Cells<R> U0, U1;
+  const R *Fx, *Fy;
+  TW *Wx0, *Wx1, *Wy0, *Wy1;
+  unsigned char* bad;
+};
+
+template <class R, class TW>
+__device__ __forceinline__ void update_pass(const Geo& g, const UpdateArgs<R, TW>& a, Ctrl* c, int pass) {
   const int par = (int)(c->steps & 1);
   R inv_max = R(0);  // over the block's tiles: one block reduction per block
   for (int j0 = blockIdx.y * blockDim.y; j0 < g.ny; j0 += gridDim.y * blockDim.y) {
@@ -273,10 +292,10 @@ __global__ void __launch_bounds__(256, UpdateBlocks<R>::value) k_update(Geo g, C
       R inv = R(0);
       if (i < g.nx && j < g.ny) {
         bool b;
-        inv = update_cell<R, TW>(g, par ? U1 : U0, par ? U0 : U1, Fx, Fy, par ? Wx0 : Wx1, par ? Wy0 : Wy1, bad, pass,
-                                 step_dt<R>(c), i, j, b);
+        inv = update_cell<R, TW>(g, par ? a.U1 : a.U0, par ? a.U0 : a.U1, a.Fx, a.Fy, par ? a.Wx0 : a.Wx1,
+                                 par ? a.Wy0 : a.Wy1, a.bad, pass, step_dt<R>(c), i, j, b);
         if (pass == 1) {
-          bad[(size_t)j * g.nx + i] = b ? 1 : 0;
+          a.bad[(size_t)j * g.nx + i] = b ? 1 : 0;
           if (b) atomicOr(&c->bad_found[0], 1);
         } else if (pass == 2) {
           if (b) atomicOr(&c->bad_found[1], 1);
@@ -290,10 +309,69 @@ __global__ void __launch_bounds__(256, UpdateBlocks<R>::value) k_update(Geo g, C
   block_bound_to<R>(inv_max, &c->dtb[pass - 1]);
 }
 
-// launch grid of an update pass in tiles of 32 x rows cells: pass 1 takes one wave of resident
+template <class R, class TW>
+__global__ void __launch_bounds__(256, UpdateBlocks<R>::value) k_update(Geo g, UpdateArgs<R, TW> a, Ctrl* c) {
+  pdl_enter();
+  if (c->skip) return;
+  update_pass<R, TW>(g, a, c, 1);
+}
+
+// Barrier of all blocks of a cooperative launch; bounded: a block that waits longer than two seconds
+// fails the step (GKS_ETIMEOUT) and returns false, as do the others.
+__device__ bool ctrl_barrier(Ctrl* c) {
+  __syncthreads();
+  __shared__ int ok;
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    volatile unsigned* gen = &c->bar_gen;
+    volatile int* status = &c->status;
+    const unsigned my = *gen;
+    __threadfence();
+    if (atomicAdd(&c->bar_count, 1u) + 1 == gridDim.x * gridDim.y) {
+      c->bar_count = 0;
+      __threadfence();
+      atomicAdd(&c->bar_gen, 1u);
+    }
+    unsigned long long t0, t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+    while (*gen == my && *status != GKS_ETIMEOUT) {
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+      if (t - t0 > 2000000000ull) atomicExch(&c->status, GKS_ETIMEOUT);
+      __nanosleep(200);
+    }
+    __threadfence();
+    ok = *gen != my;
+  }
+  __syncthreads();
+  return ok;
+}
+
+// Passes 2 and 3, when they are needed, and the step's end: one cooperative launch of at most one wave, whose blocks
+// meet at a barrier after each pass.  Usually there is no work and the first thread ends the step.  In
+// place of three launches (two passes, the end): 64^2 FP32 14.2 -> 12.2 us a step, 512^2 48.2 -> 44.3, 200 x 1
+// FP64 39.5 -> 35.6; with programmatic serialisation as well as the cooperative attribute (without:
+// 12.8, 47.2, 35.5).
+template <class R, class TW>
+__global__ void __launch_bounds__(256, UpdateBlocks<R>::value) k_finish(Geo g, UpdateArgs<R, TW> a, Ctrl* c) {
+  pdl_enter();
+  const bool first = blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0;
+  if (c->skip) return;
+  if (!c->bad_found[0]) {
+    if (first) ctrl_end(c);
+    return;
+  }
+  update_pass<R, TW>(g, a, c, 2);
+  if (!ctrl_barrier(c)) return;
+  if (*(volatile int*)&c->bad_found[1]) {
+    update_pass<R, TW>(g, a, c, 3);
+    if (!ctrl_barrier(c)) return;
+  }
+  if (first) ctrl_end(c);
+}
+
+// launch grid of an update in tiles of 32 x rows cells: pass 1 takes one wave of resident
 // blocks (blocks_per_sm per SM), each walking ceil(tiles / wave) tiles along y, so
 // that the per-block work (control reads, the CFL reduction) is shared by its tiles;
-// the fallback passes at most 8 x (SMs / 2) blocks (usually no work).  Pass 1 of the FP64 form takes
+// the fallback passes at most one block per SM (usually no work).  Pass 1 of the FP64 form takes
 // one-warp blocks (rows = 1): its bound is the FP64 pipe, which wants the warps of a small grid spread over all SMs
 // (81^2 in 256-thread blocks keeps 33 of 152 SMs busy).
 constexpr int kUpdateRows = 8;
@@ -301,15 +379,15 @@ template <class R> constexpr int update_rows(int pass) { return pass == 1 && siz
 
 dim3 update_grid(const Geo& g, int pass, int sms, int blocks_per_sm, int rows) {
   unsigned tx = (unsigned)((g.nx + 31) / 32), ty = (unsigned)((g.ny + rows - 1) / rows);
-  if (pass == 1 && sms > 0) {
+  if (pass == 1) {
     const unsigned wave = (unsigned)sms * (unsigned)(blocks_per_sm * (kUpdateRows / rows));
     const unsigned fit = wave / tx > 0 ? wave / tx : 1;  // block rows that fit in one wave
     const unsigned k = (ty + fit - 1) / fit;             // tiles per block
     ty = (ty + k - 1) / k;
   }
   if (pass > 1) {
-    const unsigned cy = (unsigned)(sms > 1 ? sms / 2 : 76);
     if (tx > 8) tx = 8;
+    const unsigned cy = (unsigned)(sms / (int)tx > 0 ? sms / (int)tx : 1);
     if (ty > cy) ty = cy;
   }
   return dim3(tx, ty);
@@ -500,6 +578,28 @@ void launch_ghost(gks_handle* h, int force) {
 }
 
 template <class R, class TW>
+cudaError_t launch_update(bool pdl, cudaStream_t s, const Geo& g, int sms, const UpdateArgs<R, TW>& a, Ctrl* c) {
+  const int rows = update_rows<R>(1);
+  return launch(pdl, k_update<R, TW>, update_grid(g, 1, sms, UpdateBlocks<R>::value, rows), dim3(32, rows), s, g, a, c);
+}
+
+template <class R, class TW>
+cudaError_t launch_finish(cudaStream_t s, const Geo& g, int sms, const UpdateArgs<R, TW>& a, Ctrl* c) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = update_grid(g, 2, sms, 1, kUpdateRows);
+  cfg.blockDim = dim3(32, kUpdateRows);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, k_finish<R, TW>, g, a, c);
+}
+
+template <class R, class TW>
 cudaError_t launch_recon(bool pdl, cudaStream_t s, const Geo& g, const R* U0, const R* U1, const TW* Wx0, const TW* Wx1,
                          const TW* Wy0, const TW* Wy1, R* rec, Ctrl* c, int force, int begin, double cfl, double dt_max,
                          double t_end) {
@@ -541,7 +641,7 @@ cudaError_t launch_faces(bool pdl, cudaStream_t s, const Geo& g, int sms, const 
   return launch(pdl, ns ? k_faces<R, TW, 1> : k_faces<R, TW, 0>, dim3(n), dim3(32), s, g, a, c, force);
 }
 
-// ev (optional, kLaunchesPerStep + 1 events): recorded before each kernel and after the last.
+// ev (optional, kProfileParts + 1 events): recorded before each kernel and after the last.
 // with_begin_end = false (face evaluation of the current state for gks_debug_flux):
 // the ghost ring is refreshed first and the step is neither opened nor closed.
 template <class R, class TW>
@@ -577,36 +677,54 @@ gks_status launch_step_kernels(gks_handle* h, double cfl, double dt_max, double 
     // the x- and y-face evolutions are independent: without per-kernel timing the y-faces run
     // on a side stream (fork after the reconstruction, join before the update), so that each
     // fills the other's tail wave
-    fork = ev == nullptr;
-    if (fork) {
-      keep(cudaEventRecord(h->fork, s));
-      keep(cudaStreamWaitEvent(h->side, h->fork, 0));
-      keep(launch(false, flux_kernel<1, R, TW>(g), grid2(g.nx, g.ny + 1, bf), bf, h->side, g, fconst<R>(g, 1),
-                  (const R*)h->rec, (TW*)h->Wy[0], (TW*)h->Wy[1], (R*)h->Fy, (const Ctrl*)h->ctrl, force));
-      keep(cudaEventRecord(h->join, h->side));
-    }
-    keep(launch(pdl, flux_kernel<0, R, TW>(g), grid2(g.nx + 1, g.ny, bf), bf, s, g, fconst<R>(g, 0), (const R*)h->rec,
-                (TW*)h->Wx[0], (TW*)h->Wx[1], (R*)h->Fx, (const Ctrl*)h->ctrl, force));
-    mark(2);
-    if (fork) {
-      keep(cudaStreamWaitEvent(s, h->join, 0));
+    if (g.mu > 0.0) {
+      // the x- and y-face evolutions are independent: without per-kernel timing the y-faces run
+      // on a side stream (fork after the reconstruction, join before the update), so that each
+      // fills the other's tail wave
+      fork = ev == nullptr;
+      auto yfaces = [&](bool p, cudaStream_t t) {
+        keep(launch(p, k_flux<1, R, TW>, grid2(g.nx, g.ny + 1, bf), bf, t, g, fconst<R>(g, 1), (const R*)h->rec,
+                    (TW*)h->Wy[0], (TW*)h->Wy[1], (R*)h->Fy, (const Ctrl*)h->ctrl, force));
+      };
+      if (fork) {
+        keep(cudaEventRecord(h->fork, s));
+        keep(cudaStreamWaitEvent(h->side, h->fork, 0));
+        yfaces(false, h->side);
+        keep(cudaEventRecord(h->join, h->side));
+      }
+      keep(launch(pdl, k_flux<0, R, TW>, grid2(g.nx + 1, g.ny, bf), bf, s, g, fconst<R>(g, 0), (const R*)h->rec,
+                  (TW*)h->Wx[0], (TW*)h->Wx[1], (R*)h->Fx, (const Ctrl*)h->ctrl, force));
+      mark(2);
+      if (fork) keep(cudaStreamWaitEvent(s, h->join, 0));
+      else yfaces(pdl, s);
     } else {
-      keep(launch(pdl, flux_kernel<1, R, TW>(g), grid2(g.nx, g.ny + 1, bf), bf, s, g, fconst<R>(g, 1),
-                  (const R*)h->rec, (TW*)h->Wy[0], (TW*)h->Wy[1], (R*)h->Fy, (const Ctrl*)h->ctrl, force));
+      const unsigned tx = (unsigned)(g.nx + 31) / 32, ny4 = (unsigned)(g.ny + 3) / 4;
+      const unsigned nbx = tx * ny4 + ((g.nx & 31) ? 0 : (unsigned)(g.ny + 127) / 128);
+      const unsigned nby = tx * ((unsigned)g.ny / 4 + 1);
+      auto faces = [&](int axes) {
+        const FaceArgs<R, TW> a{fconst<R>(g, 0), fconst<R>(g, 1), (const R*)h->rec, (TW*)h->Wx[0], (TW*)h->Wx[1],
+                                (TW*)h->Wy[0], (TW*)h->Wy[1], (R*)h->Fx, (R*)h->Fy, nbx, axes == 2 ? nbx : 0};
+        keep(launch(pdl, k_flux_euler, dim3((axes & 1 ? nbx : 0) + (axes & 2 ? nby : 0)), bf, s, g, a, (const Ctrl*)h->ctrl,
+                    force));
+      };
+      if (ev) faces(1);
+      mark(2);
+      faces(ev ? 2 : 3);
     }
   }
   mark(3);
-  for (int pass = 1; pass <= 3; ++pass) {
-    if (do_update)
-      // pass 1 follows the join (two predecessors): an ordinary launch
-      keep(launch(pdl && !(fork && pass == 1), k_update<R, TW>, update_grid(g, pass, h->sms, UpdateBlocks<R>::value, update_rows<R>(pass)),
-                  dim3(32, update_rows<R>(pass)), s, g,
-                  cellbuf<R>(h, 0), cellbuf<R>(h, 1),
-                  (const R*)h->Fx, (const R*)h->Fy, (TW*)h->Wx[0], (TW*)h->Wx[1], (TW*)h->Wy[0], (TW*)h->Wy[1],
-                  h->bad, h->ctrl, pass));
-    mark(3 + pass);
+  if (do_update) {
+    const UpdateArgs<R, TW> a{cellbuf<R>(h, 0), cellbuf<R>(h, 1), (const R*)h->Fx, (const R*)h->Fy, (TW*)h->Wx[0], (TW*)h->Wx[1],
+                              (TW*)h->Wy[0], (TW*)h->Wy[1], h->bad};
+    // after the join (two predecessors): an ordinary launch
+    keep(launch_update<R, TW>(pdl && !fork, s, g, h->sms, a, h->ctrl));
+    mark(4);
+    keep(launch_finish<R, TW>(s, g, h->sms, a, h->ctrl));
+  } else {
+    mark(4);
   }
-  if (with_begin_end) keep(launch(pdl, k_end, dim3(1), dim3(1), s, h->ctrl));
+  mark(5);
+  mark(6);
   mark(7);
   CK(le);
   CK(cudaGetLastError());
@@ -999,16 +1117,16 @@ const char* gks_last_error(const gks_handle* h) { return h ? h->err.c_str() : g_
 gks_status gks_profile_step(gks_handle* h, double CFL, float* ms) {
   if (!h || !ms || !(CFL > 0)) return fail(h, GKS_EINVAL, "gks_profile_step: CFL > 0 and ms[7] required");
   CK(cudaSetDevice(h->device));
-  cudaEvent_t ev[kLaunchesPerStep + 1];
-  for (int k = 0; k <= kLaunchesPerStep; ++k) CK(cudaEventCreate(&ev[k]));
+  cudaEvent_t ev[kProfileParts + 1];
+  for (int k = 0; k <= kProfileParts; ++k) CK(cudaEventCreate(&ev[k]));
   gks_status st = h->prec == GKS_FP64 ? launch_step_kernels<double, double>(h, CFL, INFINITY, INFINITY, true, true, 0, ev)
                                       : launch_step_kernels<float, float>(h, CFL, INFINITY, INFINITY, true, true, 0, ev);
   if (st == GKS_OK) {
-    cudaError_t e = cudaEventSynchronize(ev[kLaunchesPerStep]);
-    for (int k = 0; k < kLaunchesPerStep && e == cudaSuccess; ++k) e = cudaEventElapsedTime(&ms[k], ev[k], ev[k + 1]);
+    cudaError_t e = cudaEventSynchronize(ev[kProfileParts]);
+    for (int k = 0; k < kProfileParts && e == cudaSuccess; ++k) e = cudaEventElapsedTime(&ms[k], ev[k], ev[k + 1]);
     if (e != cudaSuccess) st = fail(h, GKS_ECUDA, std::string("gks_profile_step: ") + cudaGetErrorString(e));
   }
-  for (int k = 0; k <= kLaunchesPerStep; ++k) cudaEventDestroy(ev[k]);
+  for (int k = 0; k <= kProfileParts; ++k) cudaEventDestroy(ev[k]);
   if (st != GKS_OK) return st;
   st = read_ctrl(h);
   if (st != GKS_OK) return st;
@@ -1017,7 +1135,7 @@ gks_status gks_profile_step(gks_handle* h, double CFL, float* ms) {
 }
 
 int gks_launches_per_step(const gks_handle* h) {
-  return h && h->prec == GKS_FP64 ? kLaunchesPerStep - 1 : kLaunchesPerStep;  // FP64: both face axes in one
+  return h && h->prec == GKS_FP32_BULK && h->g.mu > 0.0 ? 5 : 4;  // reconstruction, faces, update, finish
 }
 
 gks_status gks_debug_recon(gks_handle* h, double* coef) {
@@ -1214,6 +1332,7 @@ __global__ void k_noalloc_ctrl(Ctrl* c) {
   c->bound = dbits(INFINITY);
   c->dtb[0] = c->dtb[1] = c->dtb[2] = dbits(INFINITY);
   c->bad_found[0] = c->bad_found[1] = 0;
+  c->bar_count = c->bar_gen = 0;
   c->t = 0.0;
   c->dt = 0.0;
   c->dt_f = 0.0f;
@@ -1298,11 +1417,10 @@ extern "C" gks_status gks_step_noalloc(int nx, int ny, double Lx, double Ly, dou
   e = launch_faces<double, double>(false, s, g, sms, rec, const_cast<double*>(dWx), dWx_out, const_cast<double*>(dWy),
                                    dWy_out, Fx, Fy, ctrl, 0);
   if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
-  for (int pass = 1; pass <= 3; ++pass)
-    k_update<double, double><<<update_grid(g, pass, sms, UpdateBlocks<double>::value, update_rows<double>(pass)),
-                               dim3(32, update_rows<double>(pass)), 0, s>>>(g, C0, C1, Fx, Fy, const_cast<double*>(dWx), dWx_out,
-                                                              const_cast<double*>(dWy), dWy_out, bad, ctrl, pass);
-  k_end<<<1, 1, 0, s>>>(ctrl);
+  const UpdateArgs<double, double> ua{C0, C1, Fx, Fy, const_cast<double*>(dWx), dWx_out, const_cast<double*>(dWy), dWy_out, bad};
+  e = launch_update<double, double>(false, s, g, sms, ua, ctrl);
+  if (e == cudaSuccess) e = launch_finish<double, double>(s, g, sms, ua, ctrl);
+  if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
   k_scatter_U<double><<<grid2(nx, ny, b2), b2, 0, s>>>(g, dU_out, C0, C1, ctrl, 0);
   e = cudaGetLastError();
   Ctrl hc;

@@ -223,15 +223,15 @@ GKS_FN void time_coef(R U, R V, R i2N, R kc, const R X[4], const R Y[4], R T[4])
   T[3] = -(U * X[3] + V * Y[3] + kc * (X[1] + Y[2]));
 }
 
-// Coefficient of the Maxwellian (scaled by rho) with central components e, in the basis
+// Coefficient of the Maxwellian (scaled by rho s, s = 1 / (2 lam)) with central components e, in the basis
 // (1, u, d, u^2/2 + eta), eta = (d^2 + xi^2)/2 less its mean: what half-space moments in u need.
-// l2 = 2 lam, c5 = 2 l2 / N, hs = (U^2 + 1/(2 lam)) / 2.
+// c5 = 4 lam / N, hs = (U^2 + s) / 2.
 template <class R>
-GKS_FN void half_coef(R U, R l2, R c5, R hs, const R e[4], R X[4]) {
-  X[3] = l2 * (c5 * e[3] - e[0]);
-  X[1] = l2 * e[1] - U * X[3];
-  X[0] = e[0] - U * X[1] - hs * X[3];
-  X[2] = l2 * e[2];
+GKS_FN void half_coef(R U, R s, R c5, R hs, const R e[4], R X[4]) {
+  X[3] = c5 * e[3] - e[0];
+  X[1] = e[1] - U * X[3];
+  X[0] = s * e[0] - U * X[1] - hs * X[3];
+  X[2] = e[2];
 }
 
 // A polynomial P(u, d, xi) of the half-space distribution averaged over d and xi: its mean q(u), and
@@ -510,30 +510,36 @@ GKS_FN R collision_time(const FaceConst<R>& C, bool ns, R pl, R pr, R p0, R dt) 
   return ns ? C.mu * d_rcp(p0) + jump : C.tau_eps * dt + C.tau_C * jump;
 }
 
+// Section 3.3: the equilibrium polynomial's derivatives (n, t, nn, nt, tt) from the six averages; of the
+// nn one without U0's share and factor
+template <class R>
+GKS_FN void equilibrium_derivatives(const FaceConst<R>& C, const R avg[2][3][4], R d[5][4]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const R um = avg[0][0][k], uc = avg[0][1][k], up = avg[0][2][k];
+    const R wm = avg[1][0][k], wc = avg[1][1][k], wp = avg[1][2][k];
+    const R Sr = wp + wm, Sl = up + um, Dr = wp - wm, Dl = up - um, cc = wc + uc;
+    d[0][k] = ((Sr - Sl) + R(2) * (wc - uc)) * C.i4n;  // b2
+    d[1][k] = (Dr + Dl) * C.i4t;                       // b3
+    d[2][k] = R(26) * cc - (Sr + Sl);
+    d[3][k] = (Dr - Dl) * C.i2nt;                      // b6
+    d[4][k] = ((Sr + Sl) - R(2) * cc) * C.i2t2;        // b5
+  }
+}
+
 // Equilibrium part, Eq. dis1, with g0 and the polynomial of Section 3.3.  All moments of g0 run over the
 // whole velocity space: in its frame they are closed forms in the central components of the
 // derivatives.  The compatibility conditions turn the moments of a1 u + a2 v into those of A,
 // and so on, so that the point value is U0 and its time derivatives.  (r0, u0, v0, var0): g0's
 // density, velocity and 1 / (2 lam).
-template <class R, class Src>
-GKS_FN void equilibrium_part(const FaceConst<R>& C, const Src& src, const R U0[4], R r0, R u0, R v0, R var0,
+template <class R>
+GKS_FN void equilibrium_part(const FaceConst<R>& C, R d[5][4], const R U0[4], R r0, R u0, R v0, R var0,
                              const TimeW<R>& w, R dt, R Fl[4], R P0[4], R P1[4], R Mn[4]) {
   const R U = u0, V = v0, s = var0, hq = R(0.5) * (u0 * u0 + v0 * v0), pN = C.i2N, kc = C.n2h * var0;
   R x[4], y[4], xx[4], xy[4], yy[4];
   {
-    R avg[2][3][4], d[5][4];
-    src.avg(avg);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const R um = avg[0][0][k], uc = avg[0][1][k], up = avg[0][2][k];
-      const R wm = avg[1][0][k], wc = avg[1][1][k], wp = avg[1][2][k];
-      const R Sr = wp + wm, Sl = up + um, Dr = wp - wm, Dl = up - um, cc = wc + uc;
-      d[0][k] = ((Sr - Sl) + R(2) * (wc - uc)) * C.i4n;                     // b2
-      d[1][k] = (Dr + Dl) * C.i4t;                                          // b3
-      d[2][k] = (R(26) * cc - (Sr + Sl) - R(48) * U0[k]) * C.i8n2;          // b4
-      d[3][k] = (Dr - Dl) * C.i2nt;                                         // b6
-      d[4][k] = ((Sr + Sl) - R(2) * cc) * C.i2t2;                           // b5
-    }
+    for (int k = 0; k < 4; ++k) d[2][k] = (d[2][k] - R(48) * U0[k]) * C.i8n2;  // b4
     central(U, V, hq, d[0], x);
     central(U, V, hq, d[1], y);
     central(U, V, hq, d[2], xx);
@@ -608,39 +614,50 @@ GKS_FN void equilibrium_part(const FaceConst<R>& C, const Src& src, const R U0[4
   lab(U, V, hq, p, P1);
 }
 
+// The coefficients of one side's Maxwellian in half_coef's basis, from its face state's derivatives
+// (A, tx, ty: Navier-Stokes only)
+template <class R>
+struct KineticCoefs {
+  R a1[4], a2[4], xx[4], xy[4], yy[4], A[4], tx[4], ty[4];
+};
+
+template <class R>
+GKS_FN void kinetic_coefs(const FaceConst<R>& C, const FaceState<R>& S, const SideData<R>& sd, bool ns, KineticCoefs<R>& k) {
+  const R U = sd.U, V = sd.V, s = sd.s;
+  // FP32: formed again (two instructions) rather than kept in a register across the equilibrium part
+  const R l2 = sizeof(R) == 4 ? d_rcp(s) : sd.l2;
+  const R hq = R(0.5) * (U * U + V * V), hs = R(0.5) * (U * U + s), c5 = C.i2N * l2;
+  R e1[4], e2[4], exx[4], exy[4], eyy[4];
+  central(U, V, hq, S.w[1], e1);
+  central(U, V, hq, S.w[2], e2);
+  central(U, V, hq, S.w[3], exx);
+  central(U, V, hq, S.w[4], exy);
+  central(U, V, hq, S.w[5], eyy);
+  half_coef(U, s, c5, hs, e1, k.a1);
+  half_coef(U, s, c5, hs, e2, k.a2);
+  half_coef(U, s, c5, hs, exx, k.xx);
+  half_coef(U, s, c5, hs, exy, k.xy);
+  half_coef(U, s, c5, hs, eyy, k.yy);
+  if (ns) {
+    const R kc = C.n2h * s;
+    R t[4];
+    time_coef(U, V, C.i2N, kc, e1, e2, t);
+    half_coef(U, s, c5, hs, t, k.A);
+    time_coef(U, V, C.i2N, kc, exx, exy, t);
+    half_coef(U, s, c5, hs, t, k.tx);
+    time_coef(U, V, C.i2N, kc, exy, eyy, t);
+    half_coef(U, s, c5, hs, t, k.ty);
+  }
+}
+
 // Kinetic part, Eq. dis2, of one side, added to Fl, P0, P1 and Mn: NS: f_G = g_k - tau (a u + A) g_k;
 // Euler: f_G = g_k, the terms with tn are absent (not formed).  kin_point: e > 0.
-template <class R, class Src>
-GKS_FN void kinetic_part(const FaceConst<R>& C, const Src& src, int side, const SideData<R>& sd, bool ns, bool kin_point,
+template <class R>
+GKS_FN void kinetic_part(const FaceConst<R>& C, const KineticCoefs<R>& kf, const SideData<R>& sd, bool ns, bool kin_point,
                          const TimeW<R>& w, R tn, R dt, R Fl[4], R P0[4], R P1[4], R Mn[4]) {
-  const R rho = sd.rho, U = sd.U, V = sd.V, s = sd.s, l2 = sd.l2;
-  R a1[4], a2[4], xx[4], xy[4], yy[4], A[4], tx[4], ty[4];
-  {
-    const R hq = R(0.5) * (U * U + V * V), hs = R(0.5) * (U * U + s), c5 = C.i2N * l2;
-    FaceState<R> S;
-    src.side(side, S);
-    R e1[4], e2[4], exx[4], exy[4], eyy[4];
-    central(U, V, hq, S.w[1], e1);
-    central(U, V, hq, S.w[2], e2);
-    central(U, V, hq, S.w[3], exx);
-    central(U, V, hq, S.w[4], exy);
-    central(U, V, hq, S.w[5], eyy);
-    half_coef(U, l2, c5, hs, e1, a1);
-    half_coef(U, l2, c5, hs, e2, a2);
-    half_coef(U, l2, c5, hs, exx, xx);
-    half_coef(U, l2, c5, hs, exy, xy);
-    half_coef(U, l2, c5, hs, eyy, yy);
-    if (ns) {
-      const R kc = C.n2h * s;
-      R t[4];
-      time_coef(U, V, C.i2N, kc, e1, e2, t);
-      half_coef(U, l2, c5, hs, t, A);
-      time_coef(U, V, C.i2N, kc, exx, exy, t);
-      half_coef(U, l2, c5, hs, t, tx);
-      time_coef(U, V, C.i2N, kc, exy, eyy, t);
-      half_coef(U, l2, c5, hs, t, ty);
-    }
-  }
+  const R rho = sd.rho, U = sd.U, V = sd.V, s = sd.s;
+  const R l2 = sizeof(R) == 4 ? d_rcp(s) : sd.l2;
+  const R *a1 = kf.a1, *a2 = kf.a2, *xx = kf.xx, *xy = kf.xy, *yy = kf.yy, *A = kf.A, *tx = kf.tx, *ty = kf.ty;
   R m[8];
   m[0] = sd.h;
   m[1] = sd.g;
@@ -651,12 +668,17 @@ GKS_FN void kinetic_part(const FaceConst<R>& C, const Src& src, int side, const 
   // v = V + d takes the terms in v to V times themselves and d times themselves
   auto poly = [&](R w7, R w9, R w10, HalfPoly<R>& P) {
     R B1[4], Bu[4], Bd[4], wq = R(0.5) * w10, wu = -w9;
-    const R t7 = tn * w7, t8 = -tn * w9;
+    R t7 = tn * w7, t8 = -tn * w9;
     if (ns) {
       wq -= t8;
       wu -= t7;
+      t7 *= l2;
+      t8 *= l2;
     }
-    const R wd = R(2) * wq * V, wyy = R(0.5) * C.y2 * w7 - wq * V * V;  // B1 takes V Bd, which holds wd yy
+    // the coefficients carry a factor s
+    wq *= l2;
+    wu *= l2;
+    const R wd = R(2) * wq * V, wyy = R(0.5) * C.y2 * (l2 * w7) - wq * V * V;  // B1 takes V Bd, which holds wd yy
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       Bd[k] = wu * a2[k] + wd * yy[k];
@@ -683,13 +705,13 @@ GKS_FN void kinetic_part(const FaceConst<R>& C, const Src& src, int side, const 
     poly(w.e, e9, dt * e9, P);
     half_moments<0, 4>(P, m, V, s, C.n1h, P0);
     // the part linear along the face: y (e (a2 - tau Aty) - (t + tau) e (Axy u + Ayy v))
-    const R wy = ns ? -tn * w.e - e9 : -e9, te = tn * w.e;
+    const R el = l2 * w.e, wy = l2 * (ns ? -tn * w.e - e9 : -e9), te = tn * el;
     R B1[4], Bu[4], Bd[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       Bd[k] = wy * yy[k];
       Bu[k] = wy * xy[k];
-      B1[k] = w.e * a2[k] + V * Bd[k];
+      B1[k] = el * a2[k] + V * Bd[k];
       if (ns) B1[k] = B1[k] - te * ty[k];
     }
     half_poly_linear(B1, Bu, Bd, s, C.n1h, P);
@@ -759,10 +781,20 @@ GKS_FN void face_evolution(const FaceConst<R>& C, const Src& src, R dt, R F[4], 
   // (smooth Euler flow); the point-value terms whose weights carry it are then not formed
   const bool kin_point = w.e > R(0);
   R Fl[4], P0[4], P1[4], Mn[4];
-  equilibrium_part(C, src, U0, r0, u0, v0, p0 * ir0, w, dt, Fl, P0, P1, Mn);
+  {
+    R avg[2][3][4], d[5][4];
+    src.avg(avg);
+    equilibrium_derivatives(C, avg, d);
+    equilibrium_part(C, d, U0, r0, u0, v0, p0 * ir0, w, dt, Fl, P0, P1, Mn);
+  }
 #pragma unroll
-  for (int side = 0; side < 2; ++side)
-    kinetic_part(C, src, side, sd[side], ns, kin_point, w, ns ? tau : R(0), dt, Fl, P0, P1, Mn);
+  for (int side = 0; side < 2; ++side) {
+    FaceState<R> S;
+    KineticCoefs<R> k;
+    src.side(side, S);
+    kinetic_coefs(C, S, sd[side], ns, k);
+    kinetic_part(C, k, sd[side], ns, kin_point, w, ns ? tau : R(0), dt, Fl, P0, P1, Mn);
+  }
   finish_face(C, u0, v0, Fl, P0, P1, Mn, F, Wm, Wp);
 }
 

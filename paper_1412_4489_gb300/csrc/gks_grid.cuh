@@ -24,6 +24,7 @@ struct Ctrl {
   int skip;
   long long fail_step;
   int bad_found[2];           // update pass 1 / 2 left a cell non-physical
+  unsigned bar_count, bar_gen;  // barrier of the fallback kernel's blocks
 };
 
 struct BCs {
@@ -103,16 +104,16 @@ template <> struct Lay<double> {
 #pragma unroll
     for (int v = 0; v < 4; ++v) p[f(n, v, o)] = x[v];
   }
-  static __device__ __forceinline__ void load_rec(const double* p, size_t c, double r[kRec]) {
-    const double2* q = reinterpret_cast<const double2*>(p + c * kRec);
+  static __device__ __forceinline__ void load_rec(const double* p, double r[kRec]) {
+    const double2* q = reinterpret_cast<const double2*>(p);
 #pragma unroll
     for (int k = 0; k < kRec / 2; ++k) {
       const double2 t = q[k];
       r[2 * k] = t.x; r[2 * k + 1] = t.y;
     }
   }
-  static __device__ __forceinline__ void load_avg(const double* p, size_t c, double r[4]) {
-    const double2* q = reinterpret_cast<const double2*>(p + c * kRec);
+  static __device__ __forceinline__ void load_avg(const double* p, double r[4]) {
+    const double2* q = reinterpret_cast<const double2*>(p);
     const double2 a = q[0], b = q[1];
     r[0] = a.x; r[1] = a.y; r[2] = b.x; r[3] = b.y;
   }
@@ -143,11 +144,11 @@ template <> struct Lay<float> {
   static __device__ __forceinline__ void load_f(const float* p, size_t, size_t o, float x[4]) { get(p, o, x); }
   static __device__ __forceinline__ void store_w(float* p, size_t n, int q, size_t o, const float x[4]) { put(p, q * n + o, x); }
   static __device__ __forceinline__ void store_f(float* p, size_t, size_t o, const float x[4]) { put(p, o, x); }
-  static __device__ __forceinline__ void load_rec(const float* p, size_t c, float r[kRec]) {
+  static __device__ __forceinline__ void load_rec(const float* p, float r[kRec]) {
 #pragma unroll
-    for (int k = 0; k < kRec / 4; ++k) get(p, c * (kRec / 4) + k, r + 4 * k);
+    for (int k = 0; k < kRec / 4; ++k) get(p, k, r + 4 * k);
   }
-  static __device__ __forceinline__ void load_avg(const float* p, size_t c, float r[4]) { get(p, c * (kRec / 4), r); }
+  static __device__ __forceinline__ void load_avg(const float* p, float r[4]) { get(p, 0, r); }
   static __device__ __forceinline__ void store_rec(float* p, size_t c, const float r[kRec]) {
 #pragma unroll
     for (int k = 0; k < kRec / 4; ++k) put(p, c * (kRec / 4) + k, r + 4 * k);
@@ -615,22 +616,40 @@ __device__ __forceinline__ void recon_cell_lanes(const Geo& g, const double* __r
   double a[5];
   recon_var_scaled(c, u[1], u[-1], u[g.pitch], u[-g.pitch], wx[1], wx[fxp + 1], wx[0], wx[fxp], wn[0], wn[fyp], ws[0],
                    ws[fyp], g.weno_eps, g.b1sq, a);
-  // the polynomial at the four face centres: positive density and pressure
-  // (2 rho rho E > |rho u|^2), else the constant average
-  const double p4 = (1.0 / 12.0) * a[2], p5 = (1.0 / 12.0) * a[3];
-  const double e0 = c + (p4 - 0.5 * p5), n0 = c + (p5 - 0.5 * p4);
-  const double f[4] = {e0 + 0.5 * a[0], e0 - 0.5 * a[0], n0 + 0.5 * a[1], n0 - 0.5 * a[1]};
+  // The polynomial at the four face centres: positive density and pressure (2 rho rho E > |rho u|^2), else the
+  // constant average.  First in FP32, which the FP64 pipe does not pay for, with bounds that hold for every
+  // rounding (density and energy from below, momenta from above); where those do not decide, in FP64.
+  const float cf = (float)c, f0 = (float)a[0], f1 = (float)a[1], f2 = (float)a[2], f3 = (float)a[3];
+  const float slack = 2e-6f * (fabsf(cf) + fabsf(f0) + fabsf(f1) + fabsf(f2) + fabsf(f3));
   bool ok = true;
+  {
+    const float q4 = f2 * (1.0f / 12.0f), q5 = f3 * (1.0f / 12.0f);
+    const float e = cf + (q4 - 0.5f * q5), n = cf + (q5 - 0.5f * q4);
+    const float f[4] = {e + 0.5f * f0, e - 0.5f * f0, n + 0.5f * f1, n - 0.5f * f1};
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    // lane 0: 2 rho rho E, lanes 1 and 2: minus their momentum squared; the sum over the four
-    const double E = __shfl_down_sync(0xffffffffu, f[k], 3, 4);
-    double t = f[k] * (v == 0 ? E + E : (v == 3 ? 0.0 : -f[k]));
-    t += __shfl_xor_sync(0xffffffffu, t, 1);
-    t += __shfl_xor_sync(0xffffffffu, t, 2);
-    // t > 0 and (lane 0) the density > 0, as orderings of their bits: NaN lies above infinity
-    auto positive = [](double x) { return (unsigned long long)(__double_as_longlong(x) - 1) < 0x7ff0000000000000ull; };
-    ok = ok && positive(t) && (v != 0 || positive(f[k]));
+    for (int k = 0; k < 4; ++k) {
+      const float b = v == 0 || v == 3 ? f[k] - slack : fabsf(f[k]) + slack;
+      const float E = __shfl_down_sync(0xffffffffu, b, 3, 4), m1 = __shfl_down_sync(0xffffffffu, b, 1, 4);
+      const float m2 = __shfl_down_sync(0xffffffffu, b, 2, 4);
+      ok = ok && (v != 0 || (b > 0.0f && E > 0.0f && 2.0f * b * E > 1.00001f * (m1 * m1 + m2 * m2) + 1e-30f));
+    }
+  }
+  if (__any_sync(0xffffffffu, !ok)) {
+    const double p4 = (1.0 / 12.0) * a[2], p5 = (1.0 / 12.0) * a[3];
+    const double e0 = c + (p4 - 0.5 * p5), n0 = c + (p5 - 0.5 * p4);
+    const double f[4] = {e0 + 0.5 * a[0], e0 - 0.5 * a[0], n0 + 0.5 * a[1], n0 - 0.5 * a[1]};
+    ok = true;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      // lane 0: 2 rho rho E, lanes 1 and 2: minus their momentum squared; the sum over the four
+      const double E = __shfl_down_sync(0xffffffffu, f[k], 3, 4);
+      double t = f[k] * (v == 0 ? E + E : (v == 3 ? 0.0 : -f[k]));
+      t += __shfl_xor_sync(0xffffffffu, t, 1);
+      t += __shfl_xor_sync(0xffffffffu, t, 2);
+      // t > 0 and (lane 0) the density > 0, as orderings of their bits: NaN lies above infinity
+      auto positive = [](double x) { return (unsigned long long)(__double_as_longlong(x) - 1) < 0x7ff0000000000000ull; };
+      ok = ok && positive(t) && (v != 0 || positive(f[k]));
+    }
   }
   const bool bad = !__shfl_sync(0xffffffffu, (int)ok, 0, 4);
   if (!active) return;
@@ -649,13 +668,13 @@ __device__ __forceinline__ void recon_cell_lanes(const Geo& g, const double* __r
 // face-frame slot of physical variable v (y-faces swap the momenta)
 template <int AX> __device__ __forceinline__ int slot(int v) { return AX == 0 ? v : (v == 1 ? 2 : (v == 2 ? 1 : v)); }
 
-// value and derivatives of cell (i, j)'s polynomial at the centre of its face
+// value and derivatives of a cell's polynomial (its record) at the centre of its face
 // on side s (+1: the face at +h_n/2, -1: at -h_n/2), in the face frame of axis AX
 template <int AX, class R>
-__device__ __forceinline__ void side_state(const Geo& g, const R* __restrict__ rec, int i, int j, int s, R hn,
-                                           R hn2_12, R ht2_24, FaceState<R>& S) {
+__device__ __forceinline__ void side_state(const R* __restrict__ record, int s, R hn, R hn2_12, R ht2_24,
+                                           FaceState<R>& S) {
   R r[kRec];
-  Lay<R>::load_rec(rec, rec_at(g, i, j), r);
+  Lay<R>::load_rec(record, r);
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     const R c = r[v];
@@ -678,7 +697,9 @@ template <int AX, class R>
 struct GridFaceSource {
   const Geo* g;
   const R* U;    // padded compute-type averages (the first-order fallback's constant states)
-  const R* rec;  // reconstruction records
+  const R* at;   // record of cell (i, j): the others lie at fixed distances, so one address serves a face
+  int to_l, to_r;  // from there to the records of the cells cl and cr, in records (a grid that fits the
+                   // memory has far fewer than 2^31)
   int i, j;            // face index (x-faces: i in [0, nx]; y-faces: j in [0, ny])
   int cl, cr;          // the two cells along the normal, after periodic wrap
   int img_lo, img_hi;  // boundary image on the low / high side: 0 none, else the BC kind
@@ -728,32 +749,32 @@ struct GridFaceSource {
     if (k == 0) {
       if (img_lo) {
         FaceState<R> in;
-        side_state<AX>(*g, rec, cx(cr), cy(cr), -1, hn, hn2_12, ht2_24, in);
+        side_state<AX>(at + (ptrdiff_t)to_r * kRec, -1, hn, hn2_12, ht2_24, in);
         image(img_lo, uwt_lo, Tw_lo, in, S);
       } else {
-        side_state<AX>(*g, rec, cx(cl), cy(cl), +1, hn, hn2_12, ht2_24, S);
+        side_state<AX>(at + (ptrdiff_t)to_l * kRec, +1, hn, hn2_12, ht2_24, S);
       }
     } else {
       if (img_hi) {
         FaceState<R> in;
-        side_state<AX>(*g, rec, cx(cl), cy(cl), +1, hn, hn2_12, ht2_24, in);
+        side_state<AX>(at + (ptrdiff_t)to_l * kRec, +1, hn, hn2_12, ht2_24, in);
         image(img_hi, uwt_hi, Tw_hi, in, S);
       } else {
-        side_state<AX>(*g, rec, cx(cr), cy(cr), -1, hn, hn2_12, ht2_24, S);
+        side_state<AX>(at + (ptrdiff_t)to_r * kRec, -1, hn, hn2_12, ht2_24, S);
       }
     }
   }
 
   // six cell averages around the face (ghost ring included), face frame
   __device__ __forceinline__ void avg(R a[2][3][4]) const {
+    const ptrdiff_t row = (ptrdiff_t)(g->nx + 2) * kRec;
 #pragma unroll
     for (int m = 0; m < 2; ++m)
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        const int ii = AX == 0 ? i - 1 + m : i - 1 + k;
-        const int jj = AX == 0 ? j - 1 + k : j - 1 + m;
+        const int di = (AX == 0 ? m : k) - 1, dj = (AX == 0 ? k : m) - 1;
         R w[4];
-        Lay<R>::load_avg(rec, rec_at(*g, ii, jj), w);
+        Lay<R>::load_avg(at + dj * row + di * kRec, w);
 #pragma unroll
         for (int v = 0; v < 4; ++v) a[m][k][slot<AX>(v)] = w[v];
       }
@@ -788,7 +809,7 @@ __device__ __forceinline__ GridFaceSource<AX, R> face_source(const Geo& g, const
   GridFaceSource<AX, R> src;
   src.g = &g;
   src.U = U;
-  src.rec = rec;
+  src.at = rec + rec_at(g, i, j) * kRec;
   src.i = i;
   src.j = j;
   const int f = AX == 0 ? i : j;         // face index along the normal
@@ -808,6 +829,9 @@ __device__ __forceinline__ GridFaceSource<AX, R> face_source(const Geo& g, const
     if (g.bc.kind[hi_side] == GKS_BC_PERIODIC) src.cr = 0;
     else if (g.bc.kind[hi_side] != GKS_BC_EXCHANGE) src.img_hi = g.bc.kind[hi_side];
   }
+  const int step = AX == 0 ? 1 : g.nx + 2;
+  src.to_l = src.cl == f - 1 ? -step : (nf - 1) * step;
+  src.to_r = src.cr == f ? 0 : -nf * step;
   src.gamma = GeoR<R>::gamma(g);
   src.uwt_lo = GeoR<R>::uwt(g, lo_side);
   src.Tw_lo = GeoR<R>::Tw(g, lo_side);
@@ -869,9 +893,19 @@ struct SplitShare {
   R u0[2][4][32], p[2][32], part[2][16][32];
 };
 
+// named barriers of a block: arrive without waiting, or arrive and wait (memory accesses before either are
+// seen by the threads that the barrier lets go); whole warps, threads in all
+__device__ __forceinline__ void named_arrive(int id, int threads) {
+  asm volatile("barrier.cta.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void named_sync(int id, int threads) {
+  asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
 // The evolution at 32 faces by three warps: the left side (warp 0), the right side (warp 1) and the equilibrium
-// part (warp 2), each with the same arithmetic as face_evolution.  Every thread of the 96 calls it; active: the
-// lane has a face.
+// part (warp 2), each with the same arithmetic as face_evolution.  What a warp can form before it has
+// U0 (the sides' coefficients, the equilibrium polynomial's differences) it forms while the others
+// work towards it.  Every thread of the 96 calls it; active: the lane has a face.
 template <int AX, class R, class TW, int NSM>
 __device__ __forceinline__ void flux_face_split(const Geo& g, const FaceConst<R>& C, const R* __restrict__ rec,
                                                 TW* __restrict__ Wn, R* __restrict__ F, int i, int j, bool active, R dt,
@@ -879,32 +913,35 @@ __device__ __forceinline__ void flux_face_split(const Geo& g, const FaceConst<R>
   const int role = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool ns = NSM < 0 ? C.ns : NSM == 1;
   const GridFaceSource<AX, R> src = face_source<AX, R>(g, C, rec, i, j);
-  SideData<R> sd;
-  if (active && role < 2) {
-    FaceState<R> S;
-    src.side(role, S);
-    R u[4] = {R(0), R(0), R(0), R(0)};
-    side_start(C, S.w[0], role, sd, u);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) sh.u0[role][k][lane] = u[k];
-    sh.p[role][lane] = sd.p;
-  }
-  __syncthreads();
-  R r0, ir0, u0, v0, p0, Fl[4], P0[4], P1[4], Mn[4];
-  if (active) {
-    R U0[4];
+  R U0[4], r0, ir0, u0, v0, p0, tau, Fl[4], P0[4], P1[4], Mn[4];
+  TimeW<R> w;
+  auto weights = [&]() {
 #pragma unroll
     for (int k = 0; k < 4; ++k) U0[k] = sh.u0[0][k][lane] + sh.u0[1][k][lane];
     prim(U0, C.gm1, r0, ir0, u0, v0, p0);
-    const R tau = collision_time(C, ns, sh.p[0][lane], sh.p[1][lane], p0, dt);
-    TimeW<R> w;
+    tau = collision_time(C, ns, sh.p[0][lane], sh.p[1][lane], p0, dt);
     time_weights(dt, tau, w);
-    if (role == 2) {
-      equilibrium_part(C, src, U0, r0, u0, v0, p0 * ir0, w, dt, Fl, P0, P1, Mn);
-    } else {
+  };
+  if (role < 2) {
+    SideData<R> sd;
+    FaceState<R> S;
+    KineticCoefs<R> kf;
+    if (active) {
+      src.side(role, S);
+      R u[4] = {R(0), R(0), R(0), R(0)};
+      side_start(C, S.w[0], role, sd, u);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) sh.u0[role][k][lane] = u[k];
+      sh.p[role][lane] = sd.p;
+    }
+    named_arrive(1, 96);
+    if (active) kinetic_coefs(C, S, sd, ns, kf);
+    named_sync(2, 64);
+    if (active) {
+      weights();
 #pragma unroll
       for (int k = 0; k < 4; ++k) Fl[k] = P0[k] = P1[k] = Mn[k] = R(0);
-      kinetic_part(C, src, role, sd, ns, w.e > R(0), w, ns ? tau : R(0), dt, Fl, P0, P1, Mn);
+      kinetic_part(C, kf, sd, ns, w.e > R(0), w, ns ? tau : R(0), dt, Fl, P0, P1, Mn);
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         sh.part[role][k][lane] = Fl[k];
@@ -913,22 +950,34 @@ __device__ __forceinline__ void flux_face_split(const Geo& g, const FaceConst<R>
         sh.part[role][12 + k][lane] = Mn[k];
       }
     }
+    named_arrive(3, 96);
+    return;
   }
-  __syncthreads();
-  if (active && role == 2) {
-#pragma unroll
-    for (int q = 0; q < 2; ++q)
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        Fl[k] += sh.part[q][k][lane];
-        P0[k] += sh.part[q][4 + k][lane];
-        P1[k] += sh.part[q][8 + k][lane];
-        if (C.prandtl) Mn[k] += sh.part[q][12 + k][lane];
-      }
-    R Fo[4], Wm[4], Wp[4];
-    finish_face(C, u0, v0, Fl, P0, P1, Mn, Fo, Wm, Wp);
-    store_face<AX, R, TW>(g, src, Wn, F, Fo, Wm, Wp);
+  R d[5][4];
+  if (active) {
+    R avg[2][3][4];
+    src.avg(avg);
+    equilibrium_derivatives(C, avg, d);
   }
+  named_sync(1, 96);
+  if (active) {
+    weights();
+    equilibrium_part(C, d, U0, r0, u0, v0, p0 * ir0, w, dt, Fl, P0, P1, Mn);
+  }
+  named_sync(3, 96);
+  if (!active) return;
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      Fl[k] += sh.part[q][k][lane];
+      P0[k] += sh.part[q][4 + k][lane];
+      P1[k] += sh.part[q][8 + k][lane];
+      if (C.prandtl) Mn[k] += sh.part[q][12 + k][lane];
+    }
+  R Fo[4], Wm[4], Wp[4];
+  finish_face(C, u0, v0, Fl, P0, P1, Mn, Fo, Wm, Wp);
+  store_face<AX, R, TW>(g, src, Wn, F, Fo, Wm, Wp);
 }
 
 // ---------------------------------------------------------------------------
