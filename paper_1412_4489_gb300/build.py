@@ -17,6 +17,7 @@ SOURCES = [os.path.join(HERE, "csrc", n) for n in ("gks.cu", "gks_batch.cu", "gk
 DEPS = SOURCES + [os.path.join(HERE, "csrc", "gks_device.cuh"), os.path.join(HERE, "csrc", "gks_grid.cuh"),
                   os.path.join(HERE, "csrc", "gks_face_monomials.cuh"),
                   os.path.join(HERE, "csrc", "gks_half_normal.cuh"),
+                  os.path.join(HERE, "csrc", "gks_state.cuh"),
                   os.path.join(ROOT, "include", "gks.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

@@ -27,10 +27,12 @@
 
 #include <atomic>
 #include <string>
+#include <type_traits>
 
 #include "../../include/gks.h"
 #include "gks_device.cuh"
 #include "gks_grid.cuh"
+#include "gks_state.cuh"
 
 using namespace gks;
 
@@ -393,53 +395,6 @@ dim3 update_grid(const Geo& g, int pass, int sms, int blocks_per_sm, int rows) {
   return dim3(tx, ty);
 }
 
-// CFL bound of the current state (after set_state), in FP64
-template <class R>
-__global__ void k_dtbound(Geo g, Cells<R> U0, Cells<R> U1, Ctrl* c) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  const int par = (int)(c->steps & 1);
-  const Cells<R> U = par ? U1 : U0;
-  double inv = 0.0;
-  if (i < g.nx && j < g.ny) {
-    double w[4];
-    for (int v = 0; v < 4; ++v) w[v] = U.get(g, v, i, j);
-    bool ok;
-    inv = inv_bound<double>(g, w, ok);
-    if (!ok || !(inv < INFINITY)) {
-      atomicCAS(&c->status, GKS_OK, GKS_ENONPHYSICAL);
-      inv = 0.0;
-    }
-  }
-  block_bound_to<double>(inv, &c->bound);
-}
-
-// ---------------------------------------------------------------------------
-// state transfer
-// ---------------------------------------------------------------------------
-template <class R>
-__global__ void k_scatter_U(Geo g, const double* __restrict__ src, Cells<R> U0, Cells<R> U1, const Ctrl* c,
-                            int to_dev) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= g.nx || j >= g.ny) return;
-  const Cells<R> U = (c->steps & 1) ? U1 : U0;
-  for (int v = 0; v < 4; ++v) {
-    const size_t o = ((size_t)v * g.ny + j) * g.nx + i;
-    if (to_dev) U.set(g, v, i, j, src[o]);
-    else const_cast<double*>(src)[o] = U.get(g, v, i, j);
-  }
-}
-
-// face values between the caller's planes [4][2][faces] (n = 8 x faces values) and the layout of the type
-template <class TW>
-__global__ void k_copy_W(const double* __restrict__ src, TW* W0, TW* W1, size_t n, const Ctrl* c, int to_dev) {
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  TW* W = (c->steps & 1) ? W1 : W0;
-  copy_w(src, W, n / 8, k, to_dev);
-}
-
 // face values = mean of the two adjacent averages (ghosts included)
 template <int AX, class TW>
 __global__ void k_init_W(Geo g, Cells<TW> U0, Cells<TW> U1, TW* W0, TW* W1, const Ctrl* c) {
@@ -762,64 +717,44 @@ gks_status capture(gks_handle* h, int nsteps, double cfl, double t_end, cudaGrap
   return GKS_OK;
 }
 
-gks_status reset_ctrl(gks_handle* h, double t) {
-  memset(h->hctrl, 0, sizeof(Ctrl));
-  const double inf = INFINITY;
-  uint64_t b;
-  memcpy(&b, &inf, 8);
-  h->hctrl->bound = b;
-  h->hctrl->dtb[0] = h->hctrl->dtb[1] = h->hctrl->dtb[2] = b;
-  h->hctrl->t = t;
-  CK(cudaMemcpyAsync(h->ctrl, h->hctrl, sizeof(Ctrl), cudaMemcpyHostToDevice, h->stream));
-  CK(cudaStreamSynchronize(h->stream));
-  return GKS_OK;
-}
-
-// Loads a state from device FP64 arrays.  With stage_w set, dWx /
-// dWy are host arrays copied in turn through the staging buffer (which must
-// then not hold dU).
-// The device address of a page-locked host array mapped into the device's address
-// space (cudaHostAlloc, cudaHostRegister): kernels then read or write it in place over
-// the host link.  nullptr for any other pointer (pageable host memory goes through
-// the staging buffer).
-const double* mapped_host(const void* p) {
-  cudaPointerAttributes a;
-  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-    cudaGetLastError();  // an unknown pointer: clear the error it left
-    return nullptr;
-  }
-  return a.type == cudaMemoryTypeHost && a.devicePointer ? (const double*)a.devicePointer : nullptr;
-}
-
-// dU, dWx, dWy: device-accessible arrays, except that a face-value array flagged in
-// stage_x / stage_y is a host array copied through the staging buffer first
+// Loads a state.  dU, dWx, dWy: device-accessible arrays, except that one flagged in stage_u / stage_x / stage_y is a
+// host array copied through the staging buffer first (in turn: the kernel that reads it comes before the next
+// copy in the stream).  dWx / dWy null: mean of the adjacent averages.
 template <class TW>
-gks_status load_state(gks_handle* h, const double* dU, const double* dWx, const double* dWy, bool stage_x = false,
-                      bool stage_y = false) {
+gks_status load_state(gks_handle* h, double t, const double* dU, const double* dWx, const double* dWy, bool stage_u = false,
+                      bool stage_x = false, bool stage_y = false) {
   const Geo& g = h->g;
   cudaStream_t s = h->stream;
   const dim3 b2(32, 8);
   const Cells<TW> U0 = cellbuf<TW>(h, 0), U1 = cellbuf<TW>(h, 1);
-  k_scatter_U<TW><<<grid2(g.nx, g.ny, b2), b2, 0, s>>>(g, dU, U0, U1, h->ctrl, 1);
-  launch_ghost<TW>(h, 1);
+  TW *Wx0 = (TW*)h->Wx[0], *Wx1 = (TW*)h->Wx[1], *Wy0 = (TW*)h->Wy[0], *Wy1 = (TW*)h->Wy[1];
+  const size_t nfx = n_wx(g) / 8, nfy = n_wy(g) / 8;
+  auto staged = [&](const double* src, size_t n) {
+    const cudaError_t e = cudaMemcpyAsync(h->staging, src, n * sizeof(double), cudaMemcpyHostToDevice, s);
+    return e;
+  };
+  k_state_begin<<<1, 1, 0, s>>>(h->ctrl, t, 1);
+  if (stage_u) {
+    CK(staged(dU, n_u(g)));
+    dU = h->staging;
+  }
+  k_load_cells<TW><<<blocks_of((size_t)g.nx * g.ny), 256, 0, s>>>(g, dU, U0, U1, h->ctrl);
   for (int axis = 0; axis < 2; ++axis) {
-    const double* src = axis == 0 ? dWx : dWy;
-    const size_t n = axis == 0 ? n_wx(g) : n_wy(g);
-    TW* W0 = (TW*)(axis == 0 ? h->Wx[0] : h->Wy[0]);
-    TW* W1 = (TW*)(axis == 0 ? h->Wx[1] : h->Wy[1]);
-    if (src) {
-      if (axis == 0 ? stage_x : stage_y) {
-        CK(cudaMemcpyAsync(h->staging, src, n * sizeof(double), cudaMemcpyHostToDevice, s));
-        src = h->staging;
-      }
-      k_copy_W<TW><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(src, W0, W1, n, h->ctrl, 1);
-    } else if (axis == 0) {
-      k_init_W<0, TW><<<grid2(g.nx + 1, g.ny, b2), b2, 0, s>>>(g, U0, U1, W0, W1, h->ctrl);
-    } else {
-      k_init_W<1, TW><<<grid2(g.nx, g.ny + 1, b2), b2, 0, s>>>(g, U0, U1, W0, W1, h->ctrl);
+    const double*& src = axis == 0 ? dWx : dWy;
+    const size_t n = axis == 0 ? nfx : nfy;
+    if (!src) {
+      if (axis == 0) k_init_W<0, TW><<<grid2(g.nx + 1, g.ny, b2), b2, 0, s>>>(g, U0, U1, Wx0, Wx1, h->ctrl);
+      else k_init_W<1, TW><<<grid2(g.nx, g.ny + 1, b2), b2, 0, s>>>(g, U0, U1, Wy0, Wy1, h->ctrl);
+    } else if (axis == 0 ? stage_x : stage_y) {
+      CK(staged(src, 8 * n));
+      k_face_values<TW, true><<<blocks_of(n), 256, 0, s>>>(axis == 0 ? h->staging : nullptr, axis == 0 ? nullptr : h->staging,
+                                                           nfx, nfy, Wx0, Wx1, Wy0, Wy1, h->ctrl);
+      src = nullptr;
     }
   }
-  k_dtbound<TW><<<grid2(g.nx, g.ny, b2), b2, 0, s>>>(g, U0, U1, h->ctrl);
+  if (dWx || dWy)
+    k_face_values<TW, true><<<blocks_of((dWx ? nfx : 0) + (dWy ? nfy : 0)), 256, 0, s>>>(
+        const_cast<double*>(dWx), const_cast<double*>(dWy), nfx, nfy, Wx0, Wx1, Wy0, Wy1, h->ctrl);
   CK(cudaGetLastError());
   return GKS_OK;
 }
@@ -828,12 +763,12 @@ template <class TW>
 gks_status store_state(gks_handle* h, double* dU, double* dWx, double* dWy) {
   const Geo& g = h->g;
   cudaStream_t s = h->stream;
-  const dim3 b2(32, 8);
-  if (dU) k_scatter_U<TW><<<grid2(g.nx, g.ny, b2), b2, 0, s>>>(g, dU, cellbuf<TW>(h, 0), cellbuf<TW>(h, 1), h->ctrl, 0);
-  if (dWx)
-    k_copy_W<TW><<<(unsigned)((n_wx(g) + 255) / 256), 256, 0, s>>>(dWx, (TW*)h->Wx[0], (TW*)h->Wx[1], n_wx(g), h->ctrl, 0);
-  if (dWy)
-    k_copy_W<TW><<<(unsigned)((n_wy(g) + 255) / 256), 256, 0, s>>>(dWy, (TW*)h->Wy[0], (TW*)h->Wy[1], n_wy(g), h->ctrl, 0);
+  const size_t nfx = n_wx(g) / 8, nfy = n_wy(g) / 8;
+  if (dU)
+    k_store_cells<TW><<<blocks_of((size_t)g.nx * g.ny), 256, 0, s>>>(g, dU, cellbuf<TW>(h, 0), cellbuf<TW>(h, 1), h->ctrl);
+  if (dWx || dWy)
+    k_face_values<TW, false><<<blocks_of((dWx ? nfx : 0) + (dWy ? nfy : 0)), 256, 0, s>>>(
+        dWx, dWy, nfx, nfy, (TW*)h->Wx[0], (TW*)h->Wx[1], (TW*)h->Wy[0], (TW*)h->Wy[1], h->ctrl);
   CK(cudaGetLastError());
   return GKS_OK;
 }
@@ -957,8 +892,11 @@ gks_status gks_create(int nx, int ny, double Lx, double Ly, double gamma, double
     gks_destroy(h);
     return st;
   }
-  if (reset_ctrl(h, 0.0) != GKS_OK) {
-    g_create_err = h->err;
+  k_state_begin<<<1, 1, 0, h->stream>>>(h->ctrl, 0.0, 1);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  if (e != cudaSuccess) {
+    g_create_err = std::string("gks_create: ") + cudaGetErrorString(e);
     gks_destroy(h);
     return GKS_ECUDA;
   }
@@ -969,9 +907,7 @@ gks_status gks_create(int nx, int ny, double Lx, double Ly, double gamma, double
 gks_status gks_set_state_device(gks_handle* h, const double* dU, const double* dWx, const double* dWy, double t) {
   if (!h || !dU) return fail(h, GKS_EINVAL, "gks_set_state: U is required");
   CK(cudaSetDevice(h->device));
-  gks_status st = reset_ctrl(h, t);
-  if (st != GKS_OK) return st;
-  st = h->prec == GKS_FP64 ? load_state<double>(h, dU, dWx, dWy) : load_state<float>(h, dU, dWx, dWy);
+  gks_status st = h->prec == GKS_FP64 ? load_state<double>(h, t, dU, dWx, dWy) : load_state<float>(h, t, dU, dWx, dWy);
   if (st != GKS_OK) return st;
   st = read_ctrl(h);
   if (st != GKS_OK) return st;
@@ -982,24 +918,15 @@ gks_status gks_set_state_device(gks_handle* h, const double* dU, const double* d
 gks_status gks_set_state(gks_handle* h, const double* U, const double* Wx, const double* Wy, double t) {
   if (!h || !U) return fail(h, GKS_EINVAL, "gks_set_state: U is required");
   CK(cudaSetDevice(h->device));
-  const Geo& g = h->g;
-  gks_status st = reset_ctrl(h, t);
-  if (st != GKS_OK) return st;
   // page-locked host arrays are read in place by the kernels; the others go through
-  // the staging buffer in turn (U first: the scatter reads it before the face values
-  // reuse the buffer, same stream)
-  const double* dU = mapped_host(U);
-  const double* dWx = Wx ? mapped_host(Wx) : nullptr;
-  const double* dWy = Wy ? mapped_host(Wy) : nullptr;
-  if (!dU) {
-    CK(cudaMemcpyAsync(h->staging, U, n_u(g) * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-    dU = h->staging;
-  }
-  const bool sx = Wx && !dWx, sy = Wy && !dWy;
+  // the staging buffer in turn
+  const double *dU = mapped_host(U), *dWx = Wx ? mapped_host(Wx) : nullptr, *dWy = Wy ? mapped_host(Wy) : nullptr;
+  const bool su = !dU, sx = Wx && !dWx, sy = Wy && !dWy;
+  if (su) dU = U;
   if (sx) dWx = Wx;
   if (sy) dWy = Wy;
-  st = h->prec == GKS_FP64 ? load_state<double>(h, dU, dWx, dWy, sx, sy)
-                           : load_state<float>(h, dU, dWx, dWy, sx, sy);
+  gks_status st = h->prec == GKS_FP64 ? load_state<double>(h, t, dU, dWx, dWy, su, sx, sy)
+                                      : load_state<float>(h, t, dU, dWx, dWy, su, sx, sy);
   if (st != GKS_OK) return st;
   st = read_ctrl(h);
   if (st != GKS_OK) return st;
@@ -1170,19 +1097,23 @@ gks_status gks_debug_flux(gks_handle* h, double dt, double* Fx, double* Fy, doub
   if (st != GKS_OK) return st;
   st = read_ctrl(h);
   if (st != GKS_OK) return st;
-  // new face values were written to the buffer that is not in use: as k_copy_W's other one
+  // new face values were written to the buffer that is not in use
   const size_t nfx = (size_t)g.ny * (g.nx + 1), nfy = (size_t)(g.ny + 1) * g.nx;
   struct { void *a, *b; double* dst; size_t faces; bool w; } parts[4] = {
       {h->Fx, h->Fx, Fx, nfx, false}, {h->Fy, h->Fy, Fy, nfy, false}, {h->Wx[1], h->Wx[0], Wxn, nfx, true}, {h->Wy[1], h->Wy[0], Wyn, nfy, true}};
+  auto values = [&](auto* a, auto* b, size_t faces) {
+    using T = std::remove_pointer_t<decltype(a)>;
+    k_face_values<T, false><<<blocks_of(faces), 256, 0, h->stream>>>(h->staging, nullptr, faces, 0, a, b, (T*)nullptr, (T*)nullptr, h->ctrl);
+  };
   for (auto& p : parts) {
     if (!p.dst) continue;
     const size_t n = (p.w ? 8 : 4) * p.faces;
     const unsigned blocks = (unsigned)((n + 255) / 256);
     if (h->prec == GKS_FP64) {
-      if (p.w) k_copy_W<double><<<blocks, 256, 0, h->stream>>>(h->staging, (double*)p.a, (double*)p.b, n, h->ctrl, 0);
+      if (p.w) values((double*)p.a, (double*)p.b, p.faces);
       else k_flux_out<double><<<blocks, 256, 0, h->stream>>>((const double*)p.a, h->staging, p.faces);
     } else {
-      if (p.w) k_copy_W<float><<<blocks, 256, 0, h->stream>>>(h->staging, (float*)p.a, (float*)p.b, n, h->ctrl, 0);
+      if (p.w) values((float*)p.a, (float*)p.b, p.faces);
       else k_flux_out<float><<<blocks, 256, 0, h->stream>>>((const float*)p.a, h->staging, p.faces);
     }
     CK(cudaGetLastError());
@@ -1328,20 +1259,6 @@ void* noalloc_base(int device, std::string& why) {
   return p;
 }
 
-__global__ void k_noalloc_ctrl(Ctrl* c) {
-  c->bound = dbits(INFINITY);
-  c->dtb[0] = c->dtb[1] = c->dtb[2] = dbits(INFINITY);
-  c->bad_found[0] = c->bad_found[1] = 0;
-  c->bar_count = c->bar_gen = 0;
-  c->t = 0.0;
-  c->dt = 0.0;
-  c->dt_f = 0.0f;
-  c->steps = 0;
-  c->status = GKS_OK;
-  c->skip = 0;
-  c->fail_step = -1;
-}
-
 }  // namespace
 
 extern "C" gks_status gks_step_noalloc(int nx, int ny, double Lx, double Ly, double gamma, double Pr, double mu,
@@ -1404,24 +1321,21 @@ extern "C" gks_status gks_step_noalloc(int nx, int ny, double Lx, double Ly, dou
   double* Fy = (double*)(base + b_ctrl + 2 * b_u + b_rec + b_fx);
   unsigned char* bad = base + b_ctrl + 2 * b_u + b_rec + b_fx + b_fy;
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  const dim3 b2(32, 8);
-  const int per = perimeter(g);
   const Cells<double> C0{U0}, C1{U1};
   // the control block must start from zero state; the rest is fully written before it is read
-  k_noalloc_ctrl<<<1, 1, 0, s>>>(ctrl);
-  k_scatter_U<double><<<grid2(nx, ny, b2), b2, 0, s>>>(g, dU, C0, C1, ctrl, 1);
-  k_ghost<double><<<(per + 127) / 128, 128, 0, s>>>(g, C0, C1, ctrl, 1);
-  k_dtbound<double><<<grid2(nx, ny, b2), b2, 0, s>>>(g, C0, C1, ctrl);
-  e = launch_recon<double, double>(false, s, g, U0, U1, dWx, dWx_out, dWy, dWy_out, rec, ctrl, 0, 1, CFL, dt_max, INFINITY);
+  k_state_begin<<<1, 1, 0, s>>>(ctrl, 0.0, 1);
+  e = launch(true, k_load_cells<double>, dim3(blocks_of((size_t)nx * ny)), dim3(256), s, g, dU, C0, C1, ctrl);
   if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
-  e = launch_faces<double, double>(false, s, g, sms, rec, const_cast<double*>(dWx), dWx_out, const_cast<double*>(dWy),
+  e = launch_recon<double, double>(true, s, g, U0, U1, dWx, dWx_out, dWy, dWy_out, rec, ctrl, 0, 1, CFL, dt_max, INFINITY);
+  if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
+  e = launch_faces<double, double>(true, s, g, sms, rec, const_cast<double*>(dWx), dWx_out, const_cast<double*>(dWy),
                                    dWy_out, Fx, Fy, ctrl, 0);
   if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
   const UpdateArgs<double, double> ua{C0, C1, Fx, Fy, const_cast<double*>(dWx), dWx_out, const_cast<double*>(dWy), dWy_out, bad};
-  e = launch_update<double, double>(false, s, g, sms, ua, ctrl);
+  e = launch_update<double, double>(true, s, g, sms, ua, ctrl);
   if (e == cudaSuccess) e = launch_finish<double, double>(s, g, sms, ua, ctrl);
   if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
-  k_scatter_U<double><<<grid2(nx, ny, b2), b2, 0, s>>>(g, dU_out, C0, C1, ctrl, 0);
+  k_store_cells<double><<<blocks_of((size_t)nx * ny), 256, 0, s>>>(g, dU_out, C0, C1, ctrl);
   e = cudaGetLastError();
   Ctrl hc;
   if (e == cudaSuccess) e = cudaMemcpyAsync(&hc, ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s);

@@ -23,6 +23,7 @@
 #include "../../include/gks.h"
 #include "gks_device.cuh"
 #include "gks_grid.cuh"
+#include "gks_state.cuh"
 
 using namespace gks;
 
@@ -250,48 +251,6 @@ __global__ void __launch_bounds__(kThreads, BatchBlocks<R>::value) k_batch(Args<
     if (nsteps > 0) ctrl_end(&a.ctrl[g]);
 }
 
-// ---- per-grid state transfer ----
-template <class R>
-__global__ void kb_scatter(Geo g, const double* src, Cells<R> U, int to_dev) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
-  if (i >= g.nx || j >= g.ny) return;
-  for (int v = 0; v < 4; ++v) {
-    const size_t o = ((size_t)v * g.ny + j) * g.nx + i;
-    if (to_dev) U.set(g, v, i, j, src[o]);
-    else const_cast<double*>(src)[o] = U.get(g, v, i, j);
-  }
-}
-
-template <class R>
-__global__ void kb_ghost(Geo g, Cells<R> U) {
-  ghost_at<R>(g, U, blockIdx.x * blockDim.x + threadIdx.x);
-}
-
-template <class TW>
-__global__ void kb_copyW(const double* src, TW* W, size_t n, int to_dev) {
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  copy_w(src, W, n / 8, k, to_dev);
-}
-
-template <class R>
-__global__ void kb_dtbound(Geo g, Cells<R> U, Ctrl* c) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y * blockDim.y + threadIdx.y;
-  double inv = 0.0;
-  if (i < g.nx && j < g.ny) {
-    double w[4];
-    for (int v = 0; v < 4; ++v) w[v] = U.get(g, v, i, j);
-    bool ok;
-    inv = inv_bound<double>(g, w, ok);
-    if (!ok || !(inv < INFINITY)) {
-      atomicCAS(&c->status, GKS_OK, GKS_ENONPHYSICAL);
-      inv = 0.0;
-    }
-  }
-  block_bound_to<double>(inv, &c->bound);
-}
-
-dim3 grid2(int nx, int ny, dim3 b) { return dim3((nx + b.x - 1) / b.x, (ny + b.y - 1) / b.y); }
 
 }  // namespace
 
@@ -608,83 +567,104 @@ gks_status gks_batch_create(int n, const gks_grid_desc* grids, const gks_options
   return GKS_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// buffers of grid g
+template <class R> Cells<R> batch_cells(const gks_batch* b, int g, int k) { return Cells<R>{(R*)(b->U[k] + b->off[g].u)}; }
+template <class R> R* batch_wx(const gks_batch* b, int g, int k) { return (R*)b->Wx[k] + b->off[g].wx; }
+template <class R> R* batch_wy(const gks_batch* b, int g, int k) { return (R*)b->Wy[k] + b->off[g].wy; }
+
+size_t batch_fx(const Geo& G) { return (size_t)G.ny * (G.nx + 1); }
+size_t batch_fy(const Geo& G) { return (size_t)(G.ny + 1) * G.nx; }
+
+// host arrays in; page-locked ones are read in place, the others go through the staging buffer in turn
+template <class R>
+gks_status batch_load(gks_batch* b, int g, const double* U, const double* Wx, const double* Wy, double t) {
+  const Geo& G = b->geo[g];
+  cudaStream_t s = b->stream;
+  Ctrl* c = b->d_ctrl + g;
+  const size_t cells = (size_t)G.nx * G.ny, fx = batch_fx(G), fy = batch_fy(G);
+  auto faces = [&](const double* px, const double* py) {
+    k_face_values<R, true><<<blocks_of((px ? fx : 0) + (py ? fy : 0)), 256, 0, s>>>(
+        const_cast<double*>(px), const_cast<double*>(py), fx, fy, batch_wx<R>(b, g, 0), batch_wx<R>(b, g, 1),
+        batch_wy<R>(b, g, 0), batch_wy<R>(b, g, 1), c);
+  };
+  k_state_begin<<<1, 1, 0, s>>>(c, t, 0);
+  const double *mu = mapped_host(U), *mx = mapped_host(Wx), *my = mapped_host(Wy);
+  if (!mu) BCK(cudaMemcpyAsync(b->staging, U, 4 * cells * sizeof(double), cudaMemcpyHostToDevice, s));
+  k_load_cells<R><<<blocks_of(cells), 256, 0, s>>>(G, mu ? mu : b->staging, batch_cells<R>(b, g, 0), batch_cells<R>(b, g, 1), c);
+  if (!mx) {
+    BCK(cudaMemcpyAsync(b->staging, Wx, 8 * fx * sizeof(double), cudaMemcpyHostToDevice, s));
+    faces(b->staging, nullptr);
+  }
+  if (!my) {
+    BCK(cudaMemcpyAsync(b->staging, Wy, 8 * fy * sizeof(double), cudaMemcpyHostToDevice, s));
+    faces(nullptr, b->staging);
+  }
+  if (mx || my) faces(mx, my);
+  BCK(cudaGetLastError());
+  return GKS_OK;
+}
+
+template <class R>
+gks_status batch_store(gks_batch* b, int g, double* U, double* Wx, double* Wy) {
+  const Geo& G = b->geo[g];
+  cudaStream_t s = b->stream;
+  const Ctrl* c = b->d_ctrl + g;
+  const size_t cells = (size_t)G.nx * G.ny, fx = batch_fx(G), fy = batch_fy(G);
+  auto faces = [&](double* px, double* py) {
+    k_face_values<R, false><<<blocks_of((px ? fx : 0) + (py ? fy : 0)), 256, 0, s>>>(
+        px, py, fx, fy, batch_wx<R>(b, g, 0), batch_wx<R>(b, g, 1), batch_wy<R>(b, g, 0), batch_wy<R>(b, g, 1), c);
+  };
+  auto out = [](double* p) { return p ? const_cast<double*>(mapped_host(p)) : nullptr; };
+  double *mu = out(U), *mx = out(Wx), *my = out(Wy);
+  if (U) {
+    k_store_cells<R><<<blocks_of(cells), 256, 0, s>>>(G, mu ? mu : b->staging, batch_cells<R>(b, g, 0), batch_cells<R>(b, g, 1), c);
+    if (!mu) BCK(cudaMemcpyAsync(U, b->staging, 4 * cells * sizeof(double), cudaMemcpyDeviceToHost, s));
+  }
+  if (Wx && !mx) {
+    faces(b->staging, nullptr);
+    BCK(cudaMemcpyAsync(Wx, b->staging, 8 * fx * sizeof(double), cudaMemcpyDeviceToHost, s));
+  }
+  if (Wy && !my) {
+    faces(nullptr, b->staging);
+    BCK(cudaMemcpyAsync(Wy, b->staging, 8 * fy * sizeof(double), cudaMemcpyDeviceToHost, s));
+  }
+  if (mx || my) faces(mx, my);
+  BCK(cudaGetLastError());
+  return GKS_OK;
+}
+
+// the control block of grid g into the host's mirror
+gks_status batch_read_ctrl(gks_batch* b, int g) {
+  BCK(cudaMemcpyAsync(&b->h_ctrl[g], b->d_ctrl + g, sizeof(Ctrl), cudaMemcpyDeviceToHost, b->stream));
+  BCK(cudaStreamSynchronize(b->stream));
+  return GKS_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 gks_status gks_batch_set_state(gks_batch* b, int g, const double* U, const double* Wx, const double* Wy, double t) {
   if (!b || g < 0 || g >= b->G || !U || !Wx || !Wy) return bfail(b, GKS_EINVAL, "gks_batch_set_state: bad argument");
   BCK(cudaSetDevice(b->device));
-  const Geo& G = b->geo[g];
-  const GridOff& o = b->off[g];
-  Ctrl& c = b->h_ctrl[g];
-  BCK(cudaMemcpyAsync(&c, b->d_ctrl + g, sizeof(Ctrl), cudaMemcpyDeviceToHost, b->stream));
-  BCK(cudaStreamSynchronize(b->stream));
-  const int par = (int)(c.steps & 1);
-  const dim3 b2(32, 8);
-  BCK(cudaMemcpyAsync(b->staging, U, (size_t)4 * G.nx * G.ny * sizeof(double), cudaMemcpyHostToDevice, b->stream));
-  if (b->prec == GKS_FP64) {
-    const Cells<double> C{b->U[par] + o.u};
-    kb_scatter<double><<<grid2(G.nx, G.ny, b2), b2, 0, b->stream>>>(G, b->staging, C, 1);
-    kb_ghost<double><<<(perimeter(G) + 127) / 128, 128, 0, b->stream>>>(G, C);
-  } else {
-    const Cells<float> C{(float*)(b->U[par] + o.u)};
-    kb_scatter<float><<<grid2(G.nx, G.ny, b2), b2, 0, b->stream>>>(G, b->staging, C, 1);
-    kb_ghost<float><<<(perimeter(G) + 127) / 128, 128, 0, b->stream>>>(G, C);
-  }
-  const size_t nx = (size_t)8 * G.ny * (G.nx + 1), ny = (size_t)8 * (G.ny + 1) * G.nx;
-  BCK(cudaMemcpyAsync(b->staging, Wx, nx * sizeof(double), cudaMemcpyHostToDevice, b->stream));
-  if (b->prec == GKS_FP64) kb_copyW<double><<<(unsigned)((nx + 255) / 256), 256, 0, b->stream>>>(b->staging, (double*)b->Wx[par] + o.wx, nx, 1);
-  else kb_copyW<float><<<(unsigned)((nx + 255) / 256), 256, 0, b->stream>>>(b->staging, (float*)b->Wx[par] + o.wx, nx, 1);
-  BCK(cudaMemcpyAsync(b->staging, Wy, ny * sizeof(double), cudaMemcpyHostToDevice, b->stream));
-  if (b->prec == GKS_FP64) kb_copyW<double><<<(unsigned)((ny + 255) / 256), 256, 0, b->stream>>>(b->staging, (double*)b->Wy[par] + o.wy, ny, 1);
-  else kb_copyW<float><<<(unsigned)((ny + 255) / 256), 256, 0, b->stream>>>(b->staging, (float*)b->Wy[par] + o.wy, ny, 1);
-  // control block: time t, status cleared, bound of the new state
-  c.t = t;
-  c.status = GKS_OK;
-  c.skip = 0;
-  const double inf = INFINITY;
-  memcpy(&c.bound, &inf, 8);
-  BCK(cudaMemcpyAsync(b->d_ctrl + g, &c, sizeof(Ctrl), cudaMemcpyHostToDevice, b->stream));
-  if (b->prec == GKS_FP64)
-    kb_dtbound<double><<<grid2(G.nx, G.ny, b2), b2, 0, b->stream>>>(G, Cells<double>{b->U[par] + o.u}, b->d_ctrl + g);
-  else
-    kb_dtbound<float><<<grid2(G.nx, G.ny, b2), b2, 0, b->stream>>>(G, Cells<float>{(float*)(b->U[par] + o.u)},
-                                                                   b->d_ctrl + g);
-  BCK(cudaGetLastError());
-  BCK(cudaMemcpyAsync(&c, b->d_ctrl + g, sizeof(Ctrl), cudaMemcpyDeviceToHost, b->stream));
-  BCK(cudaStreamSynchronize(b->stream));
-  if (c.status != GKS_OK) return bfail(b, GKS_ENONPHYSICAL, "gks_batch_set_state: state has rho <= 0 or p <= 0");
+  gks_status st = b->prec == GKS_FP64 ? batch_load<double>(b, g, U, Wx, Wy, t) : batch_load<float>(b, g, U, Wx, Wy, t);
+  if (st == GKS_OK) st = batch_read_ctrl(b, g);
+  if (st != GKS_OK) return st;
+  if (b->h_ctrl[g].status != GKS_OK) return bfail(b, GKS_ENONPHYSICAL, "gks_batch_set_state: state has rho <= 0 or p <= 0");
   return GKS_OK;
 }
 
 gks_status gks_batch_get_state(gks_batch* b, int g, double* U, double* Wx, double* Wy, double* t, long long* steps) {
   if (!b || g < 0 || g >= b->G) return bfail(b, GKS_EINVAL, "gks_batch_get_state: bad argument");
   BCK(cudaSetDevice(b->device));
-  const Geo& G = b->geo[g];
-  const GridOff& o = b->off[g];
-  Ctrl& c = b->h_ctrl[g];
-  BCK(cudaMemcpyAsync(&c, b->d_ctrl + g, sizeof(Ctrl), cudaMemcpyDeviceToHost, b->stream));
-  BCK(cudaStreamSynchronize(b->stream));
-  const int par = (int)(c.steps & 1);
-  const dim3 b2(32, 8);
-  if (U) {
-    if (b->prec == GKS_FP64)
-      kb_scatter<double><<<grid2(G.nx, G.ny, b2), b2, 0, b->stream>>>(G, b->staging, Cells<double>{b->U[par] + o.u}, 0);
-    else
-      kb_scatter<float><<<grid2(G.nx, G.ny, b2), b2, 0, b->stream>>>(G, b->staging,
-                                                                     Cells<float>{(float*)(b->U[par] + o.u)}, 0);
-    BCK(cudaMemcpyAsync(U, b->staging, (size_t)4 * G.nx * G.ny * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
-  }
-  const size_t nx = (size_t)8 * G.ny * (G.nx + 1), ny = (size_t)8 * (G.ny + 1) * G.nx;
-  if (Wx) {
-    if (b->prec == GKS_FP64) kb_copyW<double><<<(unsigned)((nx + 255) / 256), 256, 0, b->stream>>>(b->staging, (double*)b->Wx[par] + o.wx, nx, 0);
-    else kb_copyW<float><<<(unsigned)((nx + 255) / 256), 256, 0, b->stream>>>(b->staging, (float*)b->Wx[par] + o.wx, nx, 0);
-    BCK(cudaMemcpyAsync(Wx, b->staging, nx * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
-  }
-  if (Wy) {
-    if (b->prec == GKS_FP64) kb_copyW<double><<<(unsigned)((ny + 255) / 256), 256, 0, b->stream>>>(b->staging, (double*)b->Wy[par] + o.wy, ny, 0);
-    else kb_copyW<float><<<(unsigned)((ny + 255) / 256), 256, 0, b->stream>>>(b->staging, (float*)b->Wy[par] + o.wy, ny, 0);
-    BCK(cudaMemcpyAsync(Wy, b->staging, ny * sizeof(double), cudaMemcpyDeviceToHost, b->stream));
-  }
-  BCK(cudaGetLastError());
-  BCK(cudaStreamSynchronize(b->stream));
+  gks_status st = b->prec == GKS_FP64 ? batch_store<double>(b, g, U, Wx, Wy) : batch_store<float>(b, g, U, Wx, Wy);
+  if (st == GKS_OK) st = batch_read_ctrl(b, g);
+  if (st != GKS_OK) return st;
+  const Ctrl& c = b->h_ctrl[g];
   if (t) *t = c.t;
   if (steps) *steps = c.steps;
   if (c.status != GKS_OK) return bfail(b, (gks_status)c.status, "grid state is the last good one");

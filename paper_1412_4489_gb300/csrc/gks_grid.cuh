@@ -104,16 +104,16 @@ template <> struct Lay<double> {
 #pragma unroll
     for (int v = 0; v < 4; ++v) p[f(n, v, o)] = x[v];
   }
-  static __device__ __forceinline__ void load_rec(const double* p, double r[kRec]) {
-    const double2* q = reinterpret_cast<const double2*>(p);
+  static __device__ __forceinline__ void load_rec(const double* p, size_t c, double r[kRec]) {
+    const double2* q = reinterpret_cast<const double2*>(p + c * kRec);
 #pragma unroll
     for (int k = 0; k < kRec / 2; ++k) {
       const double2 t = q[k];
       r[2 * k] = t.x; r[2 * k + 1] = t.y;
     }
   }
-  static __device__ __forceinline__ void load_avg(const double* p, double r[4]) {
-    const double2* q = reinterpret_cast<const double2*>(p);
+  static __device__ __forceinline__ void load_avg(const double* p, size_t c, double r[4]) {
+    const double2* q = reinterpret_cast<const double2*>(p + c * kRec);
     const double2 a = q[0], b = q[1];
     r[0] = a.x; r[1] = a.y; r[2] = b.x; r[3] = b.y;
   }
@@ -144,11 +144,11 @@ template <> struct Lay<float> {
   static __device__ __forceinline__ void load_f(const float* p, size_t, size_t o, float x[4]) { get(p, o, x); }
   static __device__ __forceinline__ void store_w(float* p, size_t n, int q, size_t o, const float x[4]) { put(p, q * n + o, x); }
   static __device__ __forceinline__ void store_f(float* p, size_t, size_t o, const float x[4]) { put(p, o, x); }
-  static __device__ __forceinline__ void load_rec(const float* p, float r[kRec]) {
+  static __device__ __forceinline__ void load_rec(const float* p, size_t c, float r[kRec]) {
 #pragma unroll
-    for (int k = 0; k < kRec / 4; ++k) get(p, k, r + 4 * k);
+    for (int k = 0; k < kRec / 4; ++k) get(p, c * (kRec / 4) + k, r + 4 * k);
   }
-  static __device__ __forceinline__ void load_avg(const float* p, float r[4]) { get(p, 0, r); }
+  static __device__ __forceinline__ void load_avg(const float* p, size_t c, float r[4]) { get(p, c * (kRec / 4), r); }
   static __device__ __forceinline__ void store_rec(float* p, size_t c, const float r[kRec]) {
 #pragma unroll
     for (int k = 0; k < kRec / 4; ++k) put(p, c * (kRec / 4) + k, r + 4 * k);
@@ -278,15 +278,6 @@ __device__ __forceinline__ void df_add_product(float& hi, float& lo, float f, fl
   const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(p, bb));
   hi = s;
   lo = __fadd_rn(lo, __fadd_rn(e, pe));
-}
-
-// value k of the caller's face-value planes [4][2][faces] to (to_dev) or from the layout of the type
-template <class TW>
-__device__ __forceinline__ void copy_w(const double* src, TW* W, size_t faces, size_t k, int to_dev) {
-  const size_t q = k / faces;
-  const size_t at = Lay<TW>::w(faces, (int)(q >> 1), (int)(q & 1), k - q * faces);
-  if (to_dev) W[at] = (TW)src[k];
-  else const_cast<double*>(src)[k] = (double)W[at];
 }
 
 // Programmatic dependent launch: a step kernel launched with programmatic stream
@@ -671,10 +662,10 @@ template <int AX> __device__ __forceinline__ int slot(int v) { return AX == 0 ? 
 // value and derivatives of a cell's polynomial (its record) at the centre of its face
 // on side s (+1: the face at +h_n/2, -1: at -h_n/2), in the face frame of axis AX
 template <int AX, class R>
-__device__ __forceinline__ void side_state(const R* __restrict__ record, int s, R hn, R hn2_12, R ht2_24,
+__device__ __forceinline__ void side_state(const R* __restrict__ rec, size_t c, int s, R hn, R hn2_12, R ht2_24,
                                            FaceState<R>& S) {
   R r[kRec];
-  Lay<R>::load_rec(record, r);
+  Lay<R>::load_rec(rec, c, r);
 #pragma unroll
   for (int v = 0; v < 4; ++v) {
     const R c = r[v];
@@ -693,10 +684,13 @@ __device__ __forceinline__ void side_state(const R* __restrict__ record, int s, 
 }
 
 // Inputs of one face, fetched on demand by face_evolution
-template <int AX, class R>
+// INDEXED: each record at its own index instead of from the face's base address.  FP32 batches use it: their
+// results stay bit for bit the same, and the compiler contracts the routine's sums differently otherwise.
+template <int AX, class R, bool INDEXED = false>
 struct GridFaceSource {
   const Geo* g;
   const R* U;    // padded compute-type averages (the first-order fallback's constant states)
+  const R* rec;  // reconstruction records
   const R* at;   // record of cell (i, j): the others lie at fixed distances, so one address serves a face
   int to_l, to_r;  // from there to the records of the cells cl and cr, in records (a grid that fits the
                    // memory has far fewer than 2^31)
@@ -711,6 +705,12 @@ struct GridFaceSource {
   __device__ __forceinline__ void image(int kind, R uwt, R Tw, const FaceState<R>& in, FaceState<R>& out) const {
     if (kind == GKS_BC_OUTFLOW) out = in;
     else wall_image<R>(kind, gamma, uwt, Tw, in, out);
+  }
+
+  // state at this face of cell n along the normal, `to` records from (i, j)'s, on its side s
+  __device__ __forceinline__ void cell_state(int n, int to, int s, FaceState<R>& S) const {
+    if constexpr (INDEXED) side_state<AX>(rec, rec_at(*g, cx(n), cy(n)), s, hn, hn2_12, ht2_24, S);
+    else side_state<AX>(at + (ptrdiff_t)to * kRec, 0, s, hn, hn2_12, ht2_24, S);
   }
 
   bool first_order;  // constant states (cell averages) for the positivity fallback
@@ -749,18 +749,18 @@ struct GridFaceSource {
     if (k == 0) {
       if (img_lo) {
         FaceState<R> in;
-        side_state<AX>(at + (ptrdiff_t)to_r * kRec, -1, hn, hn2_12, ht2_24, in);
+        cell_state(cr, to_r, -1, in);
         image(img_lo, uwt_lo, Tw_lo, in, S);
       } else {
-        side_state<AX>(at + (ptrdiff_t)to_l * kRec, +1, hn, hn2_12, ht2_24, S);
+        cell_state(cl, to_l, +1, S);
       }
     } else {
       if (img_hi) {
         FaceState<R> in;
-        side_state<AX>(at + (ptrdiff_t)to_l * kRec, +1, hn, hn2_12, ht2_24, in);
+        cell_state(cl, to_l, +1, in);
         image(img_hi, uwt_hi, Tw_hi, in, S);
       } else {
-        side_state<AX>(at + (ptrdiff_t)to_r * kRec, -1, hn, hn2_12, ht2_24, S);
+        cell_state(cr, to_r, -1, S);
       }
     }
   }
@@ -774,7 +774,8 @@ struct GridFaceSource {
       for (int k = 0; k < 3; ++k) {
         const int di = (AX == 0 ? m : k) - 1, dj = (AX == 0 ? k : m) - 1;
         R w[4];
-        Lay<R>::load_avg(at + dj * row + di * kRec, w);
+        if constexpr (INDEXED) Lay<R>::load_avg(rec, rec_at(*g, i + di, j + dj), w);
+        else Lay<R>::load_avg(at + dj * row + di * kRec, 0, w);
 #pragma unroll
         for (int v = 0; v < 4; ++v) a[m][k][slot<AX>(v)] = w[v];
       }
@@ -804,11 +805,12 @@ __host__ __device__ inline FaceConst<R> grid_face_const(const Geo& g, int axis) 
 }
 
 // the inputs of face (i, j) of axis AX; U (may be null) serves constant states only
-template <int AX, class R>
-__device__ __forceinline__ GridFaceSource<AX, R> face_source(const Geo& g, const R* U, const R* rec, int i, int j) {
-  GridFaceSource<AX, R> src;
+template <int AX, class R, bool INDEXED = false>
+__device__ __forceinline__ GridFaceSource<AX, R, INDEXED> face_source(const Geo& g, const R* U, const R* rec, int i, int j) {
+  GridFaceSource<AX, R, INDEXED> src;
   src.g = &g;
   src.U = U;
+  src.rec = rec;
   src.at = rec + rec_at(g, i, j) * kRec;
   src.i = i;
   src.j = j;
@@ -842,9 +844,10 @@ __device__ __forceinline__ GridFaceSource<AX, R> face_source(const Geo& g, const
 }
 
 // the same with the cell sizes that a polynomial's face state needs
-template <int AX, class R>
-__device__ __forceinline__ GridFaceSource<AX, R> face_source(const Geo& g, const FaceConst<R>& C, const R* rec, int i, int j) {
-  GridFaceSource<AX, R> src = face_source<AX, R>(g, (const R*)nullptr, rec, i, j);
+template <int AX, class R, bool INDEXED = false>
+__device__ __forceinline__ GridFaceSource<AX, R, INDEXED> face_source(const Geo& g, const FaceConst<R>& C, const R* rec, int i,
+                                                                      int j) {
+  GridFaceSource<AX, R, INDEXED> src = face_source<AX, R, INDEXED>(g, (const R*)nullptr, rec, i, j);
   src.hn = C.dn;
   src.ht = C.dtan;
   src.hn2_12 = C.dn2_12;
@@ -854,8 +857,8 @@ __device__ __forceinline__ GridFaceSource<AX, R> face_source(const Geo& g, const
 }
 
 // the wall's flux rule, then flux and point values to memory in physical components
-template <int AX, class R, class TW>
-__device__ __forceinline__ void store_face(const Geo& g, const GridFaceSource<AX, R>& src, TW* __restrict__ Wn,
+template <int AX, class R, class TW, bool INDEXED>
+__device__ __forceinline__ void store_face(const Geo& g, const GridFaceSource<AX, R, INDEXED>& src, TW* __restrict__ Wn,
                                            R* __restrict__ F, R Fl[4], const R Wm[4], const R Wp[4]) {
   if (src.img_lo) wall_face_flux<R>(src.img_lo, src.uwt_lo, Fl);
   else if (src.img_hi) wall_face_flux<R>(src.img_hi, src.uwt_hi, Fl);
@@ -879,7 +882,7 @@ __device__ __forceinline__ void store_face(const Geo& g, const GridFaceSource<AX
 template <int AX, class R, class TW, int NSM = -1, bool MONO = false>
 __device__ __forceinline__ void flux_face(const Geo& g, const FaceConst<R>& C, const R* __restrict__ rec,
                                           TW* __restrict__ Wn, R* __restrict__ F, int i, int j, R dt) {
-  const GridFaceSource<AX, R> src = face_source<AX, R>(g, C, rec, i, j);
+  const GridFaceSource<AX, R, MONO> src = face_source<AX, R, MONO>(g, C, rec, i, j);
   R Fl[4], Wm[4], Wp[4];
   if constexpr (MONO) monomials::face_evolution<R, NSM>(C, src, dt, Fl, Wm, Wp);
   else face_evolution<R, NSM>(C, src, dt, Fl, Wm, Wp);
@@ -997,6 +1000,20 @@ __device__ __forceinline__ R inv_bound(const Geo& g, const R w[4], bool& ok) {
   return inv;
 }
 
+// FP32 proof that an FP64 state is physical and its inverse CFL bound below `below`: rho > 0, the pressure
+// above the rounding of its terms, and the bound with a margin of 1e-4.  false where FP32 cannot tell
+// (near-vacuum states, values outside FP32's range, NaN).
+__device__ __forceinline__ bool surely_below(const Geo& g, const double w[4], float below) {
+  const float r = (float)w[0], m = (float)w[1], n = (float)w[2], e = (float)w[3];
+  const float ir = __fdividef(1.0f, r), u = m * ir, v = n * ir, kin = 0.5f * (m * u + n * v);
+  const float p = g.gm1_f * (e - kin);
+  const float c = sqrtf(g.gamma_f * p * ir);
+  float inv = fmaxf((fabsf(u) + c) * g.idx_hi, (fabsf(v) + c) * g.idy_hi);
+  if (g.visc_on) inv = fmaxf(inv, g.visc_f * ir);
+  // density and energy well inside FP32's range; c rounds to 1e-3 relative where p > 1e-3 (e + kin) gm1
+  return r > 1e-18f && r < 1e18f && e < 1e18f && p > 1e-3f * g.gm1_f * (e + kin) && inv > 1e-18f && 1.001f * inv < below;
+}
+
 // warp maximum of inv, then the atomic minimum of the bound 1/inv (no block
 // barrier: the warps of a block go on independently).  Every lane of the warp must
 // call it.
@@ -1099,6 +1116,20 @@ __device__ __forceinline__ void store_state(const Geo& g, Cells<float> U, int i,
   Lay<float>::put(U.p, cell_at(g, i, j), s.hi);
   Lay<float>::put(U.p + 4 * g.plane, cell_at(g, i, j), s.lo);
 }
+
+// an FP64 value as the state holds it in variable v; returns what the state then stands for
+__device__ __forceinline__ double split_value(double w, CellState<double>& s, int v) {
+  s.w[v] = w;
+  return w;
+}
+__device__ __forceinline__ double split_value(double w, CellState<float>& s, int v) {
+  const float hi = (float)w, lo = (float)(w - (double)hi);
+  s.hi[v] = hi;
+  s.lo[v] = lo;
+  return (double)hi + (double)lo;
+}
+__device__ __forceinline__ double whole_value(const CellState<double>& s, int v) { return s.w[v]; }
+__device__ __forceinline__ double whole_value(const CellState<float>& s, int v) { return (double)s.hi[v] + (double)s.lo[v]; }
 
 // Eq. finite for one variable: FP64 planes take the FP32 or FP64 fluxes in
 // FP64 (differences of FP32 numbers are exact there); the double-float pair
