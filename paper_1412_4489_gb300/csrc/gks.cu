@@ -117,9 +117,17 @@ __global__ void __launch_bounds__(32 * ReconRows<R>::value, ReconBlocks<R, CHAR>
   }
 }
 
-// FP64 in conservative variables: four lanes to a cell (recon_cell_lanes), eight cells to a one-warp block,
+// Warps to a block of the FP64 kernels, whose pipe serves a warp instruction for a quarter of an SM in 64 cycles
+// whether its lanes are active or not: as many as spread all warps over the SMs in one block each, at most four, one
+// for each quarter (one-warp blocks end up two to a quarter while others idle).
+unsigned warps_per_block(unsigned long long warps, int sms) {
+  const unsigned long long w = (warps + sms - 1) / sms;
+  return w < 1 ? 1 : w > 4 ? 4 : (unsigned)w;
+}
+
+// FP64 in conservative variables: four lanes to a cell (recon_cell_lanes), eight cells to a warp,
 // numbered through row by row
-__global__ void __launch_bounds__(32, 16) k_recon_lanes(Geo g, const double* U0, const double* U1, const double* Wx0,
+__global__ void __launch_bounds__(128, 6) k_recon_lanes(Geo g, const double* U0, const double* U1, const double* Wx0,
                                                         const double* Wx1, const double* Wy0, const double* Wy1,
                                                         double* __restrict__ rec, Ctrl* c, int force, int begin,
                                                         double cfl, double dt_max, double t_end) {
@@ -129,7 +137,7 @@ __global__ void __launch_bounds__(32, 16) k_recon_lanes(Geo g, const double* U0,
   } else if (!force && c->skip) {
     return;
   }
-  const unsigned long long n = (unsigned long long)g.nx * g.ny, k = (unsigned long long)blockIdx.x * 8 + (threadIdx.x >> 2);
+  const unsigned long long n = (unsigned long long)g.nx * g.ny, k = (unsigned long long)blockIdx.x * (blockDim.x >> 2) + (threadIdx.x >> 2);
   const unsigned long long q = k < n ? k : n - 1;
   const int j = (int)(q / (unsigned)g.nx), i = (int)(q - (unsigned long long)j * g.nx);
   const int par = (int)(c->steps & 1);
@@ -204,12 +212,10 @@ __global__ void __launch_bounds__(128, FluxBlocks<0>::value) k_flux_euler(Geo g,
   }
 }
 
-// FP64: every face of the grid in one launch, 32 to a block, x-faces in blocks [0, nbx), y-faces after
-// them, numbered through row by row.  The FP64 pipe serves a warp instruction for a quarter of an SM in 64 cycles
-// whether its lanes are active or not, so what counts is full warps spread evenly over the quarters: one-warp
-// blocks without idle lanes at the rows' ends, and no second launch with a tail of its own.  (Instruction fetch,
-// which speaks against mixing the two axes' bodies in FP32, does not matter at this pace.)
-// first: the first block's number (a launch can take one axis alone).
+// FP64: every face of the grid in one launch, 32 to a warp, x-faces in warps [0, nbx), y-faces after
+// them, numbered through row by row: no idle lanes at the rows' ends, and no second launch with a tail of its own.
+// (Instruction fetch, which speaks against mixing the two axes' bodies in FP32, does not matter at the FP64 pipe's
+// pace.)  first: the first warp's number (a launch can take one axis alone).
 template <int AX>
 __device__ __forceinline__ bool face_at(const Geo& g, unsigned block, int lane, int& i, int& j) {
   const unsigned fx = AX == 0 ? g.nx + 1 : g.nx, fy = AX == 0 ? g.ny : g.ny + 1;
@@ -221,17 +227,17 @@ __device__ __forceinline__ bool face_at(const Geo& g, unsigned block, int lane, 
 }
 
 template <class R, class TW, int NS>
-__global__ void __launch_bounds__(32, 8) k_faces(Geo g, FaceArgs<R, TW> a, const Ctrl* c, int force) {
+__global__ void __launch_bounds__(128, 2) k_faces(Geo g, FaceArgs<R, TW> a, const Ctrl* c, int force) {
   pdl_enter();
   if (!force && c->skip) return;
-  const unsigned b = blockIdx.x + a.first;
+  const unsigned b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5) + a.first, lane = threadIdx.x & 31;
   const int par = (int)(c->steps & 1);
   const R dt = step_dt<R>(c);
   int i, j;
   if (b < a.nbx) {
-    if (face_at<0>(g, b, threadIdx.x, i, j))
+    if (face_at<0>(g, b, lane, i, j))
       flux_face<0, R, TW, NS>(g, a.Cx, a.rec, par ? a.Wx0 : a.Wx1, a.Fx, i, j, dt);
-  } else if (face_at<1>(g, b - a.nbx, threadIdx.x, i, j)) {
+  } else if (face_at<1>(g, b - a.nbx, lane, i, j)) {
     flux_face<1, R, TW, NS>(g, a.Cy, a.rec, par ? a.Wy0 : a.Wy1, a.Fy, i, j, dt);
   }
 }
@@ -257,9 +263,12 @@ __global__ void __launch_bounds__(96, 2) k_faces_split(Geo g, FaceArgs<R, TW> a,
 }
 
 // Grids of at most kSplitWarps face warps per SM (both axes) take the split launch.  Step times, one warp / three
-// warps (us, Euler): 32^2 89 / 73, 64^2 (1.7 warps per SM) 90 / 80, 70^2 (2.0) 89 / 91, 100^2
-// 109 / 111; Navier-Stokes: 107 / 80, 107 / 91, 109 / 108, 140 / 149.
-constexpr unsigned kSplitWarps = 2;
+// warps to 32 faces (us): Euler 32^2 48 / 32, 69^2 (2.0 warps per SM) 49 / 38, 81^2 (2.7) 53 / 51, 96^2
+// (3.8) 56 / 57; Navier-Stokes 66 / 38, 67 / 51, 72 / 70, 76 / 89.
+constexpr unsigned kSplitWarps = 3;
+
+// cells up to which the FP32 Euler faces are launched with programmatic serialisation
+constexpr size_t kPdlCells = 1u << 17;
 
 // ---------------------------------------------------------------------------
 // update, CFL bound of the new state, physical check
@@ -374,10 +383,8 @@ __global__ void __launch_bounds__(256, UpdateBlocks<R>::value) k_finish(Geo g, U
 // blocks (blocks_per_sm per SM), each walking ceil(tiles / wave) tiles along y, so
 // that the per-block work (control reads, the CFL reduction) is shared by its tiles;
 // the fallback passes at most one block per SM (usually no work).  Pass 1 of the FP64 form takes
-// one-warp blocks (rows = 1): its bound is the FP64 pipe, which wants the warps of a small grid spread over all SMs
-// (81^2 in 256-thread blocks keeps 33 of 152 SMs busy).
+// warps_per_block rows: its bound is the FP64 pipe too (81^2 in 256-thread blocks keeps 33 of 152 SMs busy).
 constexpr int kUpdateRows = 8;
-template <class R> constexpr int update_rows(int pass) { return pass == 1 && sizeof(R) == 8 ? 1 : kUpdateRows; }
 
 dim3 update_grid(const Geo& g, int pass, int sms, int blocks_per_sm, int rows) {
   unsigned tx = (unsigned)((g.nx + 31) / 32), ty = (unsigned)((g.ny + rows - 1) / rows);
@@ -534,7 +541,8 @@ void launch_ghost(gks_handle* h, int force) {
 
 template <class R, class TW>
 cudaError_t launch_update(bool pdl, cudaStream_t s, const Geo& g, int sms, const UpdateArgs<R, TW>& a, Ctrl* c) {
-  const int rows = update_rows<R>(1);
+  const int rows = sizeof(R) == 8 ? (int)warps_per_block((unsigned long long)((g.nx + 31) / 32) * g.ny, sms) : kUpdateRows;
+  if (sizeof(R) == 8) pdl = false;  // as the faces (launch_faces): 128^2 97.6 -> 92.2 us a step
   return launch(pdl, k_update<R, TW>, update_grid(g, 1, sms, UpdateBlocks<R>::value, rows), dim3(32, rows), s, g, a, c);
 }
 
@@ -555,12 +563,14 @@ cudaError_t launch_finish(cudaStream_t s, const Geo& g, int sms, const UpdateArg
 }
 
 template <class R, class TW>
-cudaError_t launch_recon(bool pdl, cudaStream_t s, const Geo& g, const R* U0, const R* U1, const TW* Wx0, const TW* Wx1,
+cudaError_t launch_recon(bool pdl, cudaStream_t s, const Geo& g, int sms, const R* U0, const R* U1, const TW* Wx0, const TW* Wx1,
                          const TW* Wy0, const TW* Wy1, R* rec, Ctrl* c, int force, int begin, double cfl, double dt_max,
                          double t_end) {
   if constexpr (sizeof(R) == 8) {
+    const unsigned long long warps = ((unsigned long long)g.nx * g.ny + 7) / 8;
+    const unsigned w = warps_per_block(warps, sms);
     if (!g.characteristic)
-      return launch(pdl, k_recon_lanes, dim3((unsigned)(((unsigned long long)g.nx * g.ny + 7) / 8)), dim3(32), s, g, U0, U1,
+      return launch(pdl, k_recon_lanes, dim3((unsigned)((warps + w - 1) / w)), dim3(32 * w), s, g, U0, U1,
                     Wx0, Wx1, Wy0, Wy1, rec, c, force, begin, cfl, dt_max, t_end);
     const dim3 b(32, ReconRows<R>::value);
     // block rows beyond the grid's y limit continue in z
@@ -578,13 +588,15 @@ cudaError_t launch_recon(bool pdl, cudaStream_t s, const Geo& g, const R* U0, co
 template <class R, class TW>
 cudaError_t launch_recon(gks_handle* h, int force, int begin = 0, double cfl = 0, double dt_max = 0,
                          double t_end = 0, bool pdl = false) {
-  return launch_recon<R, TW>(pdl, h->stream, h->g, cells<R>(h, 0), cells<R>(h, 1), (const TW*)h->Wx[0], (const TW*)h->Wx[1],
+  return launch_recon<R, TW>(pdl, h->stream, h->g, h->sms, cells<R>(h, 0), cells<R>(h, 1), (const TW*)h->Wx[0], (const TW*)h->Wx[1],
                              (const TW*)h->Wy[0], (const TW*)h->Wy[1], (R*)h->rec, h->ctrl, force, begin, cfl, dt_max, t_end);
 }
 
-// the FP64 face launch over both axes (axes 3) or one of them (1: x, 2: y)
+// The FP64 face launch over both axes (axes 3) or one of them (1: x, 2: y).  Without programmatic serialisation: blocks
+// placed while the reconstruction's are still resident pile up on some SMs, and the fullest SM is the
+// kernel's time (64^2 split 64 -> 38 us a step).
 template <class R, class TW>
-cudaError_t launch_faces(bool pdl, cudaStream_t s, const Geo& g, int sms, const R* rec, TW* Wx0, TW* Wx1, TW* Wy0, TW* Wy1,
+cudaError_t launch_faces(cudaStream_t s, const Geo& g, int sms, const R* rec, TW* Wx0, TW* Wx1, TW* Wy0, TW* Wy1,
                          R* Fx, R* Fy, const Ctrl* c, int force, int axes = 3) {
   const unsigned nbx = (unsigned)(((unsigned long long)(g.nx + 1) * g.ny + 31) / 32);
   const unsigned nby = (unsigned)(((unsigned long long)g.nx * (g.ny + 1) + 31) / 32);
@@ -592,8 +604,9 @@ cudaError_t launch_faces(bool pdl, cudaStream_t s, const Geo& g, int sms, const 
   const unsigned n = (axes & 1 ? nbx : 0) + (axes & 2 ? nby : 0);
   const bool ns = g.mu > 0.0, split = (unsigned long long)nbx + nby <= (unsigned long long)kSplitWarps * sms;
   if (split)
-    return launch(pdl, ns ? k_faces_split<R, TW, 1> : k_faces_split<R, TW, 0>, dim3(n), dim3(96), s, g, a, c, force);
-  return launch(pdl, ns ? k_faces<R, TW, 1> : k_faces<R, TW, 0>, dim3(n), dim3(32), s, g, a, c, force);
+    return launch(false, ns ? k_faces_split<R, TW, 1> : k_faces_split<R, TW, 0>, dim3(n), dim3(96), s, g, a, c, force);
+  const unsigned w = warps_per_block(n, sms);
+  return launch(false, ns ? k_faces<R, TW, 1> : k_faces<R, TW, 0>, dim3((n + w - 1) / w), dim3(32 * w), s, g, a, c, force);
 }
 
 // ev (optional, kProfileParts + 1 events): recorded before each kernel and after the last.
@@ -622,7 +635,7 @@ gks_status launch_step_kernels(gks_handle* h, double cfl, double dt_max, double 
   bool fork = false;
   if constexpr (sizeof(R) == 8) {
     auto faces = [&](int axes) {
-      keep(launch_faces<R, TW>(pdl, s, g, h->sms, (const R*)h->rec, (TW*)h->Wx[0], (TW*)h->Wx[1], (TW*)h->Wy[0],
+      keep(launch_faces<R, TW>(s, g, h->sms, (const R*)h->rec, (TW*)h->Wx[0], (TW*)h->Wx[1], (TW*)h->Wy[0],
                                (TW*)h->Wy[1], (R*)h->Fx, (R*)h->Fy, (const Ctrl*)h->ctrl, force, axes));
     };
     if (ev) faces(1);
@@ -659,7 +672,9 @@ gks_status launch_step_kernels(gks_handle* h, double cfl, double dt_max, double 
       auto faces = [&](int axes) {
         const FaceArgs<R, TW> a{fconst<R>(g, 0), fconst<R>(g, 1), (const R*)h->rec, (TW*)h->Wx[0], (TW*)h->Wx[1],
                                 (TW*)h->Wy[0], (TW*)h->Wy[1], (R*)h->Fx, (R*)h->Fy, nbx, axes == 2 ? nbx : 0};
-        keep(launch(pdl, k_flux_euler, dim3((axes & 1 ? nbx : 0) + (axes & 2 ? nby : 0)), bf, s, g, a, (const Ctrl*)h->ctrl,
+        // without programmatic serialisation on larger grids: blocks that wait on an SM take its slots from the
+        // reconstruction's last ones (2048^2 599 -> 587 us a step, 256^2 19.0 -> 19.8)
+        keep(launch(pdl && (size_t)g.nx * g.ny <= kPdlCells, k_flux_euler, dim3((axes & 1 ? nbx : 0) + (axes & 2 ? nby : 0)), bf, s, g, a, (const Ctrl*)h->ctrl,
                     force));
       };
       if (ev) faces(1);
@@ -1326,9 +1341,9 @@ extern "C" gks_status gks_step_noalloc(int nx, int ny, double Lx, double Ly, dou
   k_state_begin<<<1, 1, 0, s>>>(ctrl, 0.0, 1);
   e = launch(true, k_load_cells<double>, dim3(blocks_of((size_t)nx * ny)), dim3(256), s, g, dU, C0, C1, ctrl);
   if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
-  e = launch_recon<double, double>(true, s, g, U0, U1, dWx, dWx_out, dWy, dWy_out, rec, ctrl, 0, 1, CFL, dt_max, INFINITY);
+  e = launch_recon<double, double>(true, s, g, sms, U0, U1, dWx, dWx_out, dWy, dWy_out, rec, ctrl, 0, 1, CFL, dt_max, INFINITY);
   if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
-  e = launch_faces<double, double>(true, s, g, sms, rec, const_cast<double*>(dWx), dWx_out, const_cast<double*>(dWy),
+  e = launch_faces<double, double>(s, g, sms, rec, const_cast<double*>(dWx), dWx_out, const_cast<double*>(dWy),
                                    dWy_out, Fx, Fy, ctrl, 0);
   if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
   const UpdateArgs<double, double> ua{C0, C1, Fx, Fy, const_cast<double*>(dWx), dWx_out, const_cast<double*>(dWy), dWy_out, bad};
