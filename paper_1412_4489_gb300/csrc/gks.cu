@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(32 * ReconRows<R>::value, ReconBlocks<R, CHAR>
                                                const TW* Wy0, const TW* Wy1, R* __restrict__ rec, R dx, R dy,
                                                R weps, R wC, Ctrl* c, int force, int begin, double cfl,
                                                double dt_max, double t_end) {
-  pdl_enter();
+  pdl_wait();
   if (begin) {
     if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0 && threadIdx.y == 0)
       ctrl_begin(c, cfl, dt_max, t_end);
@@ -115,6 +115,7 @@ __global__ void __launch_bounds__(32 * ReconRows<R>::value, ReconBlocks<R, CHAR>
     const int i0 = blockIdx.x * blockDim.x, count = g.nx - i0 < 32 ? g.nx - i0 : 32;
     bulk_store(rec + rec_at(g, i0, j) * kRec, mine, (unsigned)(count * kRec * sizeof(R)));
   }
+  pdl_release();
 }
 
 // Warps to a block of the FP64 kernels, whose pipe serves a warp instruction for a quarter of an SM in 64 cycles
@@ -131,7 +132,7 @@ __global__ void __launch_bounds__(128, 6) k_recon_lanes(Geo g, const double* U0,
                                                         const double* Wx1, const double* Wy0, const double* Wy1,
                                                         double* __restrict__ rec, Ctrl* c, int force, int begin,
                                                         double cfl, double dt_max, double t_end) {
-  pdl_enter();
+  pdl_wait();
   if (begin) {
     if (blockIdx.x == 0 && threadIdx.x == 0) ctrl_begin(c, cfl, dt_max, t_end);
   } else if (!force && c->skip) {
@@ -142,6 +143,7 @@ __global__ void __launch_bounds__(128, 6) k_recon_lanes(Geo g, const double* U0,
   const int j = (int)(q / (unsigned)g.nx), i = (int)(q - (unsigned long long)j * g.nx);
   const int par = (int)(c->steps & 1);
   recon_cell_lanes(g, par ? U1 : U0, par ? Wx1 : Wx0, par ? Wy1 : Wy0, rec, i, j, k < n);
+  pdl_release();
 }
 
 // ---------------------------------------------------------------------------
@@ -228,7 +230,7 @@ __device__ __forceinline__ bool face_at(const Geo& g, unsigned block, int lane, 
 
 template <class R, class TW, int NS>
 __global__ void __launch_bounds__(128, 2) k_faces(Geo g, FaceArgs<R, TW> a, const Ctrl* c, int force) {
-  pdl_enter();
+  pdl_wait();
   if (!force && c->skip) return;
   const unsigned b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5) + a.first, lane = threadIdx.x & 31;
   const int par = (int)(c->steps & 1);
@@ -240,6 +242,7 @@ __global__ void __launch_bounds__(128, 2) k_faces(Geo g, FaceArgs<R, TW> a, cons
   } else if (face_at<1>(g, b - a.nbx, lane, i, j)) {
     flux_face<1, R, TW, NS>(g, a.Cy, a.rec, par ? a.Wy0 : a.Wy1, a.Fy, i, j, dt);
   }
+  pdl_release();
 }
 
 // The same with three warps to 32 faces (flux_face_split): for grids whose face warps are too few to keep the
@@ -247,7 +250,7 @@ __global__ void __launch_bounds__(128, 2) k_faces(Geo g, FaceArgs<R, TW> a, cons
 template <class R, class TW, int NS>
 __global__ void __launch_bounds__(96, 2) k_faces_split(Geo g, FaceArgs<R, TW> a, const Ctrl* c, int force) {
   __shared__ SplitShare<R> sh;
-  pdl_enter();
+  pdl_wait();
   if (!force && c->skip) return;
   const unsigned b = blockIdx.x + a.first;
   const int par = (int)(c->steps & 1), lane = threadIdx.x & 31;
@@ -260,15 +263,13 @@ __global__ void __launch_bounds__(96, 2) k_faces_split(Geo g, FaceArgs<R, TW> a,
     const bool active = face_at<1>(g, b - a.nbx, lane, i, j);
     flux_face_split<1, R, TW, NS>(g, a.Cy, a.rec, par ? a.Wy0 : a.Wy1, a.Fy, i, j, active, dt, sh);
   }
+  pdl_release();
 }
 
 // Grids of at most kSplitWarps face warps per SM (both axes) take the split launch.  Step times, one warp / three
 // warps to 32 faces (us): Euler 32^2 48 / 32, 69^2 (2.0 warps per SM) 49 / 38, 81^2 (2.7) 53 / 51, 96^2
 // (3.8) 56 / 57; Navier-Stokes 66 / 38, 67 / 51, 72 / 70, 76 / 89.
 constexpr unsigned kSplitWarps = 3;
-
-// cells up to which the FP32 Euler faces are launched with programmatic serialisation
-constexpr size_t kPdlCells = 1u << 17;
 
 // ---------------------------------------------------------------------------
 // update, CFL bound of the new state, physical check
@@ -542,7 +543,6 @@ void launch_ghost(gks_handle* h, int force) {
 template <class R, class TW>
 cudaError_t launch_update(bool pdl, cudaStream_t s, const Geo& g, int sms, const UpdateArgs<R, TW>& a, Ctrl* c) {
   const int rows = sizeof(R) == 8 ? (int)warps_per_block((unsigned long long)((g.nx + 31) / 32) * g.ny, sms) : kUpdateRows;
-  if (sizeof(R) == 8) pdl = false;  // as the faces (launch_faces): 128^2 97.6 -> 92.2 us a step
   return launch(pdl, k_update<R, TW>, update_grid(g, 1, sms, UpdateBlocks<R>::value, rows), dim3(32, rows), s, g, a, c);
 }
 
@@ -592,11 +592,9 @@ cudaError_t launch_recon(gks_handle* h, int force, int begin = 0, double cfl = 0
                              (const TW*)h->Wy[0], (const TW*)h->Wy[1], (R*)h->rec, h->ctrl, force, begin, cfl, dt_max, t_end);
 }
 
-// The FP64 face launch over both axes (axes 3) or one of them (1: x, 2: y).  Without programmatic serialisation: blocks
-// placed while the reconstruction's are still resident pile up on some SMs, and the fullest SM is the
-// kernel's time (64^2 split 64 -> 38 us a step).
+// The FP64 face launch over both axes (axes 3) or one of them (1: x, 2: y).
 template <class R, class TW>
-cudaError_t launch_faces(cudaStream_t s, const Geo& g, int sms, const R* rec, TW* Wx0, TW* Wx1, TW* Wy0, TW* Wy1,
+cudaError_t launch_faces(bool pdl, cudaStream_t s, const Geo& g, int sms, const R* rec, TW* Wx0, TW* Wx1, TW* Wy0, TW* Wy1,
                          R* Fx, R* Fy, const Ctrl* c, int force, int axes = 3) {
   const unsigned nbx = (unsigned)(((unsigned long long)(g.nx + 1) * g.ny + 31) / 32);
   const unsigned nby = (unsigned)(((unsigned long long)g.nx * (g.ny + 1) + 31) / 32);
@@ -604,9 +602,9 @@ cudaError_t launch_faces(cudaStream_t s, const Geo& g, int sms, const R* rec, TW
   const unsigned n = (axes & 1 ? nbx : 0) + (axes & 2 ? nby : 0);
   const bool ns = g.mu > 0.0, split = (unsigned long long)nbx + nby <= (unsigned long long)kSplitWarps * sms;
   if (split)
-    return launch(false, ns ? k_faces_split<R, TW, 1> : k_faces_split<R, TW, 0>, dim3(n), dim3(96), s, g, a, c, force);
+    return launch(pdl, ns ? k_faces_split<R, TW, 1> : k_faces_split<R, TW, 0>, dim3(n), dim3(96), s, g, a, c, force);
   const unsigned w = warps_per_block(n, sms);
-  return launch(false, ns ? k_faces<R, TW, 1> : k_faces<R, TW, 0>, dim3((n + w - 1) / w), dim3(32 * w), s, g, a, c, force);
+  return launch(pdl, ns ? k_faces<R, TW, 1> : k_faces<R, TW, 0>, dim3((n + w - 1) / w), dim3(32 * w), s, g, a, c, force);
 }
 
 // ev (optional, kProfileParts + 1 events): recorded before each kernel and after the last.
@@ -635,7 +633,7 @@ gks_status launch_step_kernels(gks_handle* h, double cfl, double dt_max, double 
   bool fork = false;
   if constexpr (sizeof(R) == 8) {
     auto faces = [&](int axes) {
-      keep(launch_faces<R, TW>(s, g, h->sms, (const R*)h->rec, (TW*)h->Wx[0], (TW*)h->Wx[1], (TW*)h->Wy[0],
+      keep(launch_faces<R, TW>(pdl, s, g, h->sms, (const R*)h->rec, (TW*)h->Wx[0], (TW*)h->Wx[1], (TW*)h->Wy[0],
                                (TW*)h->Wy[1], (R*)h->Fx, (R*)h->Fy, (const Ctrl*)h->ctrl, force, axes));
     };
     if (ev) faces(1);
@@ -672,9 +670,7 @@ gks_status launch_step_kernels(gks_handle* h, double cfl, double dt_max, double 
       auto faces = [&](int axes) {
         const FaceArgs<R, TW> a{fconst<R>(g, 0), fconst<R>(g, 1), (const R*)h->rec, (TW*)h->Wx[0], (TW*)h->Wx[1],
                                 (TW*)h->Wy[0], (TW*)h->Wy[1], (R*)h->Fx, (R*)h->Fy, nbx, axes == 2 ? nbx : 0};
-        // without programmatic serialisation on larger grids: blocks that wait on an SM take its slots from the
-        // reconstruction's last ones (2048^2 599 -> 587 us a step, 256^2 19.0 -> 19.8)
-        keep(launch(pdl && (size_t)g.nx * g.ny <= kPdlCells, k_flux_euler, dim3((axes & 1 ? nbx : 0) + (axes & 2 ? nby : 0)), bf, s, g, a, (const Ctrl*)h->ctrl,
+        keep(launch(pdl, k_flux_euler, dim3((axes & 1 ? nbx : 0) + (axes & 2 ? nby : 0)), bf, s, g, a, (const Ctrl*)h->ctrl,
                     force));
       };
       if (ev) faces(1);
@@ -1343,7 +1339,7 @@ extern "C" gks_status gks_step_noalloc(int nx, int ny, double Lx, double Ly, dou
   if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
   e = launch_recon<double, double>(true, s, g, sms, U0, U1, dWx, dWx_out, dWy, dWy_out, rec, ctrl, 0, 1, CFL, dt_max, INFINITY);
   if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
-  e = launch_faces<double, double>(s, g, sms, rec, const_cast<double*>(dWx), dWx_out, const_cast<double*>(dWy),
+  e = launch_faces<double, double>(true, s, g, sms, rec, const_cast<double*>(dWx), dWx_out, const_cast<double*>(dWy),
                                    dWy_out, Fx, Fy, ctrl, 0);
   if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
   const UpdateArgs<double, double> ua{C0, C1, Fx, Fy, const_cast<double*>(dWx), dWx_out, const_cast<double*>(dWy), dWy_out, bad};

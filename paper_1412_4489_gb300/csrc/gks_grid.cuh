@@ -282,12 +282,18 @@ __device__ __forceinline__ void df_add_product(float& hi, float& lo, float f, fl
 
 // Programmatic dependent launch: a step kernel launched with programmatic stream
 // serialisation first waits for its predecessor grid to complete (and its writes
-// to be visible), then lets its own successor be scheduled once every block of
-// this grid is resident, so that launch latency overlaps execution.  Without the
-// launch attribute both instructions are no-ops.
+// to be visible) and lets its own successor be scheduled, so that launch latency overlaps
+// execution: when every block of this grid is resident (pdl_enter) or only when
+// every block has done its work (pdl_wait, pdl_release).  Successors that are placed early sit where
+// there happens to be room, and take slots from this grid's last blocks: after the reconstruction and the
+// FP64 faces, whose successors' time is that of their fullest SM, the late form (64^2 FP64 split faces 64 -> 36
+// us a step, 2048^2 FP32 600 -> 587); elsewhere the early one (late after the FP32 faces or updates: 2048^2 587 ->
+// 604).  Without the launch attribute these instructions are no-ops.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" :::); }
 __device__ __forceinline__ void pdl_enter() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" :::);
+  pdl_wait();
+  pdl_release();
 }
 
 __device__ __forceinline__ unsigned long long dbits(double x) { return (unsigned long long)__double_as_longlong(x); }
