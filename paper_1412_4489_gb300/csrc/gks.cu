@@ -474,6 +474,10 @@ __global__ void k_set_dt(Ctrl* c, double dt) {
 // ===========================================================================
 // host side
 // ===========================================================================
+// steps per graph of gks_advance: a graph's start costs 3 to 5 us beyond its steps (10 steps of a 1024^2 grid
+// as 4 + 4 + 1 + 1 graphs instead of ten)
+constexpr int kGraphSteps[3] = {16, 4, 1};
+
 struct gks_handle {
   Geo g;
   int prec;
@@ -494,7 +498,7 @@ struct gks_handle {
   Ctrl* hctrl;       // pinned mirror
   double* staging;   // device FP64 scratch for host transfers
   size_t staging_n;
-  cudaGraphExec_t graph1, graph16;
+  cudaGraphExec_t graph[3];  // kGraphSteps steps each, captured when first needed
   double graph_cfl, graph_tend;
   std::string err;
 };
@@ -721,9 +725,10 @@ gks_status read_ctrl(gks_handle* h) {
 }
 
 void destroy_graphs(gks_handle* h) {
-  if (h->graph1) cudaGraphExecDestroy(h->graph1);
-  if (h->graph16) cudaGraphExecDestroy(h->graph16);
-  h->graph1 = h->graph16 = nullptr;
+  for (cudaGraphExec_t& x : h->graph) {
+    if (x) cudaGraphExecDestroy(x);
+    x = nullptr;
+  }
 }
 
 gks_status capture(gks_handle* h, int nsteps, double cfl, double t_end, cudaGraphExec_t* out) {
@@ -973,17 +978,17 @@ gks_status gks_advance(gks_handle* h, int nsteps, double CFL, double t_end) {
   if (!h) return GKS_EINVAL;
   if (nsteps < 0 || !(CFL > 0)) return fail(h, GKS_EINVAL, "gks_advance: nsteps >= 0 and CFL > 0 required");
   CK(cudaSetDevice(h->device));
-  if (!h->graph1 || h->graph_cfl != CFL || h->graph_tend != t_end) {
-    destroy_graphs(h);
-    gks_status st = capture(h, 1, CFL, t_end, &h->graph1);
-    if (st == GKS_OK) st = capture(h, 16, CFL, t_end, &h->graph16);
-    if (st != GKS_OK) { destroy_graphs(h); return st; }
-    h->graph_cfl = CFL;
-    h->graph_tend = t_end;
-  }
+  if (h->graph_cfl != CFL || h->graph_tend != t_end) destroy_graphs(h);
+  h->graph_cfl = CFL;
+  h->graph_tend = t_end;
   int left = nsteps;
-  while (left >= 16) { CK(cudaGraphLaunch(h->graph16, h->stream)); left -= 16; }
-  while (left > 0) { CK(cudaGraphLaunch(h->graph1, h->stream)); --left; }
+  for (int k = 0; k < 3; ++k) {
+    if (left >= kGraphSteps[k] && !h->graph[k]) {
+      const gks_status st = capture(h, kGraphSteps[k], CFL, t_end, &h->graph[k]);
+      if (st != GKS_OK) { destroy_graphs(h); return st; }
+    }
+    for (; left >= kGraphSteps[k]; left -= kGraphSteps[k]) CK(cudaGraphLaunch(h->graph[k], h->stream));
+  }
   return GKS_OK;
 }
 
