@@ -192,10 +192,12 @@ int gks_launches_per_step(const gks_handle* h);
 
 /* Takes one step like gks_step(h, CFL, +inf, NULL) with CUDA events recorded on
  * the handle's stream between its kernels, and writes the duration in ms of
- * each of the seven kernels to ms[0..6], in launch order: reconstruction (which
- * also opens the step), x-face evolution, y-face evolution, update (which also
- * refreshes the ghost ring), the two update passes of the positivity fallback
- * (no work unless a cell needed it), end.
+ * each part of the step to ms[0..6], in launch order: reconstruction (which
+ * also opens the step), x-face evolution, y-face evolution (launched apart here;
+ * otherwise one launch but for FP32 Navier-Stokes), update (which also refreshes
+ * the ghost ring), the finish: the positivity fallback's two update passes (no work
+ * unless a cell needed them) and the step's end, in one kernel.  The last two
+ * entries hold no kernel any more, only the events' own time.
  * Synchronous; returns the status of the step. */
 gks_status gks_profile_step(gks_handle* h, double CFL, float* ms);
 

@@ -755,11 +755,12 @@ GKS_FN void finish_face(const FaceConst<R>& C, R u0, R v0, R Fl[4], const R P0[4
 // (one warp instruction per 19 cycles and SM), so fewer operations is what makes it faster.  Each Maxwellian
 // is evaluated in its own frame, where g0's moments are closed forms in the central derivatives and a half-space's
 // reduce to one-dimensional sums over u.  Against expanding the distribution into the monomials
-// u^a v^b xi^2c (gks_face_monomials.cuh): 1,232 instead of 2,041 counted flops at a smooth
-// Euler face (exp(-dt/tau) = 0), 1,722 instead of 2,779 at another, 2,180 instead of 3,907
+// u^a v^b xi^2c (gks_face_monomials.cuh): 1,237 instead of 2,041 counted flops at a smooth
+// Euler face (exp(-dt/tau) = 0), 1,739 instead of 2,779 at another, 2,198 instead of 3,907
 // Navier-Stokes with the Prandtl correction.
 // x-faces at 512^2 FP32 26.2 -> 20.7 us (Euler), at 1024^2 108 -> 81 us (Navier-Stokes), at
-// 4096^2 1,177 -> 881 us; FP64 at 512^2 764 -> 534 us.
+// 4096^2 1,177 -> 881 us; FP64 at 512^2 764 -> 534 us.  With the table for erfc and exp, the reciprocals and the
+// launch shapes of today 19.7, 74 and 730 us, FP64 463 us.
 // ---------------------------------------------------------------------------
 template <class R, int NSM = -1, class Src>
 GKS_FN void face_evolution(const FaceConst<R>& C, const Src& src, R dt, R F[4], R Wm[4], R Wp[4]) {

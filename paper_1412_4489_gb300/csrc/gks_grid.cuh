@@ -683,7 +683,7 @@ __device__ __forceinline__ void recon_cell(const Geo& g, const R* __restrict__ U
 // recon_cell.  Four times the warps of one thread per cell: the FP64 pipe's interval of 64 cycles
 // per warp instruction makes a cell's serial time the kernel's on grids of up to some 10,000 cells, and
 // on larger ones the register need of one variable lets twice the warps be resident.  81^2 46 -> 15 us
-// (with the event's ~4), 200 x 1 25 -> 11 us, 512^2 276 -> 259 us.
+// (with the event's ~4), 200 x 1 25 -> 11 us, 512^2 276 -> 259 us (209 with its positivity check in FP32).
 __device__ __forceinline__ void recon_cell_lanes(const Geo& g, const double* __restrict__ U, const double* __restrict__ Wx,
                                                  const double* __restrict__ Wy, double* __restrict__ rec, int i, int j,
                                                  bool active) {

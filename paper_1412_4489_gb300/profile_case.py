@@ -1,6 +1,6 @@
 """Runs a few time steps of one seeded workload through the library, one step per
 ``gks_step`` call, so that a profiler sees each step's kernels in launch order
-(begin, ghost, recon, flux_x, flux_y, update passes 1-3, end).
+(reconstruction, faces, update, finish).
 
     python -m paper_1412_4489_gb300.profile_case --workload smooth --size 2048 --precision fp32 --steps 3
 
