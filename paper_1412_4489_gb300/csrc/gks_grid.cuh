@@ -521,81 +521,6 @@ __device__ __forceinline__ void recon_vectors(const R in[13][4], const ReconK<R>
   }
 }
 
-// The FP64 form of the characteristic reconstruction, in units of the cell size and with recon_var_scaled; load(k, w):
-// stencil vector k, read again for the second direction instead of kept.  The projections use the eigenvectors'
-// structure: with s = (b2, -b1 u, -b1 v, b1) . w / 2 and d = (u w0 - w1) / (2 c) the characteristic variables
-// are s + d, w0 - 2 s, w2 - v w0 and s - d (10 FP64 instructions a vector instead of 16).  1024^2 3.07 -> 2.59 ms.
-template <class Load>
-__device__ __forceinline__ void recon_char_scaled(const Geo& g, const Load& load, double a[4][5]) {
-  const double gm1 = g.gamma - 1.0;
-#pragma unroll 1
-  for (int axis = 0; axis < 2; ++axis) {
-    double in[13][4];
-#pragma unroll
-    for (int k = 0; k < 13; ++k) {
-      load(k, in[k]);
-      if (axis) {  // momenta swapped for the y direction
-        const double t = in[k][1];
-        in[k][1] = in[k][2];
-        in[k][2] = t;
-      }
-    }
-    const double rho = in[0][0], ir = d_rcp(rho), u = in[0][1] * ir, v = in[0][2] * ir;
-    const double q2 = __dadd_rn(__dmul_rn(u, u), __dmul_rn(v, v));  // the same bits for both axes: one decision
-    const double p = gm1 * (in[0][3] - 0.5 * rho * q2);
-    const bool physical = rho > 0.0 && p > 0.0;
-    const double c2 = g.gamma * p * ir, c = sqrt(c2), ic = 0.5 * d_rcp(c), H = (in[0][3] + p) * ir;
-    const double b1 = 0.5 * gm1 * d_rcp(c2), b2 = 0.5 * b1 * q2, bu = b1 * u, bv = b1 * v, cu = ic * u;
-    if (physical) {
-#pragma unroll
-      for (int k = 0; k < 13; ++k) {
-        double* w = in[k];
-        const double s = b2 * w[0] - bu * w[1] - bv * w[2] + b1 * w[3], d = cu * w[0] - ic * w[1];
-        w[2] = w[2] - v * w[0];
-        w[1] = w[0] - 2.0 * s;
-        w[0] = s + d;
-        w[3] = s - d;
-      }
-    }
-    double cc[4][5];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-      recon_var_scaled(in[0][r], in[1][r], in[2][r], in[3][r], in[4][r], in[5][r], in[6][r], in[7][r], in[8][r], in[9][r],
-                       in[10][r], in[11][r], in[12][r], g.weno_eps, g.b1sq, cc[r]);
-    // a2, a4 (m = 0, 2) from the x pass; a3, a5 (m = 1, 3) from the y pass; a6 the mean of both.  A cell that is
-    // not physical takes every coefficient from its conservative variables.
-#pragma unroll
-    for (int m = 0; m < 5; ++m) {
-      double o[4];
-      if (physical) {
-        const double sum = cc[0][m] + cc[1][m] + cc[3][m];
-        o[0] = sum;
-        o[1] = u * sum + c * (cc[3][m] - cc[0][m]);
-        o[2] = v * sum + cc[2][m];
-        o[3] = H * (cc[0][m] + cc[3][m]) + u * c * (cc[3][m] - cc[0][m]) + 0.5 * q2 * cc[1][m] + v * cc[2][m];
-      } else {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) o[r] = cc[r][m];
-      }
-      const bool mine = m == 4 || (m & 1) == axis;
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const double x = axis && (r == 1 || r == 2) ? o[3 - r] : o[r];
-        if (m == 4) a[r][m] = axis ? a[r][m] + 0.5 * x : 0.5 * x;
-        else if (mine) a[r][m] = x;
-      }
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    a[r][0] *= g.idx;
-    a[r][1] *= g.idy;
-    a[r][2] *= g.idx2;
-    a[r][3] *= g.idy2;
-    a[r][4] *= g.idxy;
-  }
-}
-
 // the record of cell (i, j)
 template <class R, bool CHAR = false>
 __device__ __forceinline__ void recon_record(const Geo& g, const R* __restrict__ U, const R* __restrict__ Wx,
@@ -607,31 +532,22 @@ __device__ __forceinline__ void recon_record(const Geo& g, const R* __restrict__
   R a[4][5], cbar[4];
   // stencil vector k: c, e, w, n, s; east face y-/y+, west y-/y+, north x-/x+, south x-/x+
   const size_t ox = (size_t)j * (nx + 1) + i, oy = (size_t)j * nx + i;
-  if constexpr (CHAR && sizeof(R) == 8) {
-    Lay<R>::load_u(g, U, i, j, cbar);
-    recon_char_scaled(g, [&](int k, R w[4]) {
-      if (k < 5) Lay<R>::load_u(g, U, i + (k == 1) - (k == 2), j + (k == 3) - (k == 4), w);
-      else if (k < 9) Lay<R>::load_w(Wx, fxp, (k - 5) & 1, ox + (k < 7), w);
-      else Lay<R>::load_w(Wy, fyp, (k - 9) & 1, oy + (k < 11 ? nx : 0), w);
-    }, a);
-  } else {
-    R in[13][4];
-    Lay<R>::load_u(g, U, i, j, in[0]);
-    Lay<R>::load_u(g, U, i + 1, j, in[1]);
-    Lay<R>::load_u(g, U, i - 1, j, in[2]);
-    Lay<R>::load_u(g, U, i, j + 1, in[3]);
-    Lay<R>::load_u(g, U, i, j - 1, in[4]);
+  R in[13][4];
+  Lay<R>::load_u(g, U, i, j, in[0]);
+  Lay<R>::load_u(g, U, i + 1, j, in[1]);
+  Lay<R>::load_u(g, U, i - 1, j, in[2]);
+  Lay<R>::load_u(g, U, i, j + 1, in[3]);
+  Lay<R>::load_u(g, U, i, j - 1, in[4]);
 #pragma unroll
-    for (int p = 0; p < 2; ++p) {
-      Lay<R>::load_w(Wx, fxp, p, ox + 1, in[5 + p]);
-      Lay<R>::load_w(Wx, fxp, p, ox, in[7 + p]);
-      Lay<R>::load_w(Wy, fyp, p, oy + nx, in[9 + p]);
-      Lay<R>::load_w(Wy, fyp, p, oy, in[11 + p]);
-    }
-#pragma unroll
-    for (int v = 0; v < 4; ++v) cbar[v] = in[0][v];
-    recon_vectors<CHAR, R>(in, K, GeoR<R>::gm1(g), GeoR<R>::gamma(g), a);
+  for (int p = 0; p < 2; ++p) {
+    Lay<R>::load_w(Wx, fxp, p, ox + 1, in[5 + p]);
+    Lay<R>::load_w(Wx, fxp, p, ox, in[7 + p]);
+    Lay<R>::load_w(Wy, fyp, p, oy + nx, in[9 + p]);
+    Lay<R>::load_w(Wy, fyp, p, oy, in[11 + p]);
   }
+#pragma unroll
+  for (int v = 0; v < 4; ++v) cbar[v] = in[0][v];
+  recon_vectors<CHAR, R>(in, K, GeoR<R>::gm1(g), GeoR<R>::gamma(g), a);
   // the polynomial at the four face centres (x = +-dx/2, y = 0 and x = 0, y = +-dy/2):
   // value = e0 +- a2 dx/2 on x-faces, n0 +- a3 dy/2 on y-faces
   R ve[4], vw[4], vn[4], vs[4];
