@@ -1156,7 +1156,7 @@ gks_status gks_part_halo_bytes(const gks_handle* h, int what, size_t* bytes) {
   if (!h || !bytes || (what != GKS_PART_STATE && what != GKS_PART_RECORDS)) return GKS_EINVAL;
   const Geo& g = h->g;
   const size_t es = h->prec == GKS_FP64 ? sizeof(double) : sizeof(float);
-  // averages: 4 FP64 planes, or the 4 hi and 4 lo FP32 planes, nx + 2 values each
+  // averages: 4 FP64 planes of nx + 2 values, or nx + 2 hi and nx + 2 lo vectors of 4 FP32 values
   *bytes = what == GKS_PART_STATE ? (size_t)8 * sizeof(float) * (g.nx + 2) : (size_t)(g.nx + 2) * kRec * es;
   return GKS_OK;
 }
