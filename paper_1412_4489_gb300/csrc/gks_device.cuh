@@ -60,6 +60,11 @@ __device__ __forceinline__ float d_div(float a, float b) { return __fdividef(a, 
 __device__ __forceinline__ double d_rcp(double a) { return 1.0 / a; }
 __device__ __forceinline__ float d_rcp(float a) { return __fdividef(1.0f, a); }
 
+// 2^-511 <= |a| < 2^512, by the exponent bits: squares and reciprocals are normal numbers
+__device__ __forceinline__ bool mid_range(double a) {
+  return (unsigned)(__double2hiint(a) & 0x7fffffff) - 0x20000000u < 0x3ff00000u;
+}
+
 template <class R> GKS_FN R sq(R a) { return a * a; }
 
 // ---------------------------------------------------------------------------
@@ -322,26 +327,30 @@ GKS_FN void prim(const R w[4], R gm1, R& rho, R& ir, R& U, R& V, R& p) {
 }
 
 // the same with 2 lam = rho / p and 1 / (2 lam).  FP64: both quotients from one reciprocal (a
-// reciprocal takes 5.4 FP64 instructions, a quotient 8.6); FP32: a reciprocal is one instruction, and the
-// product rho p would leave FP32's range earlier than rho and p do.
+// reciprocal takes 5.4 FP64 instructions, a quotient 8.6), of rho^2 p; where that or rho is not well inside FP64's
+// range, from quotients of their own.  (Inside it every product here is a normal number.)  FP32: a
+// reciprocal is one instruction, and rho^2 p would leave the range often.
 template <class R>
 GKS_FN void prim_lam(const R w[4], R gm1, R& rho, R& U, R& V, R& p, R& l2, R& var) {
   R ir;
   if constexpr (sizeof(R) == 8) {
     rho = w[0];
     const R rp = gm1 * (rho * w[3] - R(0.5) * (w[1] * w[1] + w[2] * w[2]));  // rho p
-    const R t = d_rcp(rho * rp);
-    ir = t * rp;
-    U = w[1] * ir;
-    V = w[2] * ir;
-    p = rp * ir;
-    l2 = rho * rho * (rho * t);
-    var = p * ir;
-  } else {
-    prim(w, gm1, rho, ir, U, V, p);
-    l2 = d_div(rho, p);
-    var = p * ir;
+    const R q = rho * rp;
+    if (mid_range(q) && mid_range(rho)) {
+      const R t = d_rcp(q);
+      ir = t * rp;
+      U = w[1] * ir;
+      V = w[2] * ir;
+      p = rp * ir;
+      l2 = rho * rho * (rho * t);
+      var = p * ir;
+      return;
+    }
   }
+  prim(w, gm1, rho, ir, U, V, p);
+  l2 = d_div(rho, p);
+  var = p * ir;
 }
 
 struct FaceParams {
