@@ -45,7 +45,10 @@
  * message.  A step whose new state is still not physical after the fallback is
  * not taken: the state stays the one before the step and GKS_ENONPHYSICAL is
  * reported (by gks_step, or by the next gks_sync / gks_get_state after
- * gks_advance).
+ * gks_advance).  The fallback's passes meet at device-wide waits of bounded length
+ * (gks_set_wait_limit); should one run out, which no working device lets happen, the
+ * step fails in the same way with GKS_ETIMEOUT, as gks_step_noalloc and
+ * gks_part_finish then do.  Either status stays until gks_set_state.
  */
 #ifndef GKS_H
 #define GKS_H
@@ -167,6 +170,14 @@ gks_status gks_step(gks_handle* h, double CFL, double dt_max, double* dt_taken);
  * queued steps are reported by gks_sync or gks_get_state. */
 gks_status gks_advance(gks_handle* h, int nsteps, double CFL, double t_end);
 
+/* Limit of the device waits of the positivity fallback, in seconds (default 2; 2 ms
+ * are added for each 256 cells of a block's share of the grid, and only time in
+ * which the waiting block runs counts).  test_skip_block >= 0 makes that block of the
+ * fallback's kernel skip its arrival at them -- a test hook with which every wait
+ * runs out, so that GKS_ETIMEOUT can be exercised; -1 disables it.  Holds for later
+ * gks_step, gks_advance, gks_profile_step and gks_part_finish calls; gks_step_noalloc has the defaults. */
+gks_status gks_set_wait_limit(gks_handle* h, double seconds, int test_skip_block);
+
 /* Waits for queued work; returns the pending status.  t and steps (either may
  * be NULL) receive the simulation time and the number of steps taken. */
 gks_status gks_sync(gks_handle* h, double* t, long long* steps);
@@ -246,7 +257,7 @@ gks_status gks_part_bound(gks_handle* h, double* bound);
 gks_status gks_part_recon(gks_handle* h, double dt);
 
 /* Evolves the slab's faces and updates its cells; closes the step.  Returns
- * GKS_ENONPHYSICAL (state kept) like gks_step. */
+ * GKS_ENONPHYSICAL or GKS_ETIMEOUT (state kept) like gks_step. */
 gks_status gks_part_finish(gks_handle* h);
 
 /* Copies the slab's edge row on y-side `side` (2: low, 3: high) into dst, or the
@@ -388,7 +399,8 @@ gks_status gks_measure_alu_peak(int precision, double* tflops);
  * first call before any stream capture.  The address is kept for the life of the
  * process, so the device's primary context must not be reset (cudaDeviceReset)
  * between calls.  Returns GKS_ENONPHYSICAL (outputs not
- * valid) if the new state is not physical, GKS_EINVAL if dt would be 0. */
+ * valid) if the new state is not physical, GKS_ETIMEOUT (likewise) if a wait of the
+ * positivity fallback ran out, GKS_EINVAL if dt would be 0. */
 gks_status gks_step_noalloc(int nx, int ny, double Lx, double Ly, double gamma, double Pr, double mu,
                             const gks_bc* bc, const gks_options* opt, const double* dU,
                             const double* dWx, const double* dWy, double CFL, double dt_max,

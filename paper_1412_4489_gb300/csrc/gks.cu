@@ -337,9 +337,23 @@ __global__ void __launch_bounds__(256, UpdateBlocks<R>::value) k_update(Geo g, U
   update_pass<R, TW>(g, a, c, 1);
 }
 
-// Barrier of all blocks of a cooperative launch; bounded: a block that waits longer than two seconds
-// fails the step (GKS_ETIMEOUT) and returns false, as do the others.
-__device__ bool ctrl_barrier(Ctrl* c) {
+// Limit of the fallback's device waits, and the block whose arrival they miss (a test hook; -1: none).
+struct Wait {
+  unsigned long long limit_ns;
+  int skip;
+};
+
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// Barrier of all blocks of a cooperative launch; bounded: a block that waits longer than the limit
+// fails the step (GKS_ETIMEOUT) and returns false, as do the others.  Only time in which the block runs counts: a
+// poll takes about a microsecond, so a longer gap between two of them than a millisecond is time in which this
+// context did not have the device (time slices of other processes).
+__device__ bool ctrl_barrier(Ctrl* c, Wait w) {
   __syncthreads();
   __shared__ int ok;
   if (threadIdx.x == 0 && threadIdx.y == 0) {
@@ -347,16 +361,17 @@ __device__ bool ctrl_barrier(Ctrl* c) {
     volatile int* status = &c->status;
     const unsigned my = *gen;
     __threadfence();
-    if (atomicAdd(&c->bar_count, 1u) + 1 == gridDim.x * gridDim.y) {
+    if ((int)(blockIdx.y * gridDim.x + blockIdx.x) != w.skip && atomicAdd(&c->bar_count, 1u) + 1 == gridDim.x * gridDim.y) {
       c->bar_count = 0;
       __threadfence();
       atomicAdd(&c->bar_gen, 1u);
     }
-    unsigned long long t0, t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+    unsigned long long last = global_ns(), waited = 0;
     while (*gen == my && *status != GKS_ETIMEOUT) {
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-      if (t - t0 > 2000000000ull) atomicExch(&c->status, GKS_ETIMEOUT);
+      const unsigned long long t = global_ns(), d = t - last;
+      waited += d < 1000000ull ? d : 1000000ull;
+      last = t;
+      if (waited > w.limit_ns) atomicExch(&c->status, GKS_ETIMEOUT);
       __nanosleep(200);
     }
     __threadfence();
@@ -374,17 +389,17 @@ __device__ bool ctrl_barrier(Ctrl* c) {
 // mirror (optional): page-locked host memory that the first thread leaves the control block in, for a caller that waits
 // for this step.
 template <class R, class TW>
-__global__ void __launch_bounds__(256, UpdateBlocks<R>::value) k_finish(Geo g, UpdateArgs<R, TW> a, Ctrl* c, Ctrl* mirror) {
+__global__ void __launch_bounds__(256, UpdateBlocks<R>::value) k_finish(Geo g, UpdateArgs<R, TW> a, Ctrl* c, Ctrl* mirror, Wait w) {
   pdl_enter();
   const bool first = blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0;
   if (!c->skip) {
     bool met = true;
     if (c->bad_found[0]) {
       update_pass<R, TW>(g, a, c, 2);
-      met = ctrl_barrier(c);
+      met = ctrl_barrier(c, w);
       if (met && *(volatile int*)&c->bad_found[1]) {
         update_pass<R, TW>(g, a, c, 3);
-        met = ctrl_barrier(c);
+        met = ctrl_barrier(c, w);
       }
     }
     if (first && met) ctrl_end(c);
@@ -478,6 +493,12 @@ __global__ void k_set_dt(Ctrl* c, double dt) {
 // as 4 + 4 + 1 + 1 graphs instead of ten)
 constexpr int kGraphSteps[3] = {16, 4, 1};
 
+// Default limit of the fallback's device waits.  A block waits for the others' shares of a pass, so the limit grows
+// with the share: kWaitTileSeconds for each 32 x 8 tile a block walks.  A tile whose 1,024 faces are all evolved
+// again takes below 0.2 ms in FP64 (some 1,200 FP64 instructions a thread, four warps to a quarter of an
+// SM, 64 cycles each).
+constexpr double kWaitSeconds = 2.0, kWaitTileSeconds = 2e-3;
+
 struct gks_handle {
   Geo g;
   int prec;
@@ -500,6 +521,8 @@ struct gks_handle {
   size_t staging_n;
   cudaGraphExec_t graph[3];  // kGraphSteps steps each, captured when first needed
   double graph_cfl, graph_tend;
+  double wait_s = kWaitSeconds;  // gks_set_wait_limit
+  int wait_skip = -1;
   std::string err;
 };
 
@@ -563,9 +586,14 @@ cudaError_t launch_update(bool pdl, cudaStream_t s, const Geo& g, int sms, const
 }
 
 template <class R, class TW>
-cudaError_t launch_finish(cudaStream_t s, const Geo& g, int sms, const UpdateArgs<R, TW>& a, Ctrl* c, Ctrl* mirror) {
+cudaError_t launch_finish(cudaStream_t s, const Geo& g, int sms, const UpdateArgs<R, TW>& a, Ctrl* c, Ctrl* mirror,
+                          double wait_s, int wait_skip) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = update_grid(g, 2, sms, 1, kUpdateRows);
+  const dim3 tiles = grid2(g.nx, g.ny, dim3(32, kUpdateRows));
+  const double per_block = (double)((tiles.x + cfg.gridDim.x - 1) / cfg.gridDim.x) *
+                           ((tiles.y + cfg.gridDim.y - 1) / cfg.gridDim.y);
+  const Wait w{(unsigned long long)((wait_s + kWaitTileSeconds * per_block) * 1e9), wait_skip};
   cfg.blockDim = dim3(32, kUpdateRows);
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
@@ -575,7 +603,7 @@ cudaError_t launch_finish(cudaStream_t s, const Geo& g, int sms, const UpdateArg
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, k_finish<R, TW>, g, a, c, mirror);
+  return cudaLaunchKernelEx(&cfg, k_finish<R, TW>, g, a, c, mirror, w);
 }
 
 template <class R, class TW>
@@ -701,7 +729,7 @@ gks_status launch_step_kernels(gks_handle* h, double cfl, double dt_max, double 
     // after the join (two predecessors): an ordinary launch
     keep(launch_update<R, TW>(pdl && !fork, s, g, h->sms, a, h->ctrl));
     mark(4);
-    keep(launch_finish<R, TW>(s, g, h->sms, a, h->ctrl, mirror ? h->hctrl : nullptr));
+    keep(launch_finish<R, TW>(s, g, h->sms, a, h->ctrl, mirror ? h->hctrl : nullptr, h->wait_s, h->wait_skip));
   } else {
     mark(4);
   }
@@ -716,6 +744,13 @@ gks_status launch_step_kernels(gks_handle* h, double cfl, double dt_max, double 
 gks_status launch_step(gks_handle* h, double cfl, double dt_max, double t_end, bool mirror = false) {
   if (h->prec == GKS_FP64) return launch_step_kernels<double, double>(h, cfl, dt_max, t_end, true, true, 0, nullptr, true, mirror);
   return launch_step_kernels<float, float>(h, cfl, dt_max, t_end, true, true, 0, nullptr, true, mirror);
+}
+
+// the status that the control block holds, as a call's result
+gks_status step_status(gks_handle* h, const char* what) {
+  const gks_status st = (gks_status)h->hctrl->status;
+  if (st == GKS_OK) return st;
+  return fail(h, st, st == GKS_ETIMEOUT ? "a device wait of the positivity fallback ran out; state kept" : what);
 }
 
 gks_status read_ctrl(gks_handle* h) {
@@ -970,8 +1005,7 @@ gks_status gks_step(gks_handle* h, double CFL, double dt_max, double* dt_taken) 
   if (st != GKS_OK) return st;
   CK(cudaStreamSynchronize(h->stream));  // the step left its control block in hctrl
   if (dt_taken) *dt_taken = h->hctrl->skip ? 0.0 : h->hctrl->dt;
-  if (h->hctrl->status != GKS_OK) return fail(h, (gks_status)h->hctrl->status, "step produced a non-physical state; state kept");
-  return GKS_OK;
+  return step_status(h, "step produced a non-physical state; state kept");
 }
 
 gks_status gks_advance(gks_handle* h, int nsteps, double CFL, double t_end) {
@@ -992,6 +1026,15 @@ gks_status gks_advance(gks_handle* h, int nsteps, double CFL, double t_end) {
   return GKS_OK;
 }
 
+gks_status gks_set_wait_limit(gks_handle* h, double seconds, int test_skip_block) {
+  if (!h || !(seconds > 0) || !(seconds <= 3600)) return fail(h, GKS_EINVAL, "gks_set_wait_limit: seconds must lie in (0, 3600]");
+  CK(cudaSetDevice(h->device));
+  destroy_graphs(h);  // they hold the limit
+  h->wait_s = seconds;
+  h->wait_skip = test_skip_block;
+  return GKS_OK;
+}
+
 gks_status gks_sync(gks_handle* h, double* t, long long* steps) {
   if (!h) return GKS_EINVAL;
   CK(cudaSetDevice(h->device));
@@ -999,8 +1042,7 @@ gks_status gks_sync(gks_handle* h, double* t, long long* steps) {
   if (st != GKS_OK) return st;
   if (t) *t = h->hctrl->t;
   if (steps) *steps = h->hctrl->steps;
-  if (h->hctrl->status != GKS_OK) return fail(h, (gks_status)h->hctrl->status, "a queued step produced a non-physical state; state kept");
-  return GKS_OK;
+  return step_status(h, "a queued step produced a non-physical state; state kept");
 }
 
 gks_status gks_get_state_device(gks_handle* h, double* dU, double* dWx, double* dWy, double* t) {
@@ -1011,8 +1053,7 @@ gks_status gks_get_state_device(gks_handle* h, double* dU, double* dWx, double* 
   st = read_ctrl(h);
   if (st != GKS_OK) return st;
   if (t) *t = h->hctrl->t;
-  if (h->hctrl->status != GKS_OK) return fail(h, (gks_status)h->hctrl->status, "a step produced a non-physical state; state kept");
-  return GKS_OK;
+  return step_status(h, "a step produced a non-physical state; state kept");
 }
 
 gks_status gks_get_state(gks_handle* h, double* U, double* Wx, double* Wy, double* t) {
@@ -1037,8 +1078,7 @@ gks_status gks_get_state(gks_handle* h, double* U, double* Wx, double* Wy, doubl
   gks_status st = read_ctrl(h);
   if (st != GKS_OK) return st;
   if (t) *t = h->hctrl->t;
-  if (h->hctrl->status != GKS_OK) return fail(h, (gks_status)h->hctrl->status, "a step produced a non-physical state; state kept");
-  return GKS_OK;
+  return step_status(h, "a step produced a non-physical state; state kept");
 }
 
 void gks_destroy(gks_handle* h) {
@@ -1084,8 +1124,7 @@ gks_status gks_profile_step(gks_handle* h, double CFL, float* ms) {
   if (st != GKS_OK) return st;
   st = read_ctrl(h);
   if (st != GKS_OK) return st;
-  if (h->hctrl->status != GKS_OK) return fail(h, (gks_status)h->hctrl->status, "step produced a non-physical state; state kept");
-  return GKS_OK;
+  return step_status(h, "step produced a non-physical state; state kept");
 }
 
 int gks_launches_per_step(const gks_handle* h) {
@@ -1167,8 +1206,7 @@ gks_status gks_part_bound(gks_handle* h, double* bound) {
   gks_status st = read_ctrl(h);
   if (st != GKS_OK) return st;
   memcpy(bound, &h->hctrl->bound, sizeof(double));
-  if (h->hctrl->status != GKS_OK) return fail(h, (gks_status)h->hctrl->status, "the slab's state is not physical");
-  return GKS_OK;
+  return step_status(h, "the slab's state is not physical");
 }
 
 gks_status gks_part_recon(gks_handle* h, double dt) {
@@ -1189,8 +1227,7 @@ gks_status gks_part_finish(gks_handle* h) {
                       : launch_step_kernels<float, float>(h, 0, 0, 0, true, true, 0, nullptr, false, true);
   if (st != GKS_OK) return st;
   CK(cudaStreamSynchronize(h->stream));
-  if (h->hctrl->status != GKS_OK) return fail(h, (gks_status)h->hctrl->status, "step produced a non-physical state; state kept");
-  return GKS_OK;
+  return step_status(h, "step produced a non-physical state; state kept");
 }
 
 namespace {
@@ -1359,7 +1396,7 @@ extern "C" gks_status gks_step_noalloc(int nx, int ny, double Lx, double Ly, dou
   if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
   const UpdateArgs<double, double> ua{C0, C1, Fx, Fy, const_cast<double*>(dWx), dWx_out, const_cast<double*>(dWy), dWy_out, bad};
   e = launch_update<double, double>(true, s, g, sms, ua, ctrl);
-  if (e == cudaSuccess) e = launch_finish<double, double>(s, g, sms, ua, ctrl, nullptr);
+  if (e == cudaSuccess) e = launch_finish<double, double>(s, g, sms, ua, ctrl, nullptr, kWaitSeconds, -1);
   if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
   k_store_cells<double><<<blocks_of((size_t)nx * ny), 256, 0, s>>>(g, dU_out, C0, C1, ctrl);
   e = cudaGetLastError();
@@ -1369,7 +1406,9 @@ extern "C" gks_status gks_step_noalloc(int nx, int ny, double Lx, double Ly, dou
   if (e != cudaSuccess) { g_create_err = std::string("gks_step_noalloc: ") + cudaGetErrorString(e); return GKS_ECUDA; }
   if (dt_taken) *dt_taken = hc.skip ? 0.0 : hc.dt;
   if (hc.status != GKS_OK) {
-    g_create_err = "gks_step_noalloc: the step produced a non-physical state; outputs are not valid";
+    g_create_err = hc.status == GKS_ETIMEOUT
+                       ? "gks_step_noalloc: a device wait of the positivity fallback ran out; outputs are not valid"
+                       : "gks_step_noalloc: the step produced a non-physical state; outputs are not valid";
     return (gks_status)hc.status;
   }
   if (hc.skip) { g_create_err = "gks_step_noalloc: dt = 0, no step taken; outputs are not valid"; return GKS_EINVAL; }

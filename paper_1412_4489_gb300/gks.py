@@ -69,6 +69,8 @@ def load(path: str | None = None):
     L.gks_set_state_device.argtypes = [H, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, D]
     L.gks_step.argtypes = [H, D, D, _dp]
     L.gks_advance.argtypes = [H, ctypes.c_int, D, D]
+    L.gks_set_wait_limit.argtypes = [H, D, ctypes.c_int]
+    L.gks_set_wait_limit.restype = ctypes.c_int
     L.gks_sync.argtypes = [H, _dp, ctypes.POINTER(ctypes.c_longlong)]
     L.gks_get_state.argtypes = [H, _dp, _dp, _dp, _dp]
     L.gks_get_state_device.argtypes = [H, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, _dp]
@@ -232,6 +234,10 @@ def gks_step(h, CFL, dt_max=float("inf")):
 
 def gks_advance(h, nsteps, CFL, t_end=float("inf")):
     _check(h, load().gks_advance(h, int(nsteps), float(CFL), float(t_end)))
+
+
+def gks_set_wait_limit(h, seconds, test_skip_block=-1):
+    _check(h, load().gks_set_wait_limit(h, float(seconds), int(test_skip_block)))
 
 
 def gks_sync(h):
