@@ -145,8 +145,8 @@ gks_status gks_create(int nx, int ny, double Lx, double Ly, double gamma, double
  * bound.  Synchronous.  Clears a pending GKS_ENONPHYSICAL.
  * Page-locked arrays mapped into the device's address space (cudaHostAlloc,
  * cudaHostRegister with the mapped flag, or any page-locked memory on a system
- * with unified addressing) are read in place by the kernels over the host link;
- * other host memory goes through a device staging buffer.  Either way each array
+ * with unified addressing) that start on a multiple of 8 bytes are read in place by the
+ * kernels over the host link; other host memory goes through a device staging buffer.  Either way each array
  * must hold the full size given above. */
 gks_status gks_set_state(gks_handle* h, const double* U, const double* Wx, const double* Wy,
                          double t);
@@ -293,12 +293,12 @@ gks_status gks_batch_create(int n, const gks_grid_desc* grids, const gks_options
                             void* cuda_stream, gks_batch** out);
 
 /* Copies grid g's state from host memory (all three arrays required); t is
- * its time.  Synchronous. */
+ * its time.  Page-locked arrays as in gks_set_state.  Synchronous. */
 gks_status gks_batch_set_state(gks_batch* b, int g, const double* U, const double* Wx,
                                const double* Wy, double t);
 
-/* Copies grid g's state to host memory (any pointer may be NULL).  Synchronous;
- * returns the grid's status. */
+/* Copies grid g's state to host memory (any pointer may be NULL; page-locked arrays
+ * are written in place, as by gks_get_state).  Synchronous; returns the grid's status. */
 gks_status gks_batch_get_state(gks_batch* b, int g, double* U, double* Wx, double* Wy, double* t,
                                long long* steps);
 

@@ -120,9 +120,10 @@ inline unsigned blocks_of(size_t n) { return (unsigned)((n + 255) / 256); }
 
 // The device address of a page-locked host array mapped into the device's address
 // space (cudaHostAlloc, cudaHostRegister): kernels then read or write it in place over
-// the host link.  nullptr for any other pointer (pageable host memory goes through
-// the staging buffer).
+// the host link.  nullptr for any other pointer, which goes through the staging buffer: pageable memory, and arrays
+// that do not start on a multiple of 8 bytes (a copy takes any address, a kernel's loads do not).
 inline const double* mapped_host(const void* p) {
+  if ((size_t)p % alignof(double)) return nullptr;
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();  // an unknown pointer: clear the error it left
