@@ -1007,7 +1007,7 @@ __device__ __forceinline__ R inv_bound(const Geo& g, const R w[4], bool& ok) {
 }
 
 // FP32 proof that an FP64 state is physical and its inverse CFL bound below `below`: rho > 0, the pressure
-// above the rounding of its terms, and the bound with a margin of 1e-4.  false where FP32 cannot tell
+// above the rounding of its terms, and the bound with a margin of 1e-3.  false where FP32 cannot tell
 // (near-vacuum states, values outside FP32's range, NaN).
 __device__ __forceinline__ bool surely_below(const Geo& g, const double w[4], float below) {
   const float r = (float)w[0], m = (float)w[1], n = (float)w[2], e = (float)w[3];
