@@ -9,7 +9,9 @@
 // fallback), separated by a device-wide barrier.  The barrier is a
 // counter with a generation word; every wait is bounded in time (globaltimer)
 // and gives up with GKS_ETIMEOUT instead of hanging.  The per-element
-// arithmetic is that of the single-grid kernels (gks_grid.cuh).
+// arithmetic is that of the single-grid kernels (gks_grid.cuh), but for FP32 faces, which
+// keep a routine of their own (gks_face_monomials.cuh): an FP32 batch agrees with FP32 single
+// grids to FP32 rounding.
 //
 // gks_batch_autotune times the tile shape of the face phase and the number of
 // resident blocks per SM on the batch itself and keeps the fastest.

@@ -1,7 +1,8 @@
 // Grid-level device work of one time step, per element: the ghost ring, the
 // reconstruction of one cell, the evolution at one face and the update of one
 // cell.  The single-grid kernels (gks.cu) and the persistent batched kernel
-// (gks_batch.cu) both call these, so both compute the same arithmetic.
+// (gks_batch.cu) both call these and compute the same arithmetic, but for the faces of FP32
+// batches (flux_face's MONO).
 #pragma once
 #include <cuda_runtime.h>
 #include <math.h>
