@@ -311,9 +311,9 @@ def run_ours(args):
     flux_kernels = {k: v for k, v in prof.items() if k.startswith("flux")}
     dom = max(flux_kernels, key=flux_kernels.get)
     L, R, avg = face_inputs(p)
-    ops = gks.gks_face_op_count(L, R, avg, p.Lx / p.nx, p.Ly / p.ny, 1e-3, p.gamma, 0.0, 1.0, 0.0, 1.0,
-                                gks.GKS_FP32_BULK)
-    flops_face = ops["add"] + ops["mul"] + ops["div"]
+    ops, ops64 = (gks.gks_face_op_count(L, R, avg, p.Lx / p.nx, p.Ly / p.ny, 1e-3, p.gamma, 0.0, 1.0, 0.0, 1.0, prec)
+                  for prec in (gks.GKS_FP32_BULK, gks.GKS_FP64))
+    flops_face, flops64 = (o["add"] + o["mul"] + o["div"] for o in (ops, ops64))
     nfaces = faces_x if dom == "flux_x" else p.nx * (p.ny + 1)
     achieved = flops_face * nfaces / (prof[dom] * 1e-3) / 1e12
     peak32 = SM_COUNT * FP32_LANES_PER_SM * 2 * SM_MAX_MHZ * 1e6 / 1e12
@@ -326,7 +326,6 @@ def run_ours(args):
     instr_face, _ = profile_figure("fp32", "instructions_per_face")
     issue_frac = None if instr_face is None else round(
         instr_face * nfaces / 32 / (prof[dom] * 1e-3) / (SM_COUNT * ISSUE_PER_SM_CLK * SM_MAX_MHZ * 1e6), 4)
-    flops64 = flops_face  # the same arithmetic in FP64
     achieved64 = flops64 * nfaces / (prof64[dom] * 1e-3) / 1e12
 
     out = None
@@ -356,6 +355,7 @@ def run_ours(args):
             "roofline_fp64": {"bound": "alu", "kernel": f"k_flux<{dom[-1]}> fp64", "achieved": round(achieved64, 4),
                               "peak": round(measured64, 3), "unit": "TFLOP/s", "frac": round(achieved64 / measured64, 4),
                               "peak_source": "measured FP64 FMA throughput (gks_measure_alu_peak)",
+                              "flops_per_face": flops64,
                               "kernel_ms": round(prof64[dom], 5)},
             "batched": batched,
             "validation": validation,

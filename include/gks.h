@@ -357,9 +357,10 @@ const char* gks_batch_last_error(const gks_batch* b);
  * face-frame inputs: L, R = [6][4] value and (dn, dt, dnn, dnt, dtt)
  * derivatives of the two sides, avg = [2][3][4] the six cell averages of
  * Section 3.3, cell sizes dn (normal) and dtan (along the face), time step dt.
- * precision selects the branch thresholds of GKS_FP64 or GKS_FP32_BULK.
+ * precision selects the arithmetic of GKS_FP64 (whose erfc and exp of the half spaces
+ * are polynomials, counted as such) or that of FP32 single grids (GKS_FP32_BULK).
  * counts[9] receives: additions/subtractions, multiplications, divisions,
- * comparisons, sqrt, rsqrt, exp, expm1, erfc.  Host only; needs no GPU. */
+ * comparisons, sqrt, rsqrt, exp, expm1 (none any more), erfc.  Host only; needs no GPU. */
 gks_status gks_face_op_count(const double* L, const double* R, const double* avg, double dn,
                              double dtan, double dt, double gamma, double mu, double Pr,
                              double tau_eps, double tau_C, int precision, long long* counts);

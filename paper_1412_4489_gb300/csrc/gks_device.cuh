@@ -27,18 +27,21 @@ template <class R> struct Prec;
 // terms reach it, FP32: 18);
 // exp_zero: exp(-x) is exactly 0 from here on, and not evaluated (FP32: always evaluated, a
 // branch costs more than its two instructions);
+// fp64: arithmetic chosen for the FP64 pipe (quotients from one reciprocal, half_normal's table);
 // tie: relative width within which two cross-derivative candidates count as equal.
 // FP64: far above its rounding noise, far below any real difference.  FP32: ~16
 // ulps, just above the rounding noise of the candidates; a wider band makes FP32
 // keep the first stencil where FP64 picks a smaller one of opposite sign, which
 // measured worse against the FP64 results on discontinuous data.
 template <> struct Prec<double> {
+  static constexpr bool fp64 = true;
   static constexpr double series_below = 0.5;
   static constexpr int series_terms = 18;
   static constexpr double exp_zero = 746.0;
   static constexpr double tie = 1e-8;
 };
 template <> struct Prec<float> {
+  static constexpr bool fp64 = false;
   static constexpr float series_below = 2.0f;
   static constexpr int series_terms = 18;
   static constexpr float exp_zero = INFINITY;
@@ -84,17 +87,19 @@ GKS_FN void half_start(R U, R l2, int kind, R& h, R& g) {
   const R lam = R(0.5) * l2;
   const R rs = d_rsqrt(lam);
   const R s = lam * rs;  // sqrt(lam)
-  h = R(0.5) * d_erfc(-R(kind) * s * U);
-  // boundary term of the integration by parts at u = 0
-  const R b = d_exp(-lam * U * U) * R(0.28209479177387814) * rs;  // 1/(2 sqrt(pi lam))
-  g = U * h + R(kind) * b;
-}
-__device__ __forceinline__ void half_start(double U, double l2, int kind, double& h, double& g) {
-  const double lam = 0.5 * l2, rs = rsqrt(lam), a = kind * (lam * rs) * U;
-  double t, e;
-  half_normal(fabs(a), t, e);
-  h = a > 0.0 ? 1.0 - t : t;
-  g = U * h + kind * (e * (0.28209479177387814 * rs));
+  // b: boundary term of the integration by parts at u = 0, 1/(2 sqrt(pi lam)) exp(-lam U^2)
+  if constexpr (Prec<R>::fp64) {
+    const R a = R(kind) * s * U;
+    R t, e;
+    half_normal(fabs(a), t, e);
+    h = a > R(0) ? R(1) - t : t;
+    const R b = e * (R(0.28209479177387814) * rs);
+    g = U * h + R(kind) * b;
+  } else {
+    h = R(0.5) * d_erfc(-R(kind) * s * U);
+    const R b = d_exp(-lam * U * U) * R(0.28209479177387814) * rs;
+    g = U * h + R(kind) * b;
+  }
 }
 
 // moments over u > 0 (kind +1) or u < 0 (kind -1); var = 1/(2 lam) = p/rho, formed once per
@@ -333,7 +338,7 @@ GKS_FN void prim(const R w[4], R gm1, R& rho, R& ir, R& U, R& V, R& p) {
 template <class R>
 GKS_FN void prim_lam(const R w[4], R gm1, R& rho, R& U, R& V, R& p, R& l2, R& var) {
   R ir;
-  if constexpr (sizeof(R) == 8) {
+  if constexpr (Prec<R>::fp64) {
     rho = w[0];
     const R rp = gm1 * (rho * w[3] - R(0.5) * (w[1] * w[1] + w[2] * w[2]));  // rho p
     const R q = rho * rp;
@@ -645,7 +650,7 @@ template <class R>
 GKS_FN void kinetic_coefs(const FaceConst<R>& C, const FaceState<R>& S, const SideData<R>& sd, bool ns, KineticCoefs<R>& k) {
   const R U = sd.U, V = sd.V, s = sd.s;
   // FP32: formed again (two instructions) rather than kept in a register across the equilibrium part
-  const R l2 = sizeof(R) == 4 ? d_rcp(s) : sd.l2;
+  const R l2 = Prec<R>::fp64 ? sd.l2 : d_rcp(s);
   const R hq = R(0.5) * (U * U + V * V), hs = R(0.5) * (U * U + s), c5 = C.i2N * l2;
   R e1[4], e2[4], exx[4], exy[4], eyy[4];
   central(U, V, hq, S.w[1], e1);
@@ -676,7 +681,7 @@ template <class R>
 GKS_FN void kinetic_part(const FaceConst<R>& C, const KineticCoefs<R>& kf, const SideData<R>& sd, bool ns, bool kin_point,
                          const TimeW<R>& w, R tn, R dt, R Fl[4], R P0[4], R P1[4], R Mn[4]) {
   const R rho = sd.rho, U = sd.U, V = sd.V, s = sd.s;
-  const R l2 = sizeof(R) == 4 ? d_rcp(s) : sd.l2;
+  const R l2 = Prec<R>::fp64 ? sd.l2 : d_rcp(s);
   const R *a1 = kf.a1, *a2 = kf.a2, *xx = kf.xx, *xy = kf.xy, *yy = kf.yy, *A = kf.A, *tx = kf.tx, *ty = kf.ty;
   R m[8];
   m[0] = sd.h;

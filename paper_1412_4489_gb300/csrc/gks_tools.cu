@@ -42,27 +42,36 @@ template <int P> bool operator<(const Num<P>& a, double b) { ++C.cmp; return a.v
 template <int P> bool operator>(const Num<P>& a, double b) { ++C.cmp; return a.v > b; }
 template <int P> Num<P> fabs(const Num<P>& a) { return Num<P>(::fabs(a.v)); }
 template <int P> Num<P> d_exp(const Num<P>& a) { ++C.exp; return Num<P>(::exp(a.v)); }
-template <int P> Num<P> d_expm1(const Num<P>& a) { ++C.expm1; return Num<P>(::expm1(a.v)); }
 template <int P> Num<P> d_erfc(const Num<P>& a) { ++C.erfc; return Num<P>(::erfc(a.v)); }
 template <int P> Num<P> d_sqrt(const Num<P>& a) { ++C.sqrt; return Num<P>(::sqrt(a.v)); }
 template <int P> Num<P> d_rsqrt(const Num<P>& a) { ++C.rsqrt; return Num<P>(1.0 / ::sqrt(a.v)); }
 template <int P> Num<P> d_rcp(const Num<P>& a) { ++C.div; return Num<P>(1.0 / a.v); }
 template <int P> bool mid_range(const Num<P>&) { return true; }  // a test of exponent bits: no arithmetic
 template <int P> Num<P> d_div(const Num<P>& a, const Num<P>& b) { ++C.div; return Num<P>(a.v / b.v); }
+// the table's polynomials (gks_half_normal.cuh): the node and its distance, value and derivative by Horner's rule
+// from degree 10, and the derivative's factor
+template <int P> void half_normal(const Num<P>& z, Num<P>& t, Num<P>& e) {
+  C.add += 3 + 10 + 9;
+  C.mul += 10 + 9 + 1;
+  t = Num<P>(0.5 * ::erfc(z.v));
+  e = Num<P>(::exp(-z.v * z.v));
+}
 
 }  // namespace opc
 
 #include "gks_device.cuh"
 
 namespace gks {
-// the counting types follow the branch thresholds of the precision they stand for
+// the counting types follow the branch thresholds and the arithmetic of the precision they stand for
 template <> struct Prec<opc::Num<0>> {
+  static constexpr bool fp64 = Prec<double>::fp64;
   static constexpr double series_below = Prec<double>::series_below;
   static constexpr int series_terms = Prec<double>::series_terms;
   static constexpr double exp_zero = Prec<double>::exp_zero;
   static constexpr double tie = Prec<double>::tie;
 };
 template <> struct Prec<opc::Num<1>> {
+  static constexpr bool fp64 = Prec<float>::fp64;
   static constexpr double series_below = Prec<float>::series_below;
   static constexpr int series_terms = Prec<float>::series_terms;
   static constexpr double exp_zero = Prec<float>::exp_zero;
