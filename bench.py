@@ -342,7 +342,7 @@ def run_ours(args):
             "error_fp32_bulk_vs_fp64": {"l1_rho_rel": l1, "linf_rho_rel": linf, "steps": 100,
                                         "reference": "GPU FP64 path (oracle-pinned in tests)",
                                         "other_workloads": errors},
-            "roofline": {"bound": "alu", "kernel": f"k_flux<{dom[-1]}> fp32", "achieved": round(achieved, 3),
+            "roofline": {"bound": "alu", "kernel": f"k_flux_euler ({dom[-1]}-faces) fp32", "achieved": round(achieved, 3),
                          "peak": round(peak32, 2), "unit": "TFLOP/s", "frac": round(achieved / peak32, 4),
                          "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 flop x 2070 MHz",
                          "peak_measured_fma": round(measured32, 2), "frac_of_measured_fma": round(achieved / measured32, 4),
@@ -352,7 +352,7 @@ def run_ours(args):
                          "kernel_ms": round(prof[dom], 5), "traffic": traffic,
                          "issue_slots": {"instructions_per_face": instr_face, "frac": issue_frac,
                                          "peak": "152 SMs x 4 warp instructions per clock x 2070 MHz"}},
-            "roofline_fp64": {"bound": "alu", "kernel": f"k_flux<{dom[-1]}> fp64", "achieved": round(achieved64, 4),
+            "roofline_fp64": {"bound": "alu", "kernel": f"k_faces ({dom[-1]}-faces) fp64", "achieved": round(achieved64, 4),
                               "peak": round(measured64, 3), "unit": "TFLOP/s", "frac": round(achieved64 / measured64, 4),
                               "peak_source": "measured FP64 FMA throughput (gks_measure_alu_peak)",
                               "flops_per_face": flops64,

@@ -587,7 +587,7 @@ cudaError_t launch_update(bool pdl, cudaStream_t s, const Geo& g, int sms, const
 
 template <class R, class TW>
 cudaError_t launch_finish(cudaStream_t s, const Geo& g, int sms, const UpdateArgs<R, TW>& a, Ctrl* c, Ctrl* mirror,
-                          double wait_s, int wait_skip) {
+                          double wait_s, int wait_skip, bool pdl = true) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = update_grid(g, 2, sms, 1, kUpdateRows);
   const dim3 tiles = grid2(g.nx, g.ny, dim3(32, kUpdateRows));
@@ -602,7 +602,7 @@ cudaError_t launch_finish(cudaStream_t s, const Geo& g, int sms, const UpdateArg
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
+  cfg.numAttrs = pdl ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, k_finish<R, TW>, g, a, c, mirror, w);
 }
 
@@ -729,7 +729,7 @@ gks_status launch_step_kernels(gks_handle* h, double cfl, double dt_max, double 
     // after the join (two predecessors): an ordinary launch
     keep(launch_update<R, TW>(pdl && !fork, s, g, h->sms, a, h->ctrl));
     mark(4);
-    keep(launch_finish<R, TW>(s, g, h->sms, a, h->ctrl, mirror ? h->hctrl : nullptr, h->wait_s, h->wait_skip));
+    keep(launch_finish<R, TW>(s, g, h->sms, a, h->ctrl, mirror ? h->hctrl : nullptr, h->wait_s, h->wait_skip, pdl));
   } else {
     mark(4);
   }

@@ -286,12 +286,14 @@ def gks_launches_per_step(h) -> int:
     return load().gks_launches_per_step(h)
 
 
-KERNEL_NAMES = ["recon", "flux_x", "flux_y", "update", "update2", "update3", "end"]
+# the kernels of a profiled step, in launch order; the library writes two more entries, which hold no kernel
+KERNEL_NAMES = ["recon", "flux_x", "flux_y", "update", "finish"]
+PROFILE_ENTRIES = 7
 
 
 def gks_profile_step(h, CFL):
     """One step with per-kernel CUDA-event timing; returns {kernel name: ms}."""
-    ms = (ctypes.c_float * len(KERNEL_NAMES))()
+    ms = (ctypes.c_float * PROFILE_ENTRIES)()
     _check(h, load().gks_profile_step(h, float(CFL), ms))
     return dict(zip(KERNEL_NAMES, list(ms)))
 
