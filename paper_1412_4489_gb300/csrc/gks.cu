@@ -15,7 +15,8 @@
 //              bound (warp-shuffle / block / atomic min) and the physical check
 //   k_finish   the update's second and third pass, only for the positivity fallback; advances t and
 //              the step counter
-// The ghost ring of a newly set state is filled by k_ghost.
+// A newly set state's ghost ring is filled as its cells are loaded (k_load_cells, gks_state.cuh); k_ghost refreshes it for
+// the unit-level entry points.
 // Cell averages and face values are double-buffered; the buffer in use is the
 // parity of the device step counter, so a failed step leaves the last good
 // state in place.
@@ -284,9 +285,9 @@ constexpr unsigned kSplitWarps = 3;
 // Update pass 1, 2 or 3 (see update_cell): pass 1 marks the cells it leaves
 // non-physical; pass 2 runs only if pass 1 marked cells, pass 3 only if pass 2
 // still left one; a cell non-physical after pass 3 fails the step.  Each pass
-// keeps its own running minimum of the CFL bound.  Blocks walk the grid's
-// 32 x 8 tiles with a stride of the launch grid: pass 1 is launched with one block
-// per tile, passes 2 and 3 (usually no work) with a few blocks per SM.
+// keeps its own running minimum of the CFL bound.  Blocks walk the grid's tiles
+// (32 cells by the block's height) with a stride of the launch grid (update_grid): pass 1
+// is a kernel of its own, k_update; passes 2 and 3 (usually no work) run in k_finish.
 // Resident blocks per SM the update is compiled for: the rarely taken fallback path
 // must not raise the register count of the common one (FP32: 64 registers).
 template <class R> struct UpdateBlocks;
@@ -684,9 +685,6 @@ gks_status launch_step_kernels(gks_handle* h, double cfl, double dt_max, double 
     mark(2);
     faces(ev ? 2 : 3);
   } else {
-    // the x- and y-face evolutions are independent: without per-kernel timing the y-faces run
-    // on a side stream (fork after the reconstruction, join before the update), so that each
-    // fills the other's tail wave
     if (g.mu > 0.0) {
       // the x- and y-face evolutions are independent: without per-kernel timing the y-faces run
       // on a side stream (fork after the reconstruction, join before the update), so that each

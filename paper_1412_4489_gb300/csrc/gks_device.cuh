@@ -52,8 +52,6 @@ __device__ __forceinline__ double d_exp(double x) { return exp(x); }
 __device__ __forceinline__ float d_exp(float x) { return __expf(x); }
 __device__ __forceinline__ double d_erfc(double x) { return erfc(x); }
 __device__ __forceinline__ float d_erfc(float x) { return erfcf(x); }
-__device__ __forceinline__ double d_sqrt(double x) { return sqrt(x); }
-__device__ __forceinline__ float d_sqrt(float x) { return sqrtf(x); }
 __device__ __forceinline__ double d_rsqrt(double x) { return rsqrt(x); }
 __device__ __forceinline__ float d_rsqrt(float x) { return rsqrtf(x); }
 // quotient of runtime values: IEEE in FP64; in FP32 the fast division (within
@@ -780,9 +778,9 @@ GKS_FN void finish_face(const FaceConst<R>& C, R u0, R v0, R Fl[4], const R P0[4
 // (one warp instruction per 19 cycles and SM), so fewer operations is what makes it faster.  Each Maxwellian
 // is evaluated in its own frame, where g0's moments are closed forms in the central derivatives and a half-space's
 // reduce to one-dimensional sums over u.  Against expanding the distribution into the monomials
-// u^a v^b xi^2c (gks_face_monomials.cuh): 1,237 instead of 2,041 counted flops at a smooth
-// Euler face (exp(-dt/tau) = 0), 1,739 instead of 2,779 at another, 2,198 instead of 3,907
-// Navier-Stokes with the Prandtl correction.
+// u^a v^b xi^2c (gks_face_monomials.cuh), in FP32: 1,238 instead of 2,041 counted flops at a smooth
+// Euler face (exp(-dt/tau) = 0), 1,738 instead of 2,779 at another, 2,205 instead of 3,907
+// Navier-Stokes with the Prandtl correction (FP64, erfc and exp as polynomials: 1,325, 1,825, 2,292).
 // x-faces at 512^2 FP32 26.2 -> 20.7 us (Euler), at 1024^2 108 -> 81 us (Navier-Stokes), at
 // 4096^2 1,177 -> 881 us; FP64 at 512^2 764 -> 534 us.  With the table for erfc and exp, the reciprocals and the
 // launch shapes of today 19.7, 74 and 730 us, FP64 463 us.

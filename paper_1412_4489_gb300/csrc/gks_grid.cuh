@@ -230,7 +230,7 @@ template <> __device__ __forceinline__ float step_dt<float>(const Ctrl* c) { ret
 
 // ---------------------------------------------------------------------------
 // Full-precision cell averages, the state the conservative update accumulates
-// into (get / set in FP64; put stores a compute-type value).  One allocation of 4 * plane doubles per buffer either way:
+// into (get in FP64; put stores a compute-type value).  One allocation of 4 * plane doubles per buffer either way:
 //  * FP64 mode: four FP64 planes;
 //  * FP32-bulk mode: each average is an unevaluated sum hi + lo of two FP32
 //    numbers (a double-float pair), the hi vectors in the first half and the lo vectors
@@ -242,7 +242,6 @@ template <class R> struct Cells;
 template <> struct Cells<double> {
   double* p;
   __device__ __forceinline__ double get(const Geo& g, int v, int i, int j) const { return p[Lay<double>::u(g, v, i, j)]; }
-  __device__ __forceinline__ void set(const Geo& g, int v, int i, int j, double w) const { p[Lay<double>::u(g, v, i, j)] = w; }
   __device__ __forceinline__ void put(const Geo& g, int v, int i, int j, double w) const { p[Lay<double>::u(g, v, i, j)] = w; }
   __host__ __device__ __forceinline__ const double* view() const { return p; }
 };
@@ -251,12 +250,6 @@ template <> struct Cells<float> {
   __device__ __forceinline__ double get(const Geo& g, int v, int i, int j) const {
     const size_t o = Lay<float>::u(g, v, i, j);
     return (double)p[o] + (double)p[o + 4 * g.plane];
-  }
-  __device__ __forceinline__ void set(const Geo& g, int v, int i, int j, double w) const {
-    const size_t o = Lay<float>::u(g, v, i, j);
-    const float hi = (float)w;
-    p[o] = hi;
-    p[o + 4 * g.plane] = (float)(w - (double)hi);
   }
   // a value known only in FP32 (ghost images): lo = 0
   __device__ __forceinline__ void put(const Geo& g, int v, int i, int j, float w) const {
@@ -418,7 +411,7 @@ __device__ __forceinline__ void ghosts_of_cell(const Geo& g, Cells<R> U, int i, 
   });
 }
 
-// p-th cell of the ghost ring (boundary images are taken in FP64)
+// p-th cell of the ghost ring
 template <class R>
 __device__ __forceinline__ void ghost_at(const Geo& g, Cells<R> U, int p) {
   const int row = g.nx + 2;

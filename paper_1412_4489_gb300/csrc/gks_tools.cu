@@ -43,7 +43,6 @@ template <int P> bool operator>(const Num<P>& a, double b) { ++C.cmp; return a.v
 template <int P> Num<P> fabs(const Num<P>& a) { return Num<P>(::fabs(a.v)); }
 template <int P> Num<P> d_exp(const Num<P>& a) { ++C.exp; return Num<P>(::exp(a.v)); }
 template <int P> Num<P> d_erfc(const Num<P>& a) { ++C.erfc; return Num<P>(::erfc(a.v)); }
-template <int P> Num<P> d_sqrt(const Num<P>& a) { ++C.sqrt; return Num<P>(::sqrt(a.v)); }
 template <int P> Num<P> d_rsqrt(const Num<P>& a) { ++C.rsqrt; return Num<P>(1.0 / ::sqrt(a.v)); }
 template <int P> Num<P> d_rcp(const Num<P>& a) { ++C.div; return Num<P>(1.0 / a.v); }
 template <int P> bool mid_range(const Num<P>&) { return true; }  // a test of exponent bits: no arithmetic
