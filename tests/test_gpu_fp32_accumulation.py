@@ -25,3 +25,21 @@ def test_rounding_errors_add_up_no_faster_than_in_the_batched_form(nx, ny, steps
     b.close()
     for want, single, batch in zip(*runs):
         assert np.linalg.norm(single - want) <= 1.1 * np.linalg.norm(batch - want)
+
+
+def test_long_runs_keep_below_the_batched_form():
+    """3,000 steps at the paper's CFL number: errors that repeat as the wave passes add up."""
+    p = wl.smooth_wave_2d(512, seed=2)
+    runs = []
+    for prec in (gks.GKS_FP64, gks.GKS_FP32_BULK):
+        s = gks.Solver(p, prec, tau_eps=0.0)
+        s.advance(3000, 0.2)
+        runs.append(s.state()[0])
+        s.close()
+    b = gks.Batch([p], gks.GKS_FP32_BULK, tau_eps=0.0)
+    b.step(3000, 0.2)
+    b.sync()
+    runs.append(b.state(0)[0])
+    b.close()
+    want, single, batch = runs
+    assert np.linalg.norm(single - want) <= 1.1 * np.linalg.norm(batch - want)
