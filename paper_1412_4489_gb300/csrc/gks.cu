@@ -157,8 +157,8 @@ __global__ void __launch_bounds__(128, 6) k_recon_lanes(Geo g, const double* U0,
 // face evolution
 // ---------------------------------------------------------------------------
 // resident 128-thread blocks per SM the FP32 face kernel is compiled for: Euler 5 (96 registers,
-// 20 warps per SM; 4 bytes of spill), Navier-Stokes 4 (128 registers; at 96 it spills 100-144 bytes).
-// x-faces at 2048^2, 4 / 5 blocks: Euler 222 / 207 us (195 with fewer spills); Navier-Stokes at 1024^2 79.5 / 80.4 us.  6 blocks (80
+// 20 warps per SM; 20 bytes of spill), Navier-Stokes 4 (128 registers; at 96 it spills 100-144 bytes).
+// x-faces at 2048^2, 4 / 5 blocks: Euler 222 / 207 us (194 as it is now); Navier-Stokes at 1024^2 79.5 / 80.4 us.  6 blocks (80
 // registers) are slower for both, 3 slower for Navier-Stokes.
 template <int NS> struct FluxBlocks { static constexpr int value = NS ? 4 : 5; };
 

@@ -783,7 +783,7 @@ GKS_FN void finish_face(const FaceConst<R>& C, R u0, R v0, R Fl[4], const R P0[4
 // Navier-Stokes with the Prandtl correction (FP64, erfc and exp as polynomials: 1,325, 1,825, 2,292).
 // x-faces at 512^2 FP32 26.2 -> 20.7 us (Euler), at 1024^2 108 -> 81 us (Navier-Stokes), at
 // 4096^2 1,177 -> 881 us; FP64 at 512^2 764 -> 534 us.  With the table for erfc and exp, the reciprocals and the
-// launch shapes of today 19.7, 74 and 730 us, FP64 463 us.
+// launch shapes of today 19.8, 75 and 740 us, FP64 465 us.
 // ---------------------------------------------------------------------------
 template <class R, int NSM = -1, class Src>
 GKS_FN void face_evolution(const FaceConst<R>& C, const Src& src, R dt, R F[4], R Wm[4], R Wp[4]) {
